@@ -188,6 +188,13 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
                  const unsigned long long *k4e, unsigned long long *work, const tg_tune &t,
                  cudaStream_t s);
 
+// Undivided whole-graph sums from node-level and edge-level totals (tg_sums.cu):
+// tau of every edge and, for k = 4, Theta, the D sums over higher ids (see
+// k_node_aggr), the 4-cycle and the 4-clique totals by type multiset.
+int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t *theta,
+                  const uint32_t *dlow, const unsigned long long *c4w, const unsigned long long *k4,
+                  unsigned long long *hist, cudaStream_t s);
+
 // Counts through Alg. 1's typed triangle counts (tg_reuse.cu).  full_order is
 // the grouped order of all M edges; order[0..count) the edges to count.  With
 // TG_KERNEL_CYCLES (or AUTO) the per-edge pass is tg_cyc_*, else k_count_reuse.

@@ -285,7 +285,8 @@ __global__ void __launch_bounds__(kLightWarps * 32) k_tau_light(
 
 // --------------------------------------------------- per-node aggregates ----
 // Theta_v[a][b] = sum over w in Gamma_v^a of tau_vw[b]; D_v[a][b] = sum of
-// d_w^b.  Nodes of degree up to dsmall: one thread per node, its 2 L^2 sums in
+// d_w^b, or (kLow, for the whole-graph totals of tg_sums.cu) the sum of
+// d_w^b - [b = phi_v] over the w of larger id only.  Nodes of degree up to dsmall: one thread per node, its 2 L^2 sums in
 // a private column of shared memory (k_node_aggr_small).  Larger nodes: their
 // typed ranges are cut into chunks of at most kAggrChunk entries, one warp per
 // chunk, whose sums are added to the (zeroed) rows (k_node_aggr).
@@ -308,10 +309,11 @@ __global__ void k_aggr_chunks(const int64_t *rowptr, const int32_t *toff, int64_
     }
 }
 
+template <bool kLow>
 __global__ void __launch_bounds__(kAggrSmallThreads)
     k_node_aggr_small(const int64_t *rowptr, const uint32_t *adj, const uint32_t *eid,
-                      const int32_t *toff, const uint32_t *tau, int64_t n, int32_t L,
-                      int dsmall, uint32_t *theta, uint32_t *dsum) {
+                      const int32_t *toff, const uint8_t *ntype, const uint32_t *tau, int64_t n,
+                      int32_t L, int dsmall, uint32_t *theta, uint32_t *dsum) {
     extern __shared__ uint32_t col[];  // [2 L^2][blockDim.x]
     const int tid = threadIdx.x, bd = blockDim.x;
     const int L2 = L * L;
@@ -319,16 +321,18 @@ __global__ void __launch_bounds__(kAggrSmallThreads)
         const int64_t rb = rowptr[v], re = rowptr[v + 1];
         if (re - rb > dsmall) continue;  // a warp of k_node_aggr takes it
         for (int q = 0; q < 2 * L2; ++q) col[q * bd + tid] = 0u;
+        const int tv = kLow ? ntype[v] : -1;
         for (int64_t x = rb; x < re; ++x) {
             const uint32_t wu = __ldg(adj + x);
             const int a = (int)(wu >> TG_TSHIFT);
+            const bool deg = !kLow || (int64_t)(wu & TG_IDMASK) > v;
             const uint32_t *tw = tau + (int64_t)__ldg(eid + x) * L;
             const int32_t *ow = toff + (int64_t)(wu & TG_IDMASK) * (L + 1);
             int prev = __ldg(ow);
             for (int b = 0; b < L; ++b) {
                 const int nx = __ldg(ow + b + 1);
                 col[(a * L + b) * bd + tid] += __ldg(tw + b);
-                col[(L2 + a * L + b) * bd + tid] += (uint32_t)(nx - prev);
+                if (deg) col[(L2 + a * L + b) * bd + tid] += (uint32_t)(nx - prev - (kLow && b == tv));
                 prev = nx;
             }
         }
@@ -339,8 +343,10 @@ __global__ void __launch_bounds__(kAggrSmallThreads)
     }
 }
 
+template <bool kLow>
 __global__ void k_node_aggr(const int64_t *rowptr, const uint32_t *adj, const uint32_t *eid,
-                            const int32_t *toff, const uint32_t *tau, int64_t n, int32_t L,
+                            const int32_t *toff, const uint8_t *ntype, const uint32_t *tau,
+                            int64_t n, int32_t L,
                             const uint32_t *nch, const uint32_t *cpos, uint32_t *theta,
                             uint32_t *dsum) {
     const int lane = threadIdx.x & 31;
@@ -369,6 +375,7 @@ __global__ void k_node_aggr(const int64_t *rowptr, const uint32_t *adj, const ui
             r -= ch;
         }
         const int c0 = s0 + (int)r * kAggrChunk, c1 = min(s1, c0 + kAggrChunk);
+        const int phi = kLow ? ntype[v] : -1;
         uint32_t at[TG_MAX_TYPES], ad[TG_MAX_TYPES];
 #pragma unroll
         for (int b = 0; b < TG_MAX_TYPES; ++b) {
@@ -385,7 +392,7 @@ __global__ void k_node_aggr(const int64_t *rowptr, const uint32_t *adj, const ui
                 if (b < L) {
                     at[b] += __ldg(tw + b);
                     const int nx = __ldg(ow + b + 1);
-                    ad[b] += (uint32_t)(nx - prev);
+                    if (!kLow || (int64_t)w > v) ad[b] += (uint32_t)(nx - prev - (kLow && b == phi));
                     prev = nx;
                 }
             }
@@ -962,6 +969,40 @@ int edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStream_t
 
 
 
+// Theta and D of every node (see k_node_aggr)
+template <bool kLow>
+int node_sums(const tg_graph *g, const uint32_t *tau, uint32_t *theta, uint32_t *dsum,
+              cudaStream_t s) {
+    const int L = g->L, L2 = L * L;
+    const int64_t n = g->n;
+    const int dsmall = L <= kAggrSmallMaxL ? kAggrSmall : -1;
+    // rows of the chunked nodes start at zero
+    TG_TRY_CUDA(cudaMemsetAsync(theta, 0, (size_t)n * L2 * 4, s));
+    TG_TRY_CUDA(cudaMemsetAsync(dsum, 0, (size_t)n * L2 * 4, s));
+    if (dsmall >= 0) {
+        const size_t asmem = (size_t)2 * L2 * kAggrSmallThreads * 4;
+        TG_TRY(tg_allow_max_smem((const void *)k_node_aggr_small<kLow>));
+        int per = 0;
+        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_node_aggr_small<kLow>,
+                                                                  kAggrSmallThreads, asmem));
+        const int64_t ag = std::min<int64_t>((int64_t)tg_num_sms() * (per > 0 ? per : 1),
+                                             (n + kAggrSmallThreads - 1) / kAggrSmallThreads);
+        k_node_aggr_small<kLow><<<(unsigned)std::max<int64_t>(ag, 1), kAggrSmallThreads, asmem, s>>>(
+            g->rowptr, g->adj, g->eid, g->toff, g->ntype, tau, n, L, dsmall, theta, dsum); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+    }
+    DevBuf<uint32_t> nch, cpos;
+    if (!nch.alloc(n, s) || !cpos.alloc(n, s)) return TG_ENOMEM;
+    k_aggr_chunks<<<grid_r(n), 256, 0, s>>>(g->rowptr, g->toff, n, L, dsmall, nch.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    TG_TRY(tg_scan_u32(nch.p, cpos.p, n, s));
+    int per = 0;
+    TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_node_aggr<kLow>, 256, 0));
+    k_node_aggr<kLow><<<(unsigned)((int64_t)tg_num_sms() * (per > 0 ? per : 1)), 256, 0, s>>>(
+        g->rowptr, g->adj, g->eid, g->toff, g->ntype, tau, n, L, nch.p, cpos.p, theta, dsum); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    return TG_OK;
+}
 
 template <int U>
 int launch_reuse_u(const ReuseParams &p, int threads, size_t smem, int grid_limit,
@@ -1040,39 +1081,17 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
         }
     }
     TG_TRY_CUDA(cudaEventRecord(g_last.ev[1], s));
+    const bool cycles = t.kernel == TG_KERNEL_CYCLES || t.kernel == TG_KERNEL_AUTO;
+    // the sums of the whole graph need no per-edge pass (tg_sums.cu)
+    const bool whole = cycles && hist && !rows && part.count <= 1 && order == full_order &&
+                       count == M && t.edge_pass != TG_EDGE_PASS_FUSED;
     if (k == 4) {
         if (!theta.alloc((size_t)n * L2, s) || !dsum.alloc((size_t)n * L2, s)) return TG_ENOMEM;
-        const int dsmall = L <= kAggrSmallMaxL ? kAggrSmall : -1;
-        // rows of the chunked nodes start at zero
-        TG_TRY_CUDA(cudaMemsetAsync(theta.p, 0, (size_t)n * L2 * 4, s));
-        TG_TRY_CUDA(cudaMemsetAsync(dsum.p, 0, (size_t)n * L2 * 4, s));
-        if (dsmall >= 0) {
-            const size_t asmem = (size_t)2 * L2 * kAggrSmallThreads * 4;
-            TG_TRY(tg_allow_max_smem((const void *)k_node_aggr_small));
-            int per = 0;
-            TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_node_aggr_small,
-                                                                      kAggrSmallThreads, asmem));
-            const int64_t ag = std::min<int64_t>((int64_t)tg_num_sms() * (per > 0 ? per : 1),
-                                                 (n + kAggrSmallThreads - 1) / kAggrSmallThreads);
-            k_node_aggr_small<<<(unsigned)std::max<int64_t>(ag, 1), kAggrSmallThreads, asmem, s>>>(
-                g->rowptr, g->adj, g->eid, g->toff, tau.p, n, L, dsmall, theta.p, dsum.p); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-        }
-        DevBuf<uint32_t> nch, cpos;
-        if (n > 0) {
-            if (!nch.alloc(n, s) || !cpos.alloc(n, s)) return TG_ENOMEM;
-            k_aggr_chunks<<<grid_r(n), 256, 0, s>>>(g->rowptr, g->toff, n, L, dsmall, nch.p); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-            TG_TRY(tg_scan_u32(nch.p, cpos.p, n, s));
-            int per = 0;
-            TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_node_aggr, 256, 0));
-            k_node_aggr<<<(unsigned)((int64_t)tg_num_sms() * (per > 0 ? per : 1)), 256, 0, s>>>(
-                g->rowptr, g->adj, g->eid, g->toff, tau.p, n, L, nch.p, cpos.p, theta.p, dsum.p); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-        }
+        TG_TRY(whole ? node_sums<true>(g, tau.p, theta.p, dsum.p, s)
+                     : node_sums<false>(g, tau.p, theta.p, dsum.p, s));
     }
     TG_TRY_CUDA(cudaEventRecord(g_last.ev[2], s));
-    if (t.kernel == TG_KERNEL_CYCLES || t.kernel == TG_KERNEL_AUTO) {
+    if (cycles) {
         // 4-cycles and 4-cliques per edge from whole-graph enumerations, then
         // the per-edge identities (tg_cycles.cu)
         DevBuf<unsigned long long> c4e, k4e, g4c, g4k;
@@ -1099,6 +1118,13 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
         TG_TRY_CUDA(cudaEventRecord(g_last.ev[3], s));
         if (k == 4) TG_TRY(tg_cyc_cliques(g, k4e.p, g4k.p, work, t, fast ? part : tg_part(), s));
         TG_TRY_CUDA(cudaEventRecord(g_last.ev[4], s));
+        if (whole) {
+            TG_TRY(tg_sum_totals(g, k, tau.p, theta.p, dsum.p, g4c.p, g4k.p, hist, s));
+            TG_TRY_CUDA(cudaEventRecord(g_last.ev[5], s));
+            g_last.edges = (uint64_t)count;
+            g_last.ready = true;
+            return TG_OK;
+        }
         tg_units un2;
         tg_units *ue = &un;
         if (order != full_order || count != M) {
