@@ -1390,6 +1390,22 @@ int tg_rows_device(const tg_graph *g, int k, int level, uint64_t *rows, cudaStre
                         tg_slots(g->L, k, level), nullptr, s);
 }
 
+int tg_rows_mapped(const tg_graph *g, int k, int level, uint64_t *const *rowmap, bool *done,
+                   cudaStream_t s) {
+    *done = false;
+    TG_TRY(check_counts(g, k));
+    const tg_tune t = tune_now();
+    if (t.kernel != TG_KERNEL_AUTO && t.kernel != TG_KERNEL_CYCLES) return TG_OK;
+    if (g->M > 0) {
+        tg_sched *sc = nullptr;
+        TG_TRY(get_sched(g, s, &sc));
+        TG_TRY(tg_reuse_count(g, k, level, sc->order, sc->order, g->M, nullptr,
+                              tg_slots(g->L, k, level), nullptr, t, s, tg_part(), rowmap));
+    }
+    *done = true;
+    return TG_OK;
+}
+
 extern "C" int tg_work_model(const tg_graph *g, uint64_t *entries, void *stream) {
     if (!g || !entries) return TG_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;

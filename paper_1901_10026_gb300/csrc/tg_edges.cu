@@ -52,7 +52,8 @@ struct EdgeParams {
     unsigned long long *tsum;  // split mode: B, C and DT (3 L^2 uint64) per order position
     int64_t qbase;             // split mode: order position of tsum's first row
     unsigned long long *queue;
-    uint64_t *rows;
+    uint64_t *rows;            // per-edge mode: M x width, row e of edge e
+    uint64_t *const *rowmap;   // or the row of edge e at rowmap[e]; both NULL for sums
     int64_t width;
     unsigned long long *hist;
     int64_t hist_len;
@@ -198,9 +199,10 @@ __device__ void edge_finish(const EdgeParams &p, unsigned long long *shist, int6
                             long long *xt) {
     const int lane = threadIdx.x & 31;
     const int L = p.L, P = p.P, L2 = L * L;
+    uint64_t *const erow = p.rowmap ? p.rowmap[e] : p.rows ? p.rows + e * p.width : nullptr;
     // 2- and 3-node entries
-    if (p.rows) {
-        uint64_t *row = p.rows + e * p.width;
+    if (erow) {
+        uint64_t *row = erow;
         for (int t = lane; t < L; t += 32) {
             const uint32_t tt = __ldg(tn + t);
             const int64_t si = (int64_t)(__ldg(toi + t + 1) - __ldg(toi + t)) - tt - (t == tj);
@@ -252,8 +254,8 @@ __device__ void edge_finish(const EdgeParams &p, unsigned long long *shist, int6
             uint64_t g[10];
             pair_orbits_tab(xt, L, t, u, (uint64_t)E.Si(t), (uint64_t)E.Si(u), (uint64_t)E.Sj(t),
                             (uint64_t)E.Sj(u), (uint64_t)E.Tn(t), (uint64_t)E.Tn(u), g);
-            if (p.rows) {
-                uint64_t *row = p.rows + e * p.width + 2 * L;
+            if (erow) {
+                uint64_t *row = erow + 2 * L;
                 if (p.level == TG_ORBIT) {
 #pragma unroll
                     for (int o = 0; o < 10; ++o) row[o * P + pr] = g[o];
@@ -697,7 +699,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
                  const uint32_t *theta,
                  const uint32_t *dsum, const unsigned long long *c4e,
                  const unsigned long long *k4e, unsigned long long *work, const tg_tune &t,
-                 cudaStream_t s) {
+                 cudaStream_t s, uint64_t *const *rowmap) {
     if (un.nunits == 0 || count <= 0) return TG_OK;
     const int L = g->L, L2 = L * L;
     if (g->max_degree >= ((int64_t)1 << 27)) return TG_EOVERFLOW;  // 32-lane uint32 sums
@@ -728,6 +730,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
     p.k = k;
     p.level = level;
     p.rows = rows;
+    p.rowmap = rowmap;
     p.width = width;
     p.hist = hist;
     p.hist_len = tg_global_len(L, k);
@@ -738,7 +741,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
     p.work = work;
     const size_t avail = (size_t)smem_optin_e() - 1024;
     const size_t hist_bytes = ((size_t)p.hist_len * 8 + 15) & ~(size_t)15;
-    const int hist_smem = (!rows && hist_bytes <= 48 * 1024) ? 1 : 0;
+    const int hist_smem = (hist && hist_bytes <= 48 * 1024) ? 1 : 0;
     // per warp: B, C, DT; the kernels that finish edges add the term table
     const size_t tbytes = ((size_t)3 * L2 * 8 + 15) & ~(size_t)15;
     const size_t xbytes = tbytes + (size_t)XT_N * L2 * 8;

@@ -186,7 +186,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
                  const uint32_t *theta,
                  const uint32_t *dsum, const unsigned long long *c4e,
                  const unsigned long long *k4e, unsigned long long *work, const tg_tune &t,
-                 cudaStream_t s);
+                 cudaStream_t s, uint64_t *const *rowmap = nullptr);
 
 // Undivided whole-graph sums from node-level and edge-level totals (tg_sums.cu):
 // tau of every edge and, for k = 4, Theta, the D sums over higher ids (see
@@ -204,8 +204,12 @@ int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t 
 int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_order,
                    const uint32_t *order, int64_t count, uint64_t *rows, int64_t width,
                    unsigned long long *hist, const tg_tune &t, cudaStream_t s,
-                   const tg_part &part = tg_part());
+                   const tg_part &part = tg_part(), uint64_t *const *rowmap = nullptr);
 
 // Per-edge rows of the whole graph into device memory `rows` (M x
 // tg_slots(L, k, level)), queued on s (tg_count.cu).
 int tg_rows_device(const tg_graph *g, int k, int level, uint64_t *rows, cudaStream_t s);
+// The same with the row of edge e written at rowmap[e] (a device array).  Only
+// the cycles kernel writes through a map: *done tells whether it ran.
+int tg_rows_mapped(const tg_graph *g, int k, int level, uint64_t *const *rowmap, bool *done,
+                   cudaStream_t s);

@@ -1028,7 +1028,7 @@ int launch_reuse_u(const ReuseParams &p, int threads, size_t smem, int grid_limi
 int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_order,
                    const uint32_t *order, int64_t count, uint64_t *rows, int64_t width,
                    unsigned long long *hist, const tg_tune &t, cudaStream_t s,
-                   const tg_part &part) {
+                   const tg_part &part, uint64_t *const *rowmap) {
     if (count <= 0 && part.count <= 1) return TG_OK;  // a share of a split count still enumerates
     const int L = g->L, L2 = L * L;
     const int64_t M = g->M, n = g->n;
@@ -1139,7 +1139,7 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
             TG_TRY_CUDA(cudaGetLastError());
         }
         TG_TRY(tg_cyc_edges(g, k, level, order, count, *ue, rows, width, hist, tau.p, tau_adj.p,
-                            theta.p, dsum.p, c4e.p, k4e.p, work, t, s));
+                            theta.p, dsum.p, c4e.p, k4e.p, work, t, s, rowmap));
         if (fast) TG_TRY(tg_cyc_correct(hist, L, g4c.p, g4k.p, s));
         TG_TRY_CUDA(cudaEventRecord(g_last.ev[5], s));
         g_last.edges = (uint64_t)count;
