@@ -21,9 +21,9 @@
 //     ending at each b by type (c_t(b)); pass 2 adds, for every wedge, the
 //     cycles it closes with the other middles to its two edges (per-edge
 //     mode); the far ends then add C(c_t, 2) and c_t c_t' (global mode) and
-//     clear the counters.  Global mode keeps the counters of light anchors in
-//     shared memory (k_c4_warp, k_c4_cta) and walks costly ones in warp units
-//     over L2-sized waves of counter slots (k_c4_walk, k_c4_pairs).
+//     clear the counters.  Light anchors keep their counters in shared memory
+//     (tg_c4_light.cu); global mode walks costly ones in warp units over binned
+//     waves and waves of counter slots.
 //   4-cliques (k_k4): each 4-clique x0 < v < w < x (by rank) is met once from
 //     its lowest node along "up" lists (neighbours of higher rank) and adds one
 //     to each of its six edges, keyed by the unordered types of the two nodes
@@ -36,6 +36,7 @@
 #include <new>
 #include <vector>
 
+#include "tg_cycles.cuh"
 #include "tg_device.cuh"
 
 using namespace tgd;
@@ -570,87 +571,14 @@ __global__ void k_c4_units(const int64_t *ustart, int64_t nq, const int64_t *tgt
     }
 }
 
-// Positions [f_lo, f_hi) of anchor a's walk, from member m on (its first
-// position `at`), by one warp: members are taken 32 at a time, their list
-// lengths scanned across the lanes, and each position mapped to its member by
-// a 5-step search over the lanes' running sums.  op(b, t_u) runs for every
-// entry b ranked below a of a member u.  With stride > 32 the warp takes every
-// (stride / 32)-th chunk of 32 members (no window: f_lo = 0, f_hi unbounded).
-// One chunk of 32 members (lane values len, bu, tu) of c4_warp_walk, with
-// running sums in IT (int when every list is short enough); returns the
-// chunk's length.
-template <class IT, class Op>
-__device__ __forceinline__ int64_t c4_chunk(const C4Params &p, uint32_t a, int64_t len64,
-                                            int64_t bu, int tu, int64_t at, int64_t f_lo,
-                                            int64_t f_hi, Op &op) {
-    const int lane = threadIdx.x & 31;
-    const IT len = (IT)len64;
-    IT incl = len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const IT y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const IT total = __shfl_sync(kFull, incl, 31);
-    const IT lo = (IT)(f_lo > at ? (f_lo - at < (int64_t)total ? f_lo - at : (int64_t)total) : 0);
-    const IT hi = (IT)(f_hi - at < (int64_t)total ? f_hi - at : (int64_t)total);
-    for (IT b0 = lo; b0 < hi; b0 += 32) {
-        const IT pos = b0 + lane;
-        int r = 0;  // the first member whose running sum exceeds pos
-#pragma unroll
-        for (int st = 16; st > 0; st >>= 1) {
-            const IT v = __shfl_sync(kFull, incl, r + st - 1);
-            if (v <= pos) r += st;
-        }
-        const int64_t bur = __shfl_sync(kFull, bu, r);
-        const IT str = __shfl_sync(kFull, incl - len, r);
-        const int tur = __shfl_sync(kFull, tu, r);
-        if (pos < hi) {
-            const uint32_t b = __ldg(p.adj + bur + (int64_t)(pos - str)) & TG_IDMASK;
-            if (b > a) op(b, tur);
-        }
-    }
-    return (int64_t)total;
-}
-
-// Positions [f_lo, f_hi) of anchor a's walk, from member m on (its first
-// position `at`), by one warp: members are taken 32 at a time, their list
-// lengths scanned across the lanes, and each position mapped to its member by
-// a 5-step search over the lanes' running sums.  op(b, t_u) runs for every
-// entry b ranked below a of a member u.  With stride > 32 the warp takes every
-// (stride / 32)-th chunk of 32 members (no window: f_lo = 0, f_hi unbounded).
-template <class Op>
-__device__ __forceinline__ void c4_warp_walk(const C4Params &p, uint32_t a, int64_t ba, int da,
-                                             int m, int64_t at, int64_t f_lo, int64_t f_hi,
-                                             int stride, Op op) {
-    const int lane = threadIdx.x & 31;
-    for (; m < da && at < f_hi; m += stride) {
-        const int x = m + lane;
-        int64_t len = 0, bu = 0;
-        int tu = 0;
-        if (x < da) {
-            const uint32_t wu = __ldg(p.adj + ba + x);
-            const uint32_t u = wu & TG_IDMASK;
-            if (u > a) {
-                bu = p.rowptr[u];
-                const int64_t du = p.rowptr[u + 1] - bu;
-                if (du > 1) {
-                    len = du;
-                    tu = (int)(wu >> TG_TSHIFT);
-                }
-            }
-        }
-        if (__all_sync(kFull, len < ((int64_t)1 << 26)))  // 32 lists sum below 2^31
-            at += c4_chunk<int>(p, a, len, bu, tu, at, f_lo, f_hi, op);
-        else
-            at += c4_chunk<int64_t>(p, a, len, bu, tu, at, f_lo, f_hi, op);
-    }
-}
-
-// One chunk of 32 members for k_c4_walk: as c4_chunk, with kWalkUnroll
-// batches of 32 positions in flight per step (their list loads, then their
-// counter adds, then the bitmap marks), so each lane keeps several returning
-// adds outstanding.
+// Positions [f_lo, f_hi) of one chunk of 32 members (lane values len, bu, tu;
+// the chunk's first position `at`) for k_c4_walk: the members' list lengths are
+// scanned across the lanes (running sums in IT, int when every list is short
+// enough), and each position is mapped to its member by a 5-step search over
+// the lanes' running sums.  kWalkUnroll batches of 32 positions are in flight
+// per step (their list loads, then their counter adds, then the bitmap marks),
+// so each lane keeps several returning adds outstanding.  Returns the chunk's
+// length.
 constexpr int kWalkUnroll = 4;
 
 template <class IT>
@@ -824,7 +752,7 @@ constexpr int kBinFill = 32;            // default: binned when a walk averages 
 constexpr size_t kBinTable = 64 * 1024;  // bytes of the dense far-end table
 
 // One chunk of 32 members (lane values len, bu, tu) of a binned walk unit; as
-// c4_chunk, with kBinUnroll batches of 32 positions per step.  Count pass:
+// c4_chunk_count, with kBinUnroll batches of 32 positions per step.  Count pass:
 // adds each batch's wedges to their buckets' sizes.  Fill pass: takes a run
 // of slots from each bucket's cursor and writes the entries.
 template <bool kFill, class IT>
@@ -1106,210 +1034,6 @@ __global__ void __launch_bounds__(kBinPairThreads) k_c4_bin_pairs(C4Bin p) {
     __syncthreads();
     for (int64_t q = tid; q < p.n4; q += blockDim.x)
         if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
-}
-
-__global__ void k_gather_u64(const unsigned long long *x, const uint32_t *idx, int64_t n,
-                             unsigned long long *out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = x[idx[i]];
-}
-
-// ------------------------------------------------- light anchors (global) --
-// Anchors whose walk cost (sum of d_u over their members) is at most half a
-// warp's table: one warp per anchor, the far ends in a per-warp shared-memory
-// hash set with L 16-bit middle counters per slot (a count never exceeds the
-// cost).  No global counters, no CTA barrier between anchors.
-constexpr int kC4WarpWarps = 8;
-constexpr int kC4WarpLgMax = 9;  // 512 slots per warp
-
-__device__ __forceinline__ uint32_t c4w_count(const uint32_t *cw, int k) {
-    const volatile uint32_t *v = cw;
-    return (v[k >> 1] >> ((k & 1) * 16)) & 0xffffu;
-}
-
-__global__ void __launch_bounds__(kC4WarpWarps * 32, 4) k_c4_warp(C4Params p, const uint32_t *alist,
-                                                              int64_t na,
-                                                              const unsigned long long *cost,
-                                                              int lg_max) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int L = p.L;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int emax = 1 << lg_max;
-    const int cwords = (emax * L + 1) >> 1;
-    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem);
-    uint32_t *keys = reinterpret_cast<uint32_t *>(h4 + p.n4) + (size_t)warp * (emax + cwords);
-    uint32_t *cw = keys + emax;
-    for (int64_t q = threadIdx.x; q < p.n4; q += blockDim.x) h4[q] = 0ull;
-    for (int q = lane; q < emax + cwords; q += 32) keys[q] = 0u;
-    __syncthreads();
-    unsigned long long wk = 0;
-    for (;;) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(p.queue, 32ull);
-        base = __shfl_sync(kFull, base, 0);
-        if (base >= (unsigned long long)na) break;
-        const int64_t stop = min((int64_t)base + 32, na);
-        for (int64_t i = (int64_t)base; i < stop; ++i) {
-            const uint32_t a = alist[i];
-            const int64_t ba = p.rowptr[a];
-            const int da = (int)(p.rowptr[a + 1] - ba);
-            const int ta = p.ntype[a];
-            const unsigned long long ca = cost[a];
-            int lg = 5;
-            while ((1ull << lg) < 2 * ca && lg < lg_max) ++lg;
-            c4_warp_walk(p, a, ba, da, 0, 0, 0, INT64_MAX, 32, [&](uint32_t b, int tu) {
-                const int h = hset_claim(keys, lg, b);
-                if (h >= 0) {
-                    const int k = h * L + tu;
-                    atomicAdd(cw + (k >> 1), 1u << ((k & 1) * 16));
-                    ++wk;
-                }
-            });
-            __syncwarp();
-            const int e = 1 << lg;
-            const volatile uint32_t *vk = keys;
-            for (int h = lane; h < e; h += 32) {
-                const uint32_t k = vk[h];
-                if (!k) continue;
-                uint32_t c[TG_MAX_TYPES];
-                for (int t = 0; t < L; ++t) c[t] = c4w_count(cw, h * L + t);
-                c4_add(h4, L, ta, p.ntype[k - 1u], c);
-            }
-            __syncwarp();
-            for (int q = lane; q < e; q += 32) keys[q] = 0u;
-            for (int q = lane; q < ((e * L + 1) >> 1); q += 32) cw[q] = 0u;
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int64_t q = threadIdx.x; q < p.n4; q += blockDim.x)
-        if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
-    if (p.work) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wk += __shfl_xor_sync(kFull, wk, o);
-        if (lane == 0 && wk) atomicAdd(p.work + 4, wk);
-    }
-}
-
-// Anchors of cost up to half a CTA table: one CTA per anchor, its warps taking
-// every eighth chunk of 32 members, the far ends in one shared-memory hash set
-// with 16-bit middle counters (the cost stays far below 2^16).
-constexpr int kC4CtaThreads = 256;
-constexpr int kC4CtaLgMax = 13;  // 8192 slots
-
-__global__ void __launch_bounds__(kC4CtaThreads) k_c4_cta(C4Params p, const uint32_t *alist,
-                                                          int64_t na,
-                                                          const unsigned long long *cost,
-                                                          int lg_max) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int L = p.L;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int stride = blockDim.x;  // 32 members per warp
-    const int emax = 1 << lg_max;
-    const int cwords = (emax * L + 1) >> 1;
-    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem);
-    unsigned long long *s_item = h4 + p.n4;
-    uint32_t *keys = reinterpret_cast<uint32_t *>(s_item + 1);
-    uint32_t *cw = keys + emax;
-    for (int64_t q = tid; q < p.n4; q += blockDim.x) h4[q] = 0ull;
-    for (int q = tid; q < emax + cwords; q += blockDim.x) keys[q] = 0u;
-    unsigned long long wk = 0;
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) *s_item = atomicAdd(p.queue, 1ull);
-        __syncthreads();
-        const unsigned long long item = *s_item;
-        if (item >= (unsigned long long)na) break;
-        const uint32_t a = alist[item];
-        const int64_t ba = p.rowptr[a];
-        const int da = (int)(p.rowptr[a + 1] - ba);
-        const int ta = p.ntype[a];
-        const unsigned long long ca = cost[a];
-        int lg = 5;
-        while ((1ull << lg) < 2 * ca && lg < lg_max) ++lg;
-        c4_warp_walk(p, a, ba, da, 32 * warp, 0, 0, INT64_MAX, stride, [&](uint32_t b, int tu) {
-            const int h = hset_claim(keys, lg, b);
-            if (h >= 0) {
-                const int k = h * L + tu;
-                atomicAdd(cw + (k >> 1), 1u << ((k & 1) * 16));
-                ++wk;
-            }
-        });
-        __syncthreads();
-        const int e = 1 << lg;
-        const volatile uint32_t *vk = keys;
-        for (int h = tid; h < e; h += blockDim.x) {
-            const uint32_t k = vk[h];
-            if (!k) continue;
-            uint32_t c[TG_MAX_TYPES];
-            for (int t = 0; t < L; ++t) c[t] = c4w_count(cw, h * L + t);
-            c4_add(h4, L, ta, p.ntype[k - 1u], c);
-        }
-        __syncthreads();
-        for (int q = tid; q < e; q += blockDim.x) keys[q] = 0u;
-        for (int q = tid; q < ((e * L + 1) >> 1); q += blockDim.x) cw[q] = 0u;
-    }
-    __syncthreads();
-    for (int64_t q = tid; q < p.n4; q += blockDim.x)
-        if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
-    if (p.work) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wk += __shfl_xor_sync(kFull, wk, o);
-        if (lane == 0 && wk) atomicAdd(p.work + 4, wk);
-    }
-}
-
-// Walk cost of each anchor (sum of d_u over its neighbours u ranked below it)
-// and the total.  One warp per node.
-__global__ void k_c4_cost(const int64_t *rowptr, const uint32_t *adj, int64_t n,
-                          unsigned long long *cost, unsigned long long *total) {
-    const int lane = threadIdx.x & 31;
-    const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long mine = 0;
-    for (int64_t a = wid; a < n; a += nw) {
-        const int64_t b = rowptr[a];
-        const int d = (int)(rowptr[a + 1] - b);
-        unsigned long long c = 0;
-        for (int x = lane; x < d; x += 32) {
-            const uint32_t u = __ldg(adj + b + x) & TG_IDMASK;
-            if ((int64_t)u > a) c += (unsigned long long)(rowptr[u + 1] - rowptr[u]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-        if (lane == 0) cost[a] = d >= 2 ? c : 0ull;
-        mine += c;
-    }
-    if (lane == 0 && mine) atomicAdd(total, mine);
-}
-
-// Anchor classes by walk cost c (flags[k n + a] = 1 for the class of a):
-// kClsSplit c > thr, else kClsWarp 0 < c <= lite, kClsCta lite < c <= mid,
-// kClsSlot mid < c (anchors of cost 0 close no cycle and take none).
-enum { kClsSplit = 0, kClsWarp, kClsCta, kClsSlot, kClsN };
-
-__global__ void k_c4_mark(const unsigned long long *cost, int64_t n, unsigned long long thr,
-                          unsigned long long lite, unsigned long long mid, int pidx, int pcnt,
-                          uint32_t *flags) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
-         a += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned long long c = a % pcnt == pidx ? cost[a] : 0ull;  // other parts' anchors
-        int cls = -1;
-        if (c > thr)
-            cls = kClsSplit;
-        else if (c > 0)
-            cls = c <= lite ? kClsWarp : c <= mid ? kClsCta : kClsSlot;
-#pragma unroll
-        for (int k = 0; k < kClsN; ++k) flags[k * n + a] = cls == k ? 1u : 0u;
-    }
-}
-
-__global__ void k_c4_compact(const uint32_t *flag, const uint32_t *pos, int64_t n,
-                             uint32_t *list) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
-         a += (int64_t)gridDim.x * blockDim.x)
-        if (flag[a]) list[pos[a]] = (uint32_t)a;
 }
 
 // ------------------------------------------------------------ up lists ----
@@ -2051,6 +1775,13 @@ __global__ void __launch_bounds__(kRowsThreads) k_k4_rows(K4GParams p, const uin
     }
 }
 
+__global__ void k_compact_flags(const uint32_t *flag, const uint32_t *pos, int64_t n,
+                                uint32_t *list) {
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
+         a += (int64_t)gridDim.x * blockDim.x)
+        if (flag[a]) list[pos[a]] = (uint32_t)a;
+}
+
 __global__ void k_flag_range(const int64_t *uoff, int64_t n, int lo, int hi, int pidx, int pcnt,
                              uint32_t *flag) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
@@ -2107,16 +1838,6 @@ int c4_pairs_conf(int64_t n4, PairsConf &c) {
     TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_c4_pairs, kC4Threads, c.smem));
     c.grid = (int64_t)tg_num_sms() * (per > 0 ? per : 1);
     return TG_OK;
-}
-
-// shared memory of k_c4_warp / k_c4_cta with tables of 2^lg slots
-size_t c4_warp_smem(int64_t n4, int L, int lg) {
-    const size_t e = (size_t)1 << lg;
-    return (size_t)n4 * 8 + (size_t)kC4WarpWarps * (e + ((e * L + 1) >> 1)) * 4;
-}
-size_t c4_cta_smem(int64_t n4, int L, int lg) {
-    const size_t e = (size_t)1 << lg;
-    return (size_t)n4 * 8 + 8 + (e + ((e * L + 1) >> 1)) * 4;
 }
 
 // Global-mode waves of the split anchors list[0 .. nheavy) (degrees hdeg):
@@ -2397,75 +2118,19 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
     if (per_sm < 1) per_sm = 1;
     const int64_t full_grid = (int64_t)tg_num_sms() * per_sm;
 
-    // anchor costs and classes
-    DevBuf<unsigned long long> cost, total;
-    DevBuf<uint32_t> flags, pos;
-    if (!cost.alloc(n, s) || !total.alloc(1, s) || !flags.alloc((size_t)kClsN * n, s) ||
-        !pos.alloc((size_t)kClsN * n, s))
-        return TG_ENOMEM;
-    TG_TRY_CUDA(cudaMemsetAsync(total.p, 0, 8, s));
-    const unsigned wgrid = (unsigned)std::min<int64_t>((n * 32 + 255) / 256, 65535LL * 16);
-    k_c4_cost<<<wgrid, 256, 0, s>>>(g->rowptr, g->adj, n, cost.p, total.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    unsigned long long tot = 0;
-    TG_TRY_CUDA(cudaMemcpyAsync(&tot, total.p, 8, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaStreamSynchronize(s));
-    // Global mode: anchors whose far ends fit half a warp table (2^lg_w
-    // slots) or half a CTA table (2^lg_c) count in shared memory; costlier
-    // ones are split over the grid.  Per-edge mode: anchors above a share of
-    // the total are split, the others take one CTA and a counter slot each.
-    // hash_slots caps the warp table; unroll 1 splits none, 4 every anchor.
-    int lg_w = 0, lg_c = 0;
-    if (global) {
-        lg_w = kC4WarpLgMax;
-        while (lg_w > 5 && ((1 << lg_w) > t.hash_slots ||
-                            c4_warp_smem(n4, L, lg_w) > (size_t)tg_smem_optin() - 1024))
-            --lg_w;
-        lg_c = kC4CtaLgMax;
-        while (lg_c > lg_w && c4_cta_smem(n4, L, lg_c) > (size_t)tg_smem_optin() - 1024) --lg_c;
-    }
-    const unsigned long long lite = global ? (1ull << lg_w) / 2 : 0ull;
-    const unsigned long long mid = global ? (1ull << lg_c) / 2 : 0ull;
-    unsigned long long thr =
-        global ? mid
-               : std::max<unsigned long long>(tot / (unsigned long long)(16 * full_grid),
-                                              (unsigned long long)1 << 12);
-    if (t.unroll == 1) thr = ~0ull;
-    if (t.unroll == 4) thr = 0ull;
-    const unsigned egrid = (unsigned)std::min<int64_t>((n + 255) / 256, 65535LL * 16);
-    k_c4_mark<<<egrid, 256, 0, s>>>(cost.p, n, thr, lite, mid, part.index, part.count, flags.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    for (int k = 0; k < kClsN; ++k) TG_TRY(tg_scan_u32(flags.p + (size_t)k * n, pos.p + (size_t)k * n, n, s));
-    uint32_t lastp[kClsN], lastf[kClsN];
-    for (int k = 0; k < kClsN; ++k) {
-        TG_TRY_CUDA(cudaMemcpyAsync(&lastp[k], pos.p + (size_t)k * n + n - 1, 4, cudaMemcpyDeviceToHost, s));
-        TG_TRY_CUDA(cudaMemcpyAsync(&lastf[k], flags.p + (size_t)k * n + n - 1, 4, cudaMemcpyDeviceToHost, s));
-    }
-    TG_TRY_CUDA(cudaStreamSynchronize(s));
-    int64_t ncls[kClsN];
-    DevBuf<uint32_t> lists[kClsN];
-    for (int k = 0; k < kClsN; ++k) {
-        ncls[k] = (int64_t)lastp[k] + lastf[k];
-        if (ncls[k] == 0) continue;
-        if (!lists[k].alloc(ncls[k], s)) return TG_ENOMEM;
-        k_c4_compact<<<egrid, 256, 0, s>>>(flags.p + (size_t)k * n, pos.p + (size_t)k * n, n,
-                                           lists[k].p); tg_note_launch();
-        TG_TRY_CUDA(cudaGetLastError());
-    }
-    const int64_t nheavy = ncls[kClsSplit];
-    const uint32_t *list = lists[kClsSplit].p;
+    // Anchors by walk cost: light ones count in shared memory (tg_c4_light.cu),
+    // costlier ones are split over the grid (unroll 1 splits none, 4 every
+    // anchor), the rest of them take one CTA and a counter slot each.
+    C4Lists cls;
+    TG_TRY(tg_c4_classify(g, t, part, global, cls, s));
+    const int64_t nheavy = cls.size[kC4Split];
+    std::vector<C4HeavyInfo> info((size_t)nheavy);
+    TG_TRY(tg_c4_heavy(g, cls, info.data(), s));
     std::vector<uint32_t> heavy((size_t)nheavy);
     std::vector<int64_t> hdeg((size_t)nheavy);
-    if (nheavy > 0) {
-        TG_TRY_CUDA(cudaMemcpyAsync(heavy.data(), list, nheavy * 4, cudaMemcpyDeviceToHost, s));
-        TG_TRY_CUDA(cudaStreamSynchronize(s));
-        // degrees of the split anchors: the list is ascending, so one copy of
-        // rowptr up to the largest of them
-        const int64_t top = (int64_t)heavy[(size_t)nheavy - 1] + 2;
-        std::vector<int64_t> rp((size_t)top);
-        TG_TRY_CUDA(cudaMemcpyAsync(rp.data(), g->rowptr, top * 8, cudaMemcpyDeviceToHost, s));
-        TG_TRY_CUDA(cudaStreamSynchronize(s));
-        for (int64_t q = 0; q < nheavy; ++q) hdeg[q] = rp[heavy[q] + 1] - rp[heavy[q]];
+    for (int64_t q = 0; q < nheavy; ++q) {
+        heavy[q] = info[q].a;
+        hdeg[q] = info[q].degree;
     }
 
     // counter slots: one per CTA of k_c4, one per split anchor of a wave; all
@@ -2474,7 +2139,7 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
     const int64_t slot_words = n * (L + 1) + (n + 31) / 32;
     const size_t slot_bytes = (size_t)slot_words * 4;
     int64_t want = 0;
-    if (ncls[kClsSlot] > 0) want = std::min<int64_t>(full_grid, ncls[kClsSlot]);
+    if (cls.size[kC4Slot] > 0) want = std::min<int64_t>(full_grid, cls.size[kC4Slot]);
     if (nheavy > 0)
         want = std::max<int64_t>(want, std::min<int64_t>(walk_waves ? kWaveMax : full_grid, nheavy));
     size_t free_b = 0, total_b = 0;
@@ -2485,9 +2150,6 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
         slots = 1;
     }
     DevBuf<uint32_t> scratch;
-    DevBuf<unsigned long long> queue;
-    if (!queue.alloc(kClsN, s)) return TG_ENOMEM;
-    TG_TRY_CUDA(cudaMemsetAsync(queue.p, 0, kClsN * 8, s));
     if (slots > 0) {
         if (!scratch.alloc((size_t)slots * slot_words, s)) return TG_ENOMEM;
         TG_TRY_CUDA(cudaMemsetAsync(scratch.p, 0, (size_t)slots * slot_bytes, s));
@@ -2503,7 +2165,6 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
     p.acc_l2 = global ? 0 : L2;
     p.scratch = scratch.p;
     p.slot_words = slot_words;
-    p.queue = queue.p;
     p.c4e = c4e;
     p.g4 = g4;
     p.n4 = n4;
@@ -2519,16 +2180,6 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
         // the others to waves of `slots` anchors counting in global memory,
         // whose far ends k_c4_pairs takes
         const int64_t bin_fill = t.c4_bin_fill > 0 ? t.c4_bin_fill : kBinFill;
-        std::vector<unsigned long long> hcost((size_t)nheavy);
-        {
-            DevBuf<unsigned long long> hc;
-            if (!hc.alloc(nheavy, s)) return TG_ENOMEM;
-            k_gather_u64<<<(unsigned)std::min<int64_t>((nheavy + 255) / 256, 4096), 256, 0, s>>>(
-                cost.p, list, nheavy, hc.p); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-            TG_TRY_CUDA(cudaMemcpyAsync(hcost.data(), hc.p, nheavy * 8, cudaMemcpyDeviceToHost, s));
-            TG_TRY_CUDA(cudaStreamSynchronize(s));
-        }
         size_t fb = 0, tb = 0;
         TG_TRY_CUDA(cudaMemGetInfo(&fb, &tb));
         // bucket entries of one wave: 2 bytes each, within an eighth of free memory
@@ -2539,8 +2190,8 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
             const int half = hdeg[q] < 65536 ? 1 : 0;
             const int wlg = c4_bin_wlg(L, half);
             const int64_t span = ((n - 1) >> wlg) - ((int64_t)heavy[q] >> wlg) + 1;
-            const bool bin = t.unroll != 1 && hcost[q] >= (unsigned long long)bin_fill * span &&
-                             hcost[q] <= (unsigned long long)ecap;
+            const bool bin = t.unroll != 1 && info[q].cost >= (unsigned long long)bin_fill * span &&
+                             info[q].cost <= (unsigned long long)ecap;
             (bin ? lb : ls).push_back(heavy[q]);
             (bin ? db : ds).push_back(hdeg[q]);
         }
@@ -2574,7 +2225,9 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
         }
         wave_start.push_back((int64_t)units.size());
         DevBuf<int4> du;
-        if (!du.alloc(units.size(), s)) return TG_ENOMEM;
+        DevBuf<uint32_t> dl;
+        if (!du.alloc(units.size(), s) || !dl.alloc(nheavy, s)) return TG_ENOMEM;
+        TG_TRY_CUDA(cudaMemcpyAsync(dl.p, heavy.data(), nheavy * 4, cudaMemcpyHostToDevice, s));
         TG_TRY_CUDA(cudaMemcpyAsync(du.p, units.data(), units.size() * sizeof(int4),
                                     cudaMemcpyHostToDevice, s));
         DevBuf<unsigned long long> wq;
@@ -2593,49 +2246,21 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
                 k_c4_split<<<(unsigned)grid, kC4Threads, smem, s>>>(ps); tg_note_launch();
                 TG_TRY_CUDA(cudaGetLastError());
             }
-            k_c4_pairs<<<(unsigned)pgrid, kC4Threads, psmem, s>>>(ps, list + a0, (int)na, ppriv); tg_note_launch();
+            k_c4_pairs<<<(unsigned)pgrid, kC4Threads, psmem, s>>>(ps, dl.p + a0, (int)na, ppriv); tg_note_launch();
             TG_TRY_CUDA(cudaGetLastError());
         }
-        // the host vectors are read by the copy above before they go out of scope
+        // the host vectors are read by the copies above before they go out of scope
         TG_TRY_CUDA(cudaStreamSynchronize(s));
     }
-    // light anchors: one warp each, a CTA each, in shared memory
-    if (ncls[kClsWarp] > 0) {
-        const size_t wsmem = c4_warp_smem(n4, L, lg_w);
-        TG_TRY(tg_allow_max_smem((const void *)k_c4_warp));
-        int wper = 0;
-        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper, k_c4_warp,
-                                                                  kC4WarpWarps * 32, wsmem));
-        if (wper < 1) wper = 1;
-        int64_t wg = (int64_t)tg_num_sms() * wper;
-        wg = std::min<int64_t>(wg, (ncls[kClsWarp] + 32 * kC4WarpWarps - 1) / (32 * kC4WarpWarps));
-        C4Params pw = p;
-        pw.queue = queue.p + kClsWarp;
-        k_c4_warp<<<(unsigned)wg, kC4WarpWarps * 32, wsmem, s>>>(pw, lists[kClsWarp].p,
-                                                                  ncls[kClsWarp], cost.p, lg_w); tg_note_launch();
-        TG_TRY_CUDA(cudaGetLastError());
-    }
-    if (ncls[kClsCta] > 0) {
-        const size_t csmem = c4_cta_smem(n4, L, lg_c);
-        TG_TRY(tg_allow_max_smem((const void *)k_c4_cta));
-        int cper = 0;
-        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cper, k_c4_cta, kC4CtaThreads,
-                                                                  csmem));
-        if (cper < 1) cper = 1;
-        const int64_t cg = std::min<int64_t>((int64_t)tg_num_sms() * cper, ncls[kClsCta]);
-        C4Params pc = p;
-        pc.queue = queue.p + kClsCta;
-        k_c4_cta<<<(unsigned)cg, kC4CtaThreads, csmem, s>>>(pc, lists[kClsCta].p, ncls[kClsCta],
-                                                             cost.p, lg_c); tg_note_launch();
-        TG_TRY_CUDA(cudaGetLastError());
-    }
+    TG_TRY(tg_c4_light(g, cls, c4e, g4, work, s));
     // the other anchors, one CTA and counter slot each
-    if (ncls[kClsSlot] > 0) {
+    if (cls.size[kC4Slot] > 0) {
         C4Params pl = p;
-        pl.queue = queue.p + kClsSlot;
+        pl.queue = cls.queue.p + kC4Classes + kC4Slot;
         pl.phase = 0;
-        const int64_t grid = std::min<int64_t>(slots, ncls[kClsSlot]);
-        k_c4<<<(unsigned)grid, kC4Threads, smem, s>>>(pl, lists[kClsSlot].p, ncls[kClsSlot]); tg_note_launch();
+        const int64_t grid = std::min<int64_t>(slots, cls.size[kC4Slot]);
+        k_c4<<<(unsigned)grid, kC4Threads, smem, s>>>(pl, cls.list.p + (int64_t)kC4Slot * n,
+                                                      cls.size[kC4Slot]); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
     }
     return TG_OK;
@@ -2737,7 +2362,7 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
                 k_flag_range<<<egrid, 256, 0, s>>>(uoff.p, n, lo, hi, part.index, part.count, flag.p); tg_note_launch();
                 TG_TRY_CUDA(cudaGetLastError());
                 TG_TRY(tg_scan_u32(flag.p, pos.p, n, s));
-                k_c4_compact<<<egrid, 256, 0, s>>>(flag.p, pos.p, n, list.p); tg_note_launch();
+                k_compact_flags<<<egrid, 256, 0, s>>>(flag.p, pos.p, n, list.p); tg_note_launch();
                 TG_TRY_CUDA(cudaGetLastError());
                 uint32_t lastp = 0, lastf = 0;
                 TG_TRY_CUDA(cudaMemcpyAsync(&lastp, pos.p + n - 1, 4, cudaMemcpyDeviceToHost, s));
