@@ -699,6 +699,158 @@ __global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_walk(C4Params p) {
     }
 }
 
+// Pass 1 of a wave in per-edge mode: one warp per unit, for every wedge a-u-b
+// of it whose far end has another middle the cycles closed with those, added
+// to the rows of its two edges.  A member's list of 32 entries or more is taken
+// by the whole warp: its entries are sorted by type, so the part of edge (a, u)
+// is summed over the warp per type of b and kept in registers, one add per
+// (type of b, type of the other middle); only the row of (u, b) takes an add
+// per wedge.  Shorter lists are taken 32 positions at a time across members,
+// both rows by adds.  Before, a CTA's threads added every wedge of a member to
+// one shared-memory accumulator, up to 32 lanes on one address (13.4 ms for
+// the 5.5e7 wedges of CL-125K, L = 5, against 1.8 ms here).  Bound by the adds
+// to the rows of (u, b), one per wedge and type of middle.
+constexpr int kWedgeLong = 32;
+
+template <int LP>
+__device__ __forceinline__ uint32_t wedge_counts(const C4Params &p, const uint32_t *cnt, uint32_t b,
+                                                 bool ok, uint32_t (&c)[LP]) {
+    uint32_t sum = 0;
+#pragma unroll
+    for (int t = 0; t < LP; ++t) {
+        c[t] = ok && t < p.L ? __ldg(cnt + (int64_t)b * p.L + t) : 0u;
+        sum += c[t];
+    }
+    return sum;
+}
+
+template <int LP>
+__global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_wedges(C4Params p) {
+    const int lane = threadIdx.x & 31, L = p.L, L2 = L * L;
+    for (;;) {
+        unsigned long long item = 0;
+        if (lane == 0) item = atomicAdd(p.queue, 1ull);
+        item = __shfl_sync(kFull, item, 0);
+        if (item >= (unsigned long long)p.n_units) break;
+        const C4Unit un = p.wunits[item];
+        const uint32_t a = p.heavy[un.q];
+        const int ta = p.ntype[a];
+        const int64_t ba = p.rowptr[a];
+        const int da = (int)(p.rowptr[a + 1] - ba);
+        const uint32_t *cnt = p.scratch + (un.q - p.q0) * p.slot_words;
+        int64_t at = p.mprefix[p.pbase[un.q] + un.m];
+        for (int m = un.m; m < da && at < un.hi; m += 32) {
+            const int x = m + lane;
+            int64_t len = 0, bu = 0;
+            uint32_t wu = 0;
+            if (x < da) {
+                wu = __ldg(p.adj + ba + x);
+                const uint32_t u = wu & TG_IDMASK;
+                if (u > a) {
+                    bu = p.rowptr[u];
+                    const int64_t du = p.rowptr[u + 1] - bu;
+                    if (du > 1) len = du;
+                }
+            }
+            int64_t incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int64_t first = at + incl - len;  // walk position of this member's list
+            at += __shfl_sync(kFull, incl, 31);
+            // long lists, the part inside the unit
+            unsigned todo = __ballot_sync(kFull, len >= kWedgeLong && first < un.hi && first + len > un.lo);
+            for (; todo; todo &= todo - 1u) {
+                const int src = __ffs(todo) - 1;
+                const int64_t lbu = __shfl_sync(kFull, bu, src), lf = __shfl_sync(kFull, first, src);
+                const int64_t ll = __shfl_sync(kFull, len, src);
+                const uint32_t lw = __shfl_sync(kFull, wu, src);
+                const uint32_t u = lw & TG_IDMASK;
+                const int tu = (int)(lw >> TG_TSHIFT);
+                const int64_t p0 = un.lo > lf ? un.lo - lf : 0, p1 = un.hi - lf < ll ? un.hi - lf : ll;
+                unsigned long long *row_au = p.c4e + (int64_t)__ldg(p.eid + ba + m + src) * L2;
+                unsigned long long acc = 0;  // lane t: cycles with b of type cur, the other middle of type t
+                int cur = 0;
+                for (int64_t c0 = p0; c0 < p1; c0 += 32) {
+                    const int64_t pos = lbu + c0 + lane;
+                    const uint32_t wb = c0 + lane < p1 ? __ldg(p.adj + pos) : 0u;
+                    const uint32_t b = wb & TG_IDMASK;
+                    bool ok = c0 + lane < p1 && b > a;
+                    if (!__any_sync(kFull, ok)) continue;
+                    uint32_t c[LP];
+                    ok = wedge_counts<LP>(p, cnt, b, ok, c) >= 2u;
+                    unsigned left = __ballot_sync(kFull, ok);
+                    if (!left) continue;
+                    const int tb = (int)(wb >> TG_TSHIFT);
+                    const bool ub = u > b;
+                    unsigned long long *row_ub =
+                        ok ? p.c4e + (int64_t)__ldg(p.eid + pos) * L2 + (ub ? ta * L : ta) : nullptr;
+#pragma unroll
+                    for (int t = 0; t < LP; ++t) {
+                        c[t] = ok ? c[t] - (t == tu ? 1u : 0u) : 0u;
+                        if (c[t]) atomicAdd(row_ub + (ub ? t : t * L), (unsigned long long)c[t]);
+                    }
+                    while (left) {
+                        const int g = __shfl_sync(kFull, tb, __ffs(left) - 1);
+                        left &= ~__ballot_sync(kFull, tb == g);
+                        if (g != cur) {
+                            if (lane < L && acc) atomicAdd(row_au + cur * L + lane, acc);
+                            acc = 0;
+                            cur = g;
+                        }
+#pragma unroll
+                        for (int t = 0; t < LP; ++t) {
+                            if (t >= L) continue;
+                            const unsigned sum = __reduce_add_sync(kFull, tb == g ? c[t] : 0u);
+                            if (lane == t) acc += sum;
+                        }
+                    }
+                }
+                if (lane < L && acc) atomicAdd(row_au + cur * L + lane, acc);
+            }
+            // short lists that begin inside the unit, as one sequence
+            const int ls = len < kWedgeLong && first >= un.lo && first < un.hi ? (int)len : 0;
+            int si = ls;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(kFull, si, o);
+                if (lane >= o) si += y;
+            }
+            const int total = __shfl_sync(kFull, si, 31);
+            const int64_t org = bu - (si - ls);
+            for (int c0 = 0; c0 < total; c0 += 32) {
+                const int pos = c0 + lane;
+                int r = 0;  // the member whose list holds pos
+#pragma unroll
+                for (int st = 16; st > 0; st >>= 1) {
+                    const int v = __shfl_sync(kFull, si, r + st - 1);
+                    if (v <= pos) r += st;
+                }
+                const int64_t e = __shfl_sync(kFull, org, r) + pos;
+                const uint32_t wr = __shfl_sync(kFull, wu, r);
+                const uint32_t wb = pos < total ? __ldg(p.adj + e) : 0u;
+                const uint32_t b = wb & TG_IDMASK;
+                uint32_t c[LP];
+                if (wedge_counts<LP>(p, cnt, b, pos < total && b > a, c) < 2u) continue;
+                const int tu = (int)(wr >> TG_TSHIFT);
+                const bool ub = (wr & TG_IDMASK) > b;
+                unsigned long long *row_ub = p.c4e + (int64_t)__ldg(p.eid + e) * L2 + (ub ? ta * L : ta);
+                unsigned long long *row_au =
+                    p.c4e + (int64_t)__ldg(p.eid + ba + m + r) * L2 + (int)(wb >> TG_TSHIFT) * L;
+#pragma unroll
+                for (int t = 0; t < LP; ++t) {
+                    const uint32_t v = c[t] ? c[t] - (t == tu ? 1u : 0u) : 0u;
+                    if (!v) continue;
+                    atomicAdd(row_ub + (ub ? t : t * L), (unsigned long long)v);
+                    atomicAdd(row_au + t, (unsigned long long)v);
+                }
+            }
+        }
+    }
+}
+
 // One count into the histogram under the sorted multiset {a, b, c, d}.
 __device__ __forceinline__ void k4_hist_add(unsigned long long *h4, int a, int b, int c, int d,
                                             unsigned long long v) {
@@ -1111,6 +1263,7 @@ struct K4Params {
     unsigned long long *g4;    // global mode: C(L+3,4) 4-clique counts by type multiset
     int64_t n4;
     unsigned long long *work;  // [5]: candidate tests, [6]: 4-cliques
+    int64_t min_d0;            // only x0 with up lists longer than this
 };
 
 constexpr int kK4Warps = 8;
@@ -1146,7 +1299,7 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
         const uint32_t x0 = (uint32_t)item;
         const int64_t b0 = p.uoff[x0];
         const int d0 = (int)(p.uoff[x0 + 1] - b0);
-        if (d0 < 3) continue;  // x0 is the lowest node: three more above it
+        if (d0 < 3 || d0 <= p.min_d0) continue;  // x0 is the lowest node: three more above it
         const int t0 = p.ntype[x0];
         const int32_t *to0 = p.utoff + (int64_t)x0 * (L + 1);
         for (int c0 = 0; c0 < d0; c0 += 32) {
@@ -1350,8 +1503,6 @@ struct K4GParams {
     unsigned long long *g4;
     int64_t n4;
     unsigned long long *work;
-    uint32_t *rows;       // k_k4_rows: per CTA rows_stride words of bitmap rows
-    int64_t rows_stride;
     int32_t pidx, pcnt;   // only lowest nodes x0 with x0 mod pcnt == pidx
 };
 
@@ -1525,272 +1676,7 @@ __global__ void __launch_bounds__(kK4GWarps * 32) k_k4_global(K4GParams p) {
     }
 }
 
-// 4-cliques by type multiset (global mode) from bitmaps.  The cliques whose
-// lowest node is x0 are the triangles of the graph on up(x0): with bm_v the
-// set of positions (in x0's up list) of up(v) n up(x0), every clique
-// x0 < v < w < x is met once, at the pair (v, w in bm_v), as a bit of
-// bm_v & bm_w; up(x0) is sorted by (type, id), so the bits of one type form a
-// contiguous range and popc(bm_v & bm_w & mask_t) counts the cliques whose
-// fourth node has type t.
-constexpr int kBitsWarpMax = 32;    // up lists of at most 32: one word, one warp
-constexpr int kBitsWarps = 8;
-
-__device__ __forceinline__ uint32_t range_mask(int lo, int hi) {  // bits [lo, hi) of a word
-    lo = max(0, min(32, lo));
-    hi = max(0, min(32, hi));
-    if (hi <= lo) return 0u;
-    const uint32_t h = hi == 32 ? 0xffffffffu : ((1u << hi) - 1u);
-    const uint32_t l = lo == 32 ? 0xffffffffu : ((1u << lo) - 1u);
-    return h & ~l;
-}
-
-
-__global__ void __launch_bounds__(kBitsWarps * 32) k_k4_bits_warp(K4GParams p) {
-    __shared__ uint32_t hk[kBitsWarps][2 * kBitsWarpMax], hv[kBitsWarps][2 * kBitsWarpMax];
-    __shared__ uint32_t tmask[kBitsWarps][TG_MAX_TYPES];
-    extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int L = p.L;
-    for (int64_t q = threadIdx.x; q < p.n4; q += blockDim.x) h4[q] = 0ull;
-    __syncthreads();
-    unsigned long long wk = 0, wpairs = 0;
-    for (;;) {
-        unsigned long long item = 0;
-        if (lane == 0) item = atomicAdd(p.queue, 1ull);
-        item = __shfl_sync(kFull, item, 0);
-        if (item >= (unsigned long long)p.n) break;
-        const uint32_t x0 = (uint32_t)item;
-        const int64_t b0 = __ldg(p.uoff + x0);
-        const int d0 = (int)(__ldg(p.uoff + x0 + 1) - b0);
-        if (d0 < 3 || d0 > kBitsWarpMax || (int64_t)x0 % p.pcnt != p.pidx) continue;
-        const int t0 = p.ntype[x0];
-        const int32_t *to0 = p.utoff + (int64_t)x0 * (L + 1);
-        // position of every up(x0) member, and the type ranges as masks
-        hk[warp][lane] = 0u;
-        hk[warp][lane + 32] = 0u;
-        if (lane < L) tmask[warp][lane] = range_mask(__ldg(to0 + lane), __ldg(to0 + lane + 1));
-        __syncwarp();
-        const uint32_t ve = lane < d0 ? __ldg(p.uadj + b0 + lane) : 0u;
-        if (lane < d0) hmap_put(hk[warp], hv[warp], 6, ve & TG_IDMASK, (uint32_t)lane);
-        __syncwarp();
-        // bm of the member at position pv, one member at a time
-        uint32_t mine = 0;
-        for (int pv = 0; pv < d0; ++pv) {
-            const uint32_t v = __shfl_sync(kFull, ve, pv) & TG_IDMASK;
-            const int64_t bv = __ldg(p.uoff + v);
-            const int dv = (int)(__ldg(p.uoff + v + 1) - bv);
-            uint32_t acc = 0;
-            for (int c = lane; c < dv; c += 32) {
-                const uint32_t y = __ldg(p.uadj + bv + c) & TG_IDMASK;
-                const uint32_t pos = hmap_get(hk[warp], hv[warp], 6, y);
-                if (pos != 0xffffffffu) acc |= 1u << pos;
-            }
-            acc = __reduce_or_sync(kFull, acc);
-            if (lane == pv) mine = acc;
-        }
-        // pairs (v, w in bm_v): lane pv takes the members w of its bitmap in turn
-        const int tv = (int)(ve >> TG_TSHIFT);
-        uint32_t m = lane < d0 ? mine : 0u;
-        while (__any_sync(kFull, m != 0u)) {
-            const int q = m ? __ffs(m) - 1 : 0;
-            const uint32_t bw = __shfl_sync(kFull, mine, q);
-            const int tw = (int)(__shfl_sync(kFull, ve, q) >> TG_TSHIFT);
-            if (m) {
-                const uint32_t both = mine & bw;
-                for (int t = 0; t < L; ++t) {
-                    const int c = __popc(both & tmask[warp][t]);
-                    if (c) k4_hist_add(h4, t0, tv, tw, t, (unsigned long long)c);
-                }
-                wk += __popc(both);
-                ++wpairs;
-                m &= m - 1;
-            }
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    for (int64_t q = threadIdx.x; q < p.n4; q += blockDim.x)
-        if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
-    if (p.work && wk) atomicAdd(p.work + 6, wk);
-    if (p.work && wpairs) atomicAdd(p.work + 5, wpairs);
-}
-
-// Up lists longer than one word: one CTA per x0 (from `list`).  Positions in
-// up(x0) are laid out type by type, each type's range padded to whole 32-bit
-// words, so that every word of a bitmap covers one type.  Row q (member q of
-// up(x0), node v) is the bitmap of up(v) n up(x0) over these positions; one
-// warp builds it from v's up list through a shared-memory map from node id to
-// position and stores it in the CTA's slice of global memory (the rows are
-// read back from L2).  Every clique x0 < v < w < x is one bit of
-// row_v & row_w for a w in row_v: a warp takes v, keeps row_v in registers
-// (WPL words per lane), visits the set bits w of row_v in position order and
-// adds popc(row_v & row_w) per word to per-lane counters, flushed into the
-// type-multiset histogram whenever the type of w changes (the type of x is
-// the word's type).  One pair costs one coalesced row load per warp.
-constexpr int kRowsThreads = 512;
-constexpr int kRowsMaxWords = 128;
-
-template <int WPL>
-__device__ __forceinline__ uint32_t rows_pick(const uint32_t (&r)[WPL], int i) {
-    uint32_t x = r[0];
-#pragma unroll
-    for (int k = 1; k < WPL; ++k)
-        if (i == k) x = r[k];
-    return x;
-}
-
-// The per-lane counts of the words a lane holds (w of type tw so far) into
-// the histogram under {t0, tv, tw, type of the word}; clears them.
-template <int WPL>
-__device__ __forceinline__ void rows_flush(unsigned long long *h4, uint32_t (&acc)[WPL],
-                                           const int32_t *wt, int words, int lane, int t0, int tv,
-                                           int tw, unsigned long long &wk) {
-    if (tw < 0) return;
-#pragma unroll
-    for (int i = 0; i < WPL; ++i) {
-        const int kk = lane + 32 * i;
-        if (kk < words && acc[i]) {
-            k4_hist_add(h4, t0, tv, tw, wt[kk], (unsigned long long)acc[i]);
-            wk += acc[i];
-        }
-        acc[i] = 0u;
-    }
-}
-
-template <int WPL>
-__global__ void __launch_bounds__(kRowsThreads) k_k4_rows(K4GParams p, const uint32_t *list,
-                                                          uint32_t nlist) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
-    const int L = p.L;
-    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem);
-    const size_t h4b = ((size_t)p.n4 * 8 + 15) & ~(size_t)15;
-    uint32_t *hk = reinterpret_cast<uint32_t *>(smem + h4b);  // 2^p.hlg slots
-    uint32_t *hv = hk + (1 << p.hlg);
-    int32_t *wt = reinterpret_cast<int32_t *>(hv + (1 << p.hlg));  // type of each word
-    int32_t *ws = wt + kRowsMaxWords;        // first word of each type, L + 1
-    int32_t *to = ws + TG_MAX_TYPES + 1;     // type offsets of up(x0), L + 1
-    uint32_t *rb = reinterpret_cast<uint32_t *>(to + TG_MAX_TYPES + 1) + warp * kRowsMaxWords;
-    const volatile uint32_t *vrb = rb;
-    __shared__ unsigned long long s_item;
-    uint32_t *rows = p.rows + (size_t)blockIdx.x * (size_t)p.rows_stride;
-    for (int64_t q = tid; q < p.n4; q += blockDim.x) h4[q] = 0ull;
-    unsigned long long wk = 0, wpairs = 0;
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_item = atomicAdd(p.queue, 1ull);
-        __syncthreads();
-        const unsigned long long item = s_item;
-        if (item >= nlist) break;
-        const uint32_t x0 = list[item];
-        const int64_t b0 = __ldg(p.uoff + x0);
-        const int d0 = (int)(__ldg(p.uoff + x0 + 1) - b0);
-        const int t0 = p.ntype[x0];
-        const int32_t *to0 = p.utoff + (int64_t)x0 * (L + 1);
-        int lg = 5;
-        while ((1 << lg) < 2 * d0 && lg < p.hlg) ++lg;
-        if (tid <= L) to[tid] = __ldg(to0 + tid);
-        if (tid == 0) {
-            int w = 0;
-            for (int t = 0; t < L; ++t) {
-                ws[t] = w;
-                w += (__ldg(to0 + t + 1) - __ldg(to0 + t) + 31) >> 5;
-            }
-            ws[L] = w;
-        }
-        for (int q = tid; q < (1 << lg); q += blockDim.x) hk[q] = 0u;
-        __syncthreads();
-        const int words = ws[L];
-        for (int k = tid; k < words; k += blockDim.x) {
-            int t = 0;
-            while (t + 1 < L && ws[t + 1] <= k) ++t;
-            wt[k] = t;
-        }
-        for (int q = tid; q < d0; q += blockDim.x) {
-            const uint32_t e = __ldg(p.uadj + b0 + q);
-            const int t = (int)(e >> TG_TSHIFT);
-            hmap_put(hk, hv, lg, e & TG_IDMASK, (uint32_t)(32 * ws[t] + (q - to[t])));
-        }
-        __syncthreads();
-        // rows: warp per member v
-        for (int q = warp; q < d0; q += W) {
-            for (int k = lane; k < words; k += 32) rb[k] = 0u;
-            __syncwarp();
-            const uint32_t v = __ldg(p.uadj + b0 + q) & TG_IDMASK;
-            const int64_t bv = __ldg(p.uoff + v);
-            const int dv = (int)(__ldg(p.uoff + v + 1) - bv);
-            for (int c = lane; c < dv; c += 32) {
-                const uint32_t pp = hmap_get(hk, hv, lg, __ldg(p.uadj + bv + c) & TG_IDMASK);
-                if (pp != 0xffffffffu) atomicOr(rb + (pp >> 5), 1u << (pp & 31u));
-            }
-            __syncwarp();
-            for (int k = lane; k < words; k += 32) rows[(size_t)q * words + k] = vrb[k];
-            __syncwarp();
-        }
-        __syncthreads();
-        // pairs (v, w in row_v): warp per v
-        for (int q = warp; q < d0; q += W) {
-            const int tv = (int)(__ldg(p.uadj + b0 + q) >> TG_TSHIFT);
-            const uint32_t *rowv = rows + (size_t)q * words;
-            uint32_t rv[WPL], acc[WPL];
-#pragma unroll
-            for (int i = 0; i < WPL; ++i) {
-                const int kk = lane + 32 * i;
-                rv[i] = kk < words ? __ldcg(rowv + kk) : 0u;
-                acc[i] = 0u;
-            }
-            int cur = -1;
-            for (int k = 0; k < words; ++k) {
-                uint32_t x = __shfl_sync(kFull, rows_pick<WPL>(rv, k >> 5), k & 31);
-                if (!x) continue;
-                const int tw = wt[k];
-                if (tw != cur) {
-                    rows_flush<WPL>(h4, acc, wt, words, lane, t0, tv, cur, wk);
-                    cur = tw;
-                }
-                const int qb = to[tw] + 32 * (k - ws[tw]);  // member index of the word's bit 0
-                while (x) {
-                    const int b = __ffs(x) - 1;
-                    x &= x - 1u;
-                    const uint32_t *roww = rows + (size_t)(qb + b) * words;
-#pragma unroll
-                    for (int i = 0; i < WPL; ++i) {
-                        const int kk = lane + 32 * i;
-                        if (kk < words) acc[i] += (uint32_t)__popc(rv[i] & __ldcg(roww + kk));
-                    }
-                    ++wpairs;
-                }
-            }
-            rows_flush<WPL>(h4, acc, wt, words, lane, t0, tv, cur, wk);
-        }
-    }
-    __syncthreads();
-    for (int64_t q = tid; q < p.n4; q += blockDim.x)
-        if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
-    if (p.work) {
-        // wpairs is the same in every lane of a warp: count it once
-        if (lane == 0 && wpairs) atomicAdd(p.work + 5, wpairs);
-        if (wk) atomicAdd(p.work + 6, wk);
-    }
-}
-
-__global__ void k_compact_flags(const uint32_t *flag, const uint32_t *pos, int64_t n,
-                                uint32_t *list) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n;
-         a += (int64_t)gridDim.x * blockDim.x)
-        if (flag[a]) list[pos[a]] = (uint32_t)a;
-}
-
-__global__ void k_flag_range(const int64_t *uoff, int64_t n, int lo, int hi, int pidx, int pcnt,
-                             uint32_t *flag) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t d = uoff[v + 1] - uoff[v];
-        flag[v] = (d >= lo && d <= hi && v % pcnt == pidx) ? 1u : 0u;
-    }
-}
-
+// The longest up list.
 __global__ void k_max_i64(const int64_t *x, int64_t n, unsigned long long *mx) {
     unsigned long long m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -1840,10 +1726,10 @@ int c4_pairs_conf(int64_t n4, PairsConf &c) {
     return TG_OK;
 }
 
-// Global-mode waves of the split anchors list[0 .. nheavy) (degrees hdeg):
-// walk positions per anchor (k_c4_prefix), warp units of about a quarter of a
-// warp's share of each wave (k_c4_units), then per wave of K anchors (K =
-// slots of p.scratch) k_c4_walk and k_c4_pairs.
+// Waves of the split anchors list[0 .. nheavy) (degrees hdeg): walk positions
+// per anchor (k_c4_prefix), warp units of about a quarter of a warp's share of
+// each wave (k_c4_units), then per wave of K anchors (K = slots of p.scratch)
+// k_c4_walk, in per-edge mode k_c4_wedges, and k_c4_pairs.
 int c4_walk_waves(const C4Params &p, const tg_graph *g, const uint32_t *list, int64_t nheavy,
                   const std::vector<int64_t> &hdeg, int64_t K, cudaStream_t s) {
     PairsConf pc;
@@ -1866,17 +1752,22 @@ int c4_walk_waves(const C4Params &p, const tg_graph *g, const uint32_t *list, in
     int wper = 0;
     TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper, k_c4_walk, kC4WalkWarps * 32, 0));
     if (wper < 1) wper = 1;
+    void (*const wedges)(C4Params) = g->L <= 4 ? k_c4_wedges<4> : g->L <= 8 ? k_c4_wedges<8> : k_c4_wedges<16>;
+    int eper = 0;
+    TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&eper, wedges, kC4WalkWarps * 32, 0));
+    if (eper < 1) eper = 1;
     const int64_t walk_grid = (int64_t)tg_num_sms() * wper;
     const int64_t warps = walk_grid * kC4WalkWarps;
     // waves: runs of at most K consecutive anchors of one counter width; an
     // anchor with fewer than 2^16 neighbours counts in 16-bit halves (no
-    // count can reach 2^16), the others in 32-bit words
+    // count can reach 2^16), the others and per-edge mode in 32-bit words
+    const int64_t half_max = p.g4 ? 65536 : 0;
     std::vector<int64_t> wq0, wq1;
     std::vector<int> whalf;
     for (int64_t q = 0; q < nheavy;) {
-        const int half = hdeg[q] < 65536 ? 1 : 0;
+        const int half = hdeg[q] < half_max ? 1 : 0;
         int64_t e = q + 1;
-        while (e < nheavy && e - q < K && (hdeg[e] < 65536 ? 1 : 0) == half) ++e;
+        while (e < nheavy && e - q < K && (hdeg[e] < half_max ? 1 : 0) == half) ++e;
         wq0.push_back(q);
         wq1.push_back(e);
         whalf.push_back(half);
@@ -1900,11 +1791,11 @@ int c4_walk_waves(const C4Params &p, const tg_graph *g, const uint32_t *list, in
     DevBuf<C4Unit> dun;
     DevBuf<unsigned long long> dq;
     if (!dus.alloc(nheavy + 1, s) || !dtg.alloc(nheavy, s) || !dun.alloc(nunits ? nunits : 1, s) ||
-        !dq.alloc(nwaves, s))
+        !dq.alloc(2 * nwaves, s))
         return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemcpyAsync(dus.p, us.data(), (nheavy + 1) * 8, cudaMemcpyHostToDevice, s));
     TG_TRY_CUDA(cudaMemcpyAsync(dtg.p, tg.data(), nheavy * 8, cudaMemcpyHostToDevice, s));
-    TG_TRY_CUDA(cudaMemsetAsync(dq.p, 0, nwaves * 8, s));
+    TG_TRY_CUDA(cudaMemsetAsync(dq.p, 0, 2 * nwaves * 8, s));
     if (nunits > 0) {
         const unsigned ug = (unsigned)std::min<int64_t>((nunits + 255) / 256, 65535LL * 16);
         k_c4_units<<<ug, 256, 0, s>>>(dus.p, nheavy, dtg.p, dtot.p, dmp.p, dpb.p, list, g->rowptr,
@@ -1930,6 +1821,12 @@ int c4_walk_waves(const C4Params &p, const tg_graph *g, const uint32_t *list, in
             const int64_t grid = std::min<int64_t>(walk_grid, need);
             k_c4_walk<<<(unsigned)grid, kC4WalkWarps * 32, 0, s>>>(pd); tg_note_launch();
             TG_TRY_CUDA(cudaGetLastError());
+            if (!p.g4) {
+                pd.queue = dq.p + nwaves + w;
+                wedges<<<(unsigned)std::min<int64_t>((int64_t)tg_num_sms() * eper, need), kC4WalkWarps * 32,
+                         0, s>>>(pd); tg_note_launch();
+                TG_TRY_CUDA(cudaGetLastError());
+            }
         }
         k_c4_pairs<<<(unsigned)pgrid, kC4Threads, psmem, s>>>(pd, list + q0, (int)(q1 - q0), ppriv); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
@@ -2135,7 +2032,7 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
 
     // counter slots: one per CTA of k_c4, one per split anchor of a wave; all
     // within a quarter of free memory
-    const bool walk_waves = global && t.hash_slots >= 64;
+    const bool walk_waves = t.hash_slots >= 64;
     const int64_t slot_words = n * (L + 1) + (n + 31) / 32;
     const size_t slot_bytes = (size_t)slot_words * 4;
     int64_t want = 0;
@@ -2174,9 +2071,9 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
     p.bits_off = n * (L + 1);
 
     if (nheavy > 0 && walk_waves) {
-        // global mode: each split anchor's walk is cut into position ranges of
-        // about equal length (warp units); anchors whose walk averages
-        // bin_fill wedges per far-end window they span go to the binned waves,
+        // each split anchor's walk is cut into position ranges of about equal
+        // length (warp units); in global mode anchors whose walk averages
+        // bin_fill wedges per far-end window they span go to the binned waves;
         // the others to waves of `slots` anchors counting in global memory,
         // whose far ends k_c4_pairs takes
         const int64_t bin_fill = t.c4_bin_fill > 0 ? t.c4_bin_fill : kBinFill;
@@ -2190,7 +2087,7 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
             const int half = hdeg[q] < 65536 ? 1 : 0;
             const int wlg = c4_bin_wlg(L, half);
             const int64_t span = ((n - 1) >> wlg) - ((int64_t)heavy[q] >> wlg) + 1;
-            const bool bin = t.unroll != 1 && info[q].cost >= (unsigned long long)bin_fill * span &&
+            const bool bin = global && t.unroll != 1 && info[q].cost >= (unsigned long long)bin_fill * span &&
                              info[q].cost <= (unsigned long long)ecap;
             (bin ? lb : ls).push_back(heavy[q]);
             (bin ? db : ds).push_back(hdeg[q]);
@@ -2308,16 +2205,24 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     DevBuf<unsigned long long> queue;
     if (!queue.alloc(1, s)) return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemsetAsync(queue.p, 0, 8, s));
-    if (global) {
-        // hash sets sized to the largest up list, within the hash_slots cap
+    // bitmap kernels (tg_k4.cu); up lists beyond them, or with a hash_slots cap
+    // below 64 all of them, go to the hash-set kernels
+    int64_t maxup = 0, bits_max = 0;
+    if (t.hash_slots >= 64) {
+        int64_t nlong = 0;
+        const C4UpLists up{uoff.p, uadj.p, ueid.p, utoff.p};
+        TG_TRY(tg_k4_bits(g, up, k4e, g4, work, part, &nlong, &maxup, &bits_max, s));
+        if (nlong == 0) return TG_OK;
+    } else if (global) {
         DevBuf<unsigned long long> mx;
         if (!mx.alloc(1, s)) return TG_ENOMEM;
         TG_TRY_CUDA(cudaMemsetAsync(mx.p, 0, 8, s));
         k_max_i64<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(utot.p, n, mx.p); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
-        unsigned long long maxup = 0;
         TG_TRY_CUDA(cudaMemcpyAsync(&maxup, mx.p, 8, cudaMemcpyDeviceToHost, s));
         TG_TRY_CUDA(cudaStreamSynchronize(s));
+    }
+    if (global) {
         const size_t h4b = ((size_t)n4 * 8 + 15) & ~(size_t)15;
         K4GParams q{};
         q.uoff = uoff.p;
@@ -2333,80 +2238,8 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
         q.work = work;
         q.pidx = part.index;
         q.pcnt = part.count;
-        // bitmap kernels: one word for up lists of at most 32 (warp per x0),
-        // padded rows of up to kRowsMaxWords words beyond (CTA per x0, in
-        // three widths); a hash_slots cap below 64 sends every x0 to the
-        // hash-set kernel instead
-        const int bits_max = t.hash_slots >= 64 ? 32 * kRowsMaxWords - 31 * L : 0;
-        if (bits_max > 0) {
-            TG_TRY(tg_allow_max_smem((const void *)k_k4_bits_warp));
-            int wper = 0;
-            TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper, k_k4_bits_warp,
-                                                                      kBitsWarps * 32, h4b));
-            if (wper < 1) wper = 1;
-            int64_t wgrid2 = (int64_t)tg_num_sms() * wper;
-            if (wgrid2 > (n + kBitsWarps - 1) / kBitsWarps) wgrid2 = (n + kBitsWarps - 1) / kBitsWarps;
-            if (wgrid2 < 1) wgrid2 = 1;
-            k_k4_bits_warp<<<(unsigned)wgrid2, kBitsWarps * 32, h4b, s>>>(q); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-            DevBuf<uint32_t> flag, pos, list;
-            const unsigned egrid = (unsigned)std::min<int64_t>((n + 255) / 256, 65535LL * 16);
-            for (int wpl = 1; wpl <= 4; wpl *= 2) {
-                // up lists whose padded rows need at most 32 * wpl words: every
-                // type range adds at most 31 positions of padding
-                const int lo = wpl == 1 ? kBitsWarpMax + 1 : 32 * 16 * wpl - 31 * L + 1;
-                const int hi = 32 * 32 * wpl - 31 * L;
-                if ((unsigned long long)lo > maxup || hi < lo) continue;
-                if (!flag.p && (!flag.alloc(n, s) || !pos.alloc(n, s) || !list.alloc(n, s)))
-                    return TG_ENOMEM;
-                k_flag_range<<<egrid, 256, 0, s>>>(uoff.p, n, lo, hi, part.index, part.count, flag.p); tg_note_launch();
-                TG_TRY_CUDA(cudaGetLastError());
-                TG_TRY(tg_scan_u32(flag.p, pos.p, n, s));
-                k_compact_flags<<<egrid, 256, 0, s>>>(flag.p, pos.p, n, list.p); tg_note_launch();
-                TG_TRY_CUDA(cudaGetLastError());
-                uint32_t lastp = 0, lastf = 0;
-                TG_TRY_CUDA(cudaMemcpyAsync(&lastp, pos.p + n - 1, 4, cudaMemcpyDeviceToHost, s));
-                TG_TRY_CUDA(cudaMemcpyAsync(&lastf, flag.p + n - 1, 4, cudaMemcpyDeviceToHost, s));
-                TG_TRY_CUDA(cudaStreamSynchronize(s));
-                const uint32_t nlist = lastp + lastf;
-                if (nlist == 0) continue;
-                const int dmax = (int)std::min<unsigned long long>(maxup, (unsigned long long)hi);
-                int hlg = 5;
-                while ((1 << hlg) < 2 * dmax) ++hlg;
-                const size_t rsmem = h4b + (size_t)2 * (1u << hlg) * 4 +
-                                     (size_t)(kRowsMaxWords + 2 * (TG_MAX_TYPES + 1)) * 4 +
-                                     (size_t)(kRowsThreads / 32) * kRowsMaxWords * 4;
-                const void *kfn = wpl == 1 ? (const void *)k_k4_rows<1>
-                                  : wpl == 2 ? (const void *)k_k4_rows<2>
-                                             : (const void *)k_k4_rows<4>;
-                TG_TRY(tg_allow_max_smem(kfn));
-                int rper = 0;
-                TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, kfn, kRowsThreads,
-                                                                          rsmem));
-                if (rper < 1) rper = 1;
-                int64_t rgrid = (int64_t)tg_num_sms() * rper;
-                if (rgrid > nlist) rgrid = nlist;
-                K4GParams r = q;
-                r.hlg = hlg;
-                r.rows_stride = (int64_t)dmax * 32 * wpl;
-                DevBuf<uint32_t> rows;
-                if (!rows.alloc((size_t)rgrid * (size_t)r.rows_stride, s)) return TG_ENOMEM;
-                r.rows = rows.p;
-                TG_TRY_CUDA(cudaMemsetAsync(queue.p, 0, 8, s));
-                if (wpl == 1)
-                    k_k4_rows<1><<<(unsigned)rgrid, kRowsThreads, rsmem, s>>>(r, list.p, nlist);
-                else if (wpl == 2)
-                    k_k4_rows<2><<<(unsigned)rgrid, kRowsThreads, rsmem, s>>>(r, list.p, nlist);
-                else
-                    k_k4_rows<4><<<(unsigned)rgrid, kRowsThreads, rsmem, s>>>(r, list.p, nlist);
-                tg_note_launch();
-                TG_TRY_CUDA(cudaGetLastError());
-            }
-        }
-        if (maxup <= (unsigned long long)bits_max) return TG_OK;
-        // hash sets for the longer up lists, sized to the largest one, within
-        // the hash_slots cap
-        int gcap = (int)std::min<unsigned long long>(std::min(1024, t.hash_slots), (maxup + 31) & ~31ull);
+        // hash sets sized to the largest up list, within the hash_slots cap
+        int gcap = (int)std::min<int64_t>(std::min(1024, t.hash_slots), (maxup + 31) & ~(int64_t)31);
         if (gcap < 32) gcap = 32;
         int hlg = 5;
         while ((1 << hlg) < 2 * gcap) ++hlg;
@@ -2428,8 +2261,7 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
         if (ggrid < 1) ggrid = 1;
         q.cap = gcap;
         q.hlg = hlg;
-        q.min_d0 = bits_max;
-        TG_TRY_CUDA(cudaMemsetAsync(queue.p, 0, 8, s));
+        q.min_d0 = (int32_t)bits_max;
         k_k4_global<<<(unsigned)ggrid, kK4GWarps * 32, gsmem, s>>>(q); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
         return TG_OK;
@@ -2449,6 +2281,7 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     p.g4 = g4;
     p.n4 = n4;
     p.work = work;
+    p.min_d0 = bits_max;
     k_k4<<<(unsigned)grid, kK4Warps * 32, smem, s>>>(p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     return TG_OK;
