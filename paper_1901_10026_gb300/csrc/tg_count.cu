@@ -984,16 +984,25 @@ extern "C" int tg_autotune(const tg_graph *g, int32_t k, tg_tune *best, void *st
 
 // ----------------------------------------------------------- schedule -----
 struct tg_sched {
-    uint32_t *order = nullptr;          // M edge ids grouped by high-degree endpoint
+    tg_lists lists;                     // up lists, edge ids grouped by high-degree endpoint
+    uint32_t *sorted = nullptr;         // the edge ids sorted by (j, i) (shards, on first use)
     unsigned long long *s = nullptr;    // n neighbour-degree sums
-    int64_t M = 0, n = 0;
 };
+
+static void sched_dfree(tg_sched *sc, cudaStream_t s) {
+    tg_dfree(sc->lists.uoff, 0, s);
+    tg_dfree(sc->lists.utoff, 0, s);
+    tg_dfree(sc->lists.uadj, 0, s);
+    tg_dfree(sc->lists.ueid, 0, s);
+    tg_dfree(sc->lists.order, 0, s);
+    tg_dfree(sc->sorted, 0, s);
+    tg_dfree(sc->s, 0, s);
+}
 
 void tg_sched_free(tg_graph *g) {
     if (!g->sched) return;
     (void)cudaDeviceSynchronize();
-    tg_dfree(g->sched->order, 0, nullptr);
-    tg_dfree(g->sched->s, 0, nullptr);
+    sched_dfree(g->sched, nullptr);
     (void)cudaDeviceSynchronize();
     delete g->sched;
     g->sched = nullptr;
@@ -1001,8 +1010,7 @@ void tg_sched_free(tg_graph *g) {
 
 void tg_sched_free_on(tg_graph *g, cudaStream_t s) {
     if (!g->sched) return;
-    tg_dfree(g->sched->order, 0, s);
-    tg_dfree(g->sched->s, 0, s);
+    sched_dfree(g->sched, s);
     delete g->sched;
     g->sched = nullptr;
 }
@@ -1031,16 +1039,36 @@ static int get_sched(const tg_graph *g, cudaStream_t s, tg_sched **out) {
         *out = g->sched;
         return TG_OK;
     }
+    tg_sched *sc = new (std::nothrow) tg_sched();
+    if (!sc) return TG_ENOMEM;
+    int r = tg_build_lists(g, sc->lists, s);
+    // other threads may read the lists on their own streams from here on
+    if (r == TG_OK && cudaStreamSynchronize(s) != cudaSuccess) r = TG_ECUDA;
+    if (r != TG_OK) {
+        sched_dfree(sc, s);
+        delete sc;
+        return r;
+    }
+    g->sched = sc;
+    *out = sc;
+    return TG_OK;
+}
+
+int tg_graph_lists(const tg_graph *g, const tg_lists **out, cudaStream_t s) {
+    tg_sched *sc = nullptr;
+    TG_TRY(get_sched(g, s, &sc));
+    *out = &sc->lists;
+    return TG_OK;
+}
+
+// The edge ids sorted by (j, i): the order that shards are slices of.
+static int sched_sorted(const tg_graph *g, tg_sched *sc, cudaStream_t s) {
+    std::lock_guard<std::mutex> lk(g->mu);
+    if (sc->sorted) return TG_OK;
     DevBuf<uint32_t> order;
     TG_TRY(grouped_order(g, 0, g->M, s, order));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
-    tg_sched *sc = new (std::nothrow) tg_sched();
-    if (!sc) return TG_ENOMEM;
-    sc->M = g->M;
-    sc->n = g->n;
-    sc->order = order.release();
-    g->sched = sc;
-    *out = sc;
+    sc->sorted = order.release();
     return TG_OK;
 }
 
@@ -1210,11 +1238,11 @@ static int sums_impl(const tg_graph *g, int k, int64_t e0, int64_t e1,
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
     if (e0 == 0 && e1 == g->M)
-        return launch_count(g, k, TG_GRAPHLET, sc->order, sc->order, 0, g->M, nullptr, 0, dsums,
+        return launch_count(g, k, TG_GRAPHLET, sc->lists.order, sc->lists.order, 0, g->M, nullptr, 0, dsums,
                             s);
     DevBuf<uint32_t> order;
     TG_TRY(grouped_order(g, e0, e1 - e0, s, order));
-    return launch_count(g, k, TG_GRAPHLET, sc->order, order.p, 0, e1 - e0, nullptr, 0, dsums, s);
+    return launch_count(g, k, TG_GRAPHLET, sc->lists.order, order.p, 0, e1 - e0, nullptr, 0, dsums, s);
 }
 extern "C" int tg_count_global(const tg_graph *g, int32_t k, uint64_t *out, void *stream) {
     TG_TRY(check_counts(g, k));
@@ -1323,12 +1351,13 @@ extern "C" int tg_count_shard(const tg_graph *g, int32_t k, int32_t shard, int32
         TG_TRY_CUDA(cudaMemsetAsync(dsums, 0, len * 8, s));
         tg_sched *sc = nullptr;
         TG_TRY(get_sched(g, s, &sc));
+        TG_TRY(sched_sorted(g, sc, s));
         const int64_t M = g->M;
         int64_t q[2] = {0, 0};
         if (M > 0) {
             DevBuf<int64_t> cost, pre, qs;
             if (!cost.alloc(M + 1, s) || !pre.alloc(M + 1, s) || !qs.alloc(2, s)) return TG_ENOMEM;
-            k_order_cost<<<grid_for(M + 1), 256, 0, s>>>(sc->order, g->edges, g->rowptr, M, cost.p); tg_note_launch();
+            k_order_cost<<<grid_for(M + 1), 256, 0, s>>>(sc->sorted, g->edges, g->rowptr, M, cost.p); tg_note_launch();
             TG_TRY_CUDA(cudaGetLastError());
             TG_TRY(tg_scan_i64(cost.p, pre.p, M + 1, s));
             k_split_points<<<1, 32, 0, s>>>(pre.p, M, shard, nshards, qs.p); tg_note_launch();
@@ -1343,14 +1372,14 @@ extern "C" int tg_count_shard(const tg_graph *g, int32_t k, int32_t shard, int32
             part.index = shard;
             part.count = nshards;
             if (k == 4)
-                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->order, sc->order + q[0], q[1] - q[0],
+                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists.order, sc->sorted + q[0], q[1] - q[0],
                                       nullptr, 0, dsums, t, s, part));
             else if (q[1] > q[0])
-                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->order, sc->order + q[0], q[1] - q[0],
+                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists.order, sc->sorted + q[0], q[1] - q[0],
                                       nullptr, 0, dsums, t, s));
         } else if (q[1] > q[0]) {
             // the per-edge kernels need nothing beyond the slice's edges
-            TG_TRY(launch_count(g, k, TG_GRAPHLET, sc->order, sc->order + q[0], 0, q[1] - q[0],
+            TG_TRY(launch_count(g, k, TG_GRAPHLET, sc->lists.order, sc->sorted + q[0], 0, q[1] - q[0],
                                 nullptr, 0, dsums, s));
         }
     }
@@ -1369,13 +1398,13 @@ extern "C" int tg_count_per_edge(const tg_graph *g, int32_t k, int32_t level, ui
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
     if (tg_is_device_ptr(rows)) {
-        TG_TRY(launch_count(g, k, level, sc->order, sc->order, 0, g->M, rows, width, nullptr, s));
+        TG_TRY(launch_count(g, k, level, sc->lists.order, sc->lists.order, 0, g->M, rows, width, nullptr, s));
         TG_TRY_CUDA(cudaStreamSynchronize(s));
         return TG_OK;
     }
     DevBuf<uint64_t> d;
     if (!d.alloc((size_t)g->M * width, s)) return TG_ENOMEM;
-    TG_TRY(launch_count(g, k, level, sc->order, sc->order, 0, g->M, d.p, width, nullptr, s));
+    TG_TRY(launch_count(g, k, level, sc->lists.order, sc->lists.order, 0, g->M, d.p, width, nullptr, s));
     TG_TRY_CUDA(cudaMemcpyAsync(rows, d.p, (size_t)g->M * width * 8, cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
     return TG_OK;
@@ -1386,7 +1415,7 @@ int tg_rows_device(const tg_graph *g, int k, int level, uint64_t *rows, cudaStre
     if (g->M == 0) return TG_OK;
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
-    return launch_count(g, k, level, sc->order, sc->order, 0, g->M, rows,
+    return launch_count(g, k, level, sc->lists.order, sc->lists.order, 0, g->M, rows,
                         tg_slots(g->L, k, level), nullptr, s);
 }
 
@@ -1399,7 +1428,7 @@ int tg_rows_mapped(const tg_graph *g, int k, int level, uint64_t *const *rowmap,
     if (g->M > 0) {
         tg_sched *sc = nullptr;
         TG_TRY(get_sched(g, s, &sc));
-        TG_TRY(tg_reuse_count(g, k, level, sc->order, sc->order, g->M, nullptr,
+        TG_TRY(tg_reuse_count(g, k, level, sc->lists.order, sc->lists.order, g->M, nullptr,
                               tg_slots(g->L, k, level), nullptr, t, s, tg_part(), rowmap));
     }
     *done = true;

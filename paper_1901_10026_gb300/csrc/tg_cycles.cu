@@ -1188,68 +1188,9 @@ __global__ void __launch_bounds__(kBinPairThreads) k_c4_bin_pairs(C4Bin p) {
         if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
 }
 
-// ------------------------------------------------------------ up lists ----
-// Up list of v: its neighbours of higher rank (smaller new id), kept with
-// their typed offsets and edge ids.  In a (type, id)-sorted list they are a
-// prefix of every typed range.  One warp per node; lane t < L finds the end
-// of the prefix of type t.
-__global__ void k_up_count(const int64_t *rowptr, const uint32_t *adj, const int32_t *toff,
-                           int64_t n, int32_t L, int32_t *utoff, int64_t *utot) {
-    const int lane = threadIdx.x & 31;
-    const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = wid; v < n; v += nw) {
-        const int64_t b = rowptr[v];
-        const int32_t *to = toff + v * (L + 1);
-        int c = 0;
-        if (lane < L) {
-            int lo = __ldg(to + lane), hi = __ldg(to + lane + 1);
-            const int start = lo;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if ((int64_t)(__ldg(adj + b + mid) & TG_IDMASK) < v)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            c = lo - start;
-        }
-        int incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane < L) utoff[v * (L + 1) + lane + 1] = incl;
-        if (lane == 0) utoff[v * (L + 1)] = 0;
-        if (lane == L - 1) utot[v] = incl;
-    }
-}
-
-__global__ void k_up_fill(const int64_t *rowptr, const uint32_t *adj, const uint32_t *eid,
-                          const int32_t *toff, const int32_t *utoff, const int64_t *uoff,
-                          int64_t n, int32_t L, uint32_t *uadj, uint32_t *ueid) {
-    const int lane = threadIdx.x & 31;
-    const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = wid; v < n; v += nw) {
-        const int64_t b = rowptr[v], ub = uoff[v];
-        const int32_t *to = toff + v * (L + 1);
-        const int32_t *uto = utoff + v * (L + 1);
-        for (int t = 0; t < L; ++t) {
-            const int src = __ldg(to + t), dst = __ldg(uto + t);
-            const int c = __ldg(uto + t + 1) - dst;
-            for (int x = lane; x < c; x += 32) {
-                uadj[ub + dst + x] = __ldg(adj + b + src + x);
-                ueid[ub + dst + x] = __ldg(eid + b + src + x);
-            }
-        }
-    }
-}
-
 // ----------------------------------------------------------- 4-cliques ----
 struct K4Params {
-    const int64_t *uoff;       // up lists (see k_up_count)
+    const int64_t *uoff;       // up lists (tg_lists)
     const uint32_t *uadj;
     const uint32_t *ueid;
     const int32_t *utoff;
@@ -1677,11 +1618,11 @@ __global__ void __launch_bounds__(kK4GWarps * 32) k_k4_global(K4GParams p) {
 }
 
 // The longest up list.
-__global__ void k_max_i64(const int64_t *x, int64_t n, unsigned long long *mx) {
+__global__ void k_max_up(const int64_t *uoff, int64_t n, unsigned long long *mx) {
     unsigned long long m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)x[i]);
+        m = max(m, (unsigned long long)(uoff[i + 1] - uoff[i]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
     if ((threadIdx.x & 31) == 0 && m) atomicMax(mx, m);
@@ -2186,22 +2127,9 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     const int64_t need = (g->n + kK4Warps - 1) / kK4Warps;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    // up lists: each edge once, at its lower-ranked end
-    DevBuf<int32_t> utoff;
-    DevBuf<int64_t> utot, uoff;
-    DevBuf<uint32_t> uadj, ueid;
     const int64_t n = g->n;
-    if (!utoff.alloc((size_t)n * (L + 1), s) || !utot.alloc(n + 1, s) || !uoff.alloc(n + 1, s) ||
-        !uadj.alloc(g->M, s) || !ueid.alloc(g->M, s))
-        return TG_ENOMEM;
-    TG_TRY_CUDA(cudaMemsetAsync(utot.p + n, 0, 8, s));
-    const unsigned wgrid = (unsigned)std::min<int64_t>((n * 32 + 255) / 256, 65535LL * 16);
-    k_up_count<<<wgrid, 256, 0, s>>>(g->rowptr, g->adj, g->toff, n, L, utoff.p, utot.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY(tg_scan_i64(utot.p, uoff.p, n + 1, s));
-    k_up_fill<<<wgrid, 256, 0, s>>>(g->rowptr, g->adj, g->eid, g->toff, utoff.p, uoff.p, n, L,
-                                    uadj.p, ueid.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
+    const tg_lists *up = nullptr;
+    TG_TRY(tg_graph_lists(g, &up, s));
     DevBuf<unsigned long long> queue;
     if (!queue.alloc(1, s)) return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemsetAsync(queue.p, 0, 8, s));
@@ -2210,14 +2138,13 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     int64_t maxup = 0, bits_max = 0;
     if (t.hash_slots >= 64) {
         int64_t nlong = 0;
-        const C4UpLists up{uoff.p, uadj.p, ueid.p, utoff.p};
-        TG_TRY(tg_k4_bits(g, up, k4e, g4, work, part, &nlong, &maxup, &bits_max, s));
+        TG_TRY(tg_k4_bits(g, *up, k4e, g4, work, part, &nlong, &maxup, &bits_max, s));
         if (nlong == 0) return TG_OK;
     } else if (global) {
         DevBuf<unsigned long long> mx;
         if (!mx.alloc(1, s)) return TG_ENOMEM;
         TG_TRY_CUDA(cudaMemsetAsync(mx.p, 0, 8, s));
-        k_max_i64<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(utot.p, n, mx.p); tg_note_launch();
+        k_max_up<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(up->uoff, n, mx.p); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
         TG_TRY_CUDA(cudaMemcpyAsync(&maxup, mx.p, 8, cudaMemcpyDeviceToHost, s));
         TG_TRY_CUDA(cudaStreamSynchronize(s));
@@ -2225,9 +2152,9 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     if (global) {
         const size_t h4b = ((size_t)n4 * 8 + 15) & ~(size_t)15;
         K4GParams q{};
-        q.uoff = uoff.p;
-        q.uadj = uadj.p;
-        q.utoff = utoff.p;
+        q.uoff = up->uoff;
+        q.uadj = up->uadj;
+        q.utoff = up->utoff;
         q.ntype = g->ntype;
         q.n = n;
         q.m = g->M;
@@ -2267,10 +2194,10 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
         return TG_OK;
     }
     K4Params p{};
-    p.uoff = uoff.p;
-    p.uadj = uadj.p;
-    p.ueid = ueid.p;
-    p.utoff = utoff.p;
+    p.uoff = up->uoff;
+    p.uadj = up->uadj;
+    p.ueid = up->ueid;
+    p.utoff = up->utoff;
     p.ntype = g->ntype;
     p.n = g->n;
     p.L = L;

@@ -36,16 +36,9 @@ int tg_c4_light(const tg_graph *g, const C4Lists &cls, unsigned long long *c4e,
 // The split anchors, ascending, with their costs and degrees.
 int tg_c4_heavy(const tg_graph *g, const C4Lists &cls, C4HeavyInfo *host, cudaStream_t s);
 
-// Up lists (neighbours of higher rank, sorted by (type, id)) of every node.
-struct C4UpLists {
-    const int64_t *uoff;
-    const uint32_t *uadj, *ueid;
-    const int32_t *utoff;
-};
-
 // 4-cliques whose lowest node's up list has at most *bits_max entries
 // (tg_k4.cu), to the type-multiset totals g4 or (g4 = NULL) the per-edge
 // counters k4e.  *nlong and *longest: the lists left out, the longest of them.
-int tg_k4_bits(const tg_graph *g, const C4UpLists &up, unsigned long long *k4e, unsigned long long *g4,
+int tg_k4_bits(const tg_graph *g, const tg_lists &up, unsigned long long *k4e, unsigned long long *g4,
                unsigned long long *work, const tg_part &part, int64_t *nlong, int64_t *longest,
                int64_t *bits_max, cudaStream_t s);

@@ -22,6 +22,16 @@
 
 struct tg_sched;  // per-graph counting schedule (tg_count.cu)
 
+// Oriented lists of a graph (tg_lists.cu): the up list of node v, its neighbours
+// of smaller id sorted by (type, id), is uadj[uoff[v] .. uoff[v + 1]) with edge
+// ids ueid and type offsets utoff[v (L + 1) ..]; order holds the M edge ids
+// grouped by their end of smaller id j, in j's list order.
+struct tg_lists {
+    int64_t *uoff = nullptr;
+    int32_t *utoff = nullptr;
+    uint32_t *uadj = nullptr, *ueid = nullptr, *order = nullptr;
+};
+
 struct tg_graph {
     int64_t n = 0;
     int64_t m_input = 0;
@@ -118,6 +128,11 @@ int tg_radix_sort_kv(uint64_t *keys, uint64_t *tmp, uint32_t *vals, uint32_t *vt
                      int bits, cudaStream_t s, uint64_t **result, uint32_t **vresult);
 
 int tg_bitlen(uint64_t x);  // number of bits needed to represent x (0 -> 0)
+
+// The oriented lists of a graph, queued on s (tg_lists.cu).
+int tg_build_lists(const tg_graph *g, tg_lists &out, cudaStream_t s);
+// The graph's cached lists, made on first use (tg_count.cu).
+int tg_graph_lists(const tg_graph *g, const tg_lists **out, cudaStream_t s);
 
 // Counts every kernel this library launches (reported by tg_launch_count).
 void tg_note_launch();

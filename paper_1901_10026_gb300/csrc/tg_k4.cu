@@ -618,7 +618,7 @@ int launch_cliques(const unsigned long long (&size)[2 * kUpClasses], CliqueParam
 
 }  // namespace
 
-int tg_k4_bits(const tg_graph *g, const C4UpLists &up, unsigned long long *k4e, unsigned long long *g4,
+int tg_k4_bits(const tg_graph *g, const tg_lists &up, unsigned long long *k4e, unsigned long long *g4,
                unsigned long long *work, const tg_part &part, int64_t *nlong, int64_t *longest,
                int64_t *bits_max, cudaStream_t s) {
     const int64_t n = g->n;
