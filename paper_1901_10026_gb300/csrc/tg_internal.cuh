@@ -176,6 +176,9 @@ struct tg_units {
     uint32_t nunits = 0, nheavy = 0, nlight = 0;
 };
 
+// The units of the edges ord[0 .. cnt) (grouped by their end j; tg_reuse.cu).
+int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStream_t s, tg_units &un);
+
 // Whole-graph enumerations and the per-edge pass of the cycles kernel
 // (tg_cycles.cu).  Per-edge mode: c4e holds M x L x L and k4e M x L(L+1)/2
 // zeroed counters (g4 = NULL).  Global mode (c4e / k4e = NULL): g4 gets, by

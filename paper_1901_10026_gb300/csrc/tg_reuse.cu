@@ -925,50 +925,6 @@ int timing_begin(cudaStream_t s, unsigned long long **work) {
     return TG_OK;
 }
 
-// Work units of the grouped order (see k_unit_flags), split by class.
-int edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStream_t s,
-               tg_units &un) {
-    DevBuf<uint32_t> flag, pos, gs, ge;
-    DevBuf<int64_t> cost, cum;
-    if (!flag.alloc(cnt, s) || !pos.alloc(cnt, s) || !gs.alloc(g->n, s) || !ge.alloc(g->n, s) ||
-        !cost.alloc(cnt + 1, s) || !cum.alloc(cnt + 1, s))
-        return TG_ENOMEM;
-    k_group_bounds<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, g->rowptr, cnt, gs.p, ge.p, cost.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY(tg_scan_i64(cost.p, cum.p, cnt + 1, s));
-    k_unit_flags<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, cnt, gs.p, ge.p, cum.p, flag.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY(tg_scan_u32(flag.p, pos.p, cnt, s));
-    uint32_t lastp = 0, lastf = 0;
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastp, pos.p + cnt - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastf, flag.p + cnt - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaStreamSynchronize(s));
-    un.nunits = lastp + lastf;
-    if (!un.ustart.alloc((size_t)un.nunits + 1, s)) return TG_ENOMEM;
-    k_unit_starts<<<grid_r(cnt), 256, 0, s>>>(flag.p, pos.p, cnt, un.ustart.p, un.nunits); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    // classes: light (one warp each) and heavy (one CTA each)
-    DevBuf<uint32_t> cflag, cpos;
-    if (!cflag.alloc(un.nunits, s) || !cpos.alloc(un.nunits, s) ||
-        !un.light.alloc(un.nunits, s) || !un.heavy.alloc(un.nunits, s))
-        return TG_ENOMEM;
-    k_unit_class<<<grid_r(un.nunits), 256, 0, s>>>(ord, g->edges, g->rowptr, un.ustart.p, un.nunits,
-                                                   cflag.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY(tg_scan_u32(cflag.p, cpos.p, un.nunits, s));
-    k_unit_lists<<<grid_r(un.nunits), 256, 0, s>>>(cflag.p, cpos.p, un.nunits, un.light.p,
-                                                   un.heavy.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastp, cpos.p + un.nunits - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastf, cflag.p + un.nunits - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaStreamSynchronize(s));
-    un.nlight = lastp + lastf;
-    un.nheavy = un.nunits - un.nlight;
-    return TG_OK;
-}
-
-
-
 // Theta and D of every node (see k_node_aggr)
 template <bool kLow>
 int node_sums(const tg_graph *g, const uint32_t *tau, uint32_t *theta, uint32_t *dsum,
@@ -1023,6 +979,48 @@ int launch_reuse_u(const ReuseParams &p, int threads, size_t smem, int grid_limi
 
 }  // namespace
 
+// Work units of the grouped order (see k_unit_flags), split by class.
+int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStream_t s,
+               tg_units &un) {
+    DevBuf<uint32_t> flag, pos, gs, ge;
+    DevBuf<int64_t> cost, cum;
+    if (!flag.alloc(cnt, s) || !pos.alloc(cnt, s) || !gs.alloc(g->n, s) || !ge.alloc(g->n, s) ||
+        !cost.alloc(cnt + 1, s) || !cum.alloc(cnt + 1, s))
+        return TG_ENOMEM;
+    k_group_bounds<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, g->rowptr, cnt, gs.p, ge.p, cost.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    TG_TRY(tg_scan_i64(cost.p, cum.p, cnt + 1, s));
+    k_unit_flags<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, cnt, gs.p, ge.p, cum.p, flag.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    TG_TRY(tg_scan_u32(flag.p, pos.p, cnt, s));
+    uint32_t lastp = 0, lastf = 0;
+    TG_TRY_CUDA(cudaMemcpyAsync(&lastp, pos.p + cnt - 1, 4, cudaMemcpyDeviceToHost, s));
+    TG_TRY_CUDA(cudaMemcpyAsync(&lastf, flag.p + cnt - 1, 4, cudaMemcpyDeviceToHost, s));
+    TG_TRY_CUDA(cudaStreamSynchronize(s));
+    un.nunits = lastp + lastf;
+    if (!un.ustart.alloc((size_t)un.nunits + 1, s)) return TG_ENOMEM;
+    k_unit_starts<<<grid_r(cnt), 256, 0, s>>>(flag.p, pos.p, cnt, un.ustart.p, un.nunits); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    // classes: light (one warp each) and heavy (one CTA each)
+    DevBuf<uint32_t> cflag, cpos;
+    if (!cflag.alloc(un.nunits, s) || !cpos.alloc(un.nunits, s) ||
+        !un.light.alloc(un.nunits, s) || !un.heavy.alloc(un.nunits, s))
+        return TG_ENOMEM;
+    k_unit_class<<<grid_r(un.nunits), 256, 0, s>>>(ord, g->edges, g->rowptr, un.ustart.p, un.nunits,
+                                                   cflag.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    TG_TRY(tg_scan_u32(cflag.p, cpos.p, un.nunits, s));
+    k_unit_lists<<<grid_r(un.nunits), 256, 0, s>>>(cflag.p, cpos.p, un.nunits, un.light.p,
+                                                   un.heavy.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    TG_TRY_CUDA(cudaMemcpyAsync(&lastp, cpos.p + un.nunits - 1, 4, cudaMemcpyDeviceToHost, s));
+    TG_TRY_CUDA(cudaMemcpyAsync(&lastf, cflag.p + un.nunits - 1, 4, cudaMemcpyDeviceToHost, s));
+    TG_TRY_CUDA(cudaStreamSynchronize(s));
+    un.nlight = lastp + lastf;
+    un.nheavy = un.nunits - un.nlight;
+    return TG_OK;
+}
+
 // Runs Alg. 1 for every edge (tau), the per-node sums, then the per-edge
 // counts for the edges order[0..count) (grouped by their high-degree end).
 int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_order,
@@ -1042,7 +1040,7 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
     {
         // tau of every edge, in the grouped order of the whole graph
         const uint32_t *ord = full_order;
-        TG_TRY(edge_units(g, ord, M, s, un));
+        TG_TRY(tg_edge_units(g, ord, M, s, un));
         DevBuf<unsigned long long> q;
         if (!q.alloc(2, s)) return TG_ENOMEM;
         TG_TRY_CUDA(cudaMemsetAsync(q.p, 0, 16, s));
@@ -1128,7 +1126,7 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
         tg_units un2;
         tg_units *ue = &un;
         if (order != full_order || count != M) {
-            if (count > 0) TG_TRY(edge_units(g, order, count, s, un2));
+            if (count > 0) TG_TRY(tg_edge_units(g, order, count, s, un2));
             ue = &un2;
         }
         // triangle counts per adjacency entry, for the per-edge pass's reads
