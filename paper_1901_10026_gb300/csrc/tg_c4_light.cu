@@ -137,11 +137,12 @@ __global__ void __launch_bounds__(kCostThreads) k_c4_classify(
 }
 
 __global__ void k_c4_heavy_info(const uint32_t *list, int64_t count, const int64_t *rowptr,
-                                const unsigned long long *cost, C4HeavyInfo *out) {
+                                const uint8_t *ntype, const unsigned long long *cost,
+                                C4HeavyInfo *out) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < count;
          q += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t a = list[q];
-        out[q] = C4HeavyInfo{cost[a], rowptr[a + 1] - rowptr[a], a, 0u};
+        out[q] = C4HeavyInfo{cost[a], rowptr[a + 1] - rowptr[a], a, ntype[a]};
     }
 }
 
@@ -561,7 +562,7 @@ int tg_c4_heavy(const tg_graph *g, const C4Lists &cls, C4HeavyInfo *host, cudaSt
     DevBuf<C4HeavyInfo> info;
     if (!info.alloc(count, s)) return TG_ENOMEM;
     k_c4_heavy_info<<<(unsigned)std::min<int64_t>((count + 255) / 256, 4096), 256, 0, s>>>(
-        cls.list.p + (int64_t)kC4Split * cls.n, count, g->rowptr, cls.cost.p, info.p);
+        cls.list.p + (int64_t)kC4Split * cls.n, count, g->rowptr, g->ntype, cls.cost.p, info.p);
     tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     TG_TRY_CUDA(cudaMemcpyAsync(host, info.p, count * sizeof(C4HeavyInfo), cudaMemcpyDeviceToHost, s));

@@ -864,131 +864,177 @@ __device__ __forceinline__ void k4_hist_add(unsigned long long *h4, int a, int b
 
 // ------------------------------------------------- binned waves (global) --
 // Anchors whose walk is long against the number of far-end windows it spans
-// (hubs): the counters stay on chip.  Every wedge a-u-b of a wave's walks
-// becomes the 16-bit entry (b mod 2^wlg) | (type of u) << wlg in the bucket of
-// (anchor, b >> wlg).  A count pass sizes the buckets and a fill pass writes
-// them, each with one counter add per distinct bucket among a warp's 32
-// wedges (a member's list is sorted by (type, id), so neighbouring wedges
-// mostly share a window; a run of equal buckets among consecutive lanes takes
-// its slots with one add).  k_c4_bin_pairs then gives each bucket to a CTA,
-// which counts its entries by (b, t) in a dense shared-memory table of the
-// window's 2^wlg far ends and adds each far end's cycle pairs to the
-// type-multiset histogram (c4_add).  DRAM sees the walk twice and 2 bytes
-// per wedge written and read once, instead of a counter read and write per
-// wedge.
+// (hubs): the counters stay on chip.  Far ends are numbered type by type, in
+// id order inside a type, each type padded to whole windows of 2^wlg, so a window
+// holds far ends of one type and a list sorted by (type, id) runs through the
+// windows in order.  Every wedge a-u-b of a wave's walks becomes the 16-bit entry
+// (b mod 2^wlg) << tlg | type of u in the bucket of (anchor, window).  A count
+// pass sizes the buckets and a fill pass writes them, each with one counter add
+// per run of consecutive lanes in one bucket.  k_c4_bin_gram then counts each
+// bucket's entries by (b, t) in a dense shared-memory table of the window's far
+// ends and sums c_t c_t' over the far ends in registers, for runs of anchors of
+// one type in one window, whose sums all go to the multisets {ta, tb, t, t'}.
+// DRAM sees the walk twice and 2 bytes per wedge written and read once, instead
+// of a counter read and write per wedge.
+//
+// With windows over the node ids (types mixed) a far end's pairs went, one 64-bit
+// shared add each, to a table by (type of b, pair).  4-cycle phase, before -> now:
+// R-MAT-21 (1.43e10 wedges, L = 8) 316 -> 184 ms, CL-1M (9.1e8, L = 5) 33.5 -> 20.9
+// ms, CL-100K (5.8e7) 4.1 -> 2.5 ms.
 struct C4Bin {
     const int64_t *rowptr;
     const uint32_t *adj;
-    const uint8_t *ntype;
-    int32_t L, wlg, half;
+    const uint32_t *badj;      // adjacency entries with the far-end number for the id
+    const uint32_t *thr;       // per binned anchor and type: far ends from here rank below it
+    int32_t L, wlg, tlg, half;
     const uint32_t *heavy;     // the binned anchors
+    const uint8_t *htype;      // their types
     const int64_t *mprefix;    // walk positions of their members (k_c4_prefix)
     const int64_t *pbase;
     const C4Unit *units;       // warp units of the wave
     int64_t n_units;
     int64_t q0;                // first anchor of the wave (bucket row = q - q0)
-    int64_t n;                 // nodes
-    int64_t W;                 // far-end windows, ceil(n / 2^wlg)
+    int64_t W;                 // far-end windows
+    uint32_t tbase[TG_MAX_TYPES + 1];  // first far-end number of each type (whole windows)
     uint32_t *cnt;             // K W bucket sizes (count pass), write cursors (fill pass)
     uint16_t *bins;            // the wave's entries, bucket after bucket
     const uint32_t *offs;      // K W + 1 bucket offsets
-    int64_t nb;                // buckets of the wave, K W
+    const int2 *runs;          // anchors [x, y) of one type, at most kBinRun
+    int64_t nitems;            // runs x windows
     unsigned long long *queue;
     unsigned long long *g4;
     int64_t n4;
     unsigned long long *work;  // [4]: wedges
 };
 
-constexpr int kBinUnroll = 2;
-constexpr int kBinFill = 32;            // default: binned when a walk averages this many wedges per window
-constexpr size_t kBinTable = 64 * 1024;  // bytes of the dense far-end table
+// Numbering of the far ends: nodes [0, n) (the non-isolated ones) in blocks of
+// kRankBlock; per type the blocks' counts (cnt[t nblk + block], then scanned).
+constexpr int kRankBlock = 1024;
 
-// One chunk of 32 members (lane values len, bu, tu) of a binned walk unit; as
-// c4_chunk_count, with kBinUnroll batches of 32 positions per step.  Count pass:
-// adds each batch's wedges to their buckets' sizes.  Fill pass: takes a run
-// of slots from each bucket's cursor and writes the entries.
-template <bool kFill, class IT>
-__device__ __forceinline__ int64_t c4_chunk_bin(const C4Bin &p, uint32_t a, uint32_t *cb,
-                                                int64_t len64, int64_t bu, int tu, int64_t at,
-                                                int64_t f_lo, int64_t f_hi,
-                                                unsigned long long &wk) {
-    const int lane = threadIdx.x & 31;
-    const IT len = (IT)len64;
-    IT incl = len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const IT y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
+__global__ void __launch_bounds__(kRankBlock) k_bin_hist(const uint8_t *ntype, int64_t n, int64_t nblk,
+                                                         int L, uint32_t *cnt) {
+    __shared__ uint32_t c[TG_MAX_TYPES];
+    if (threadIdx.x < TG_MAX_TYPES) c[threadIdx.x] = 0u;
+    __syncthreads();
+    const int64_t v = blockIdx.x * (int64_t)kRankBlock + threadIdx.x;
+    const int t = v < n ? (int)ntype[v] : -1;
+    for (int k = 0; k < L; ++k) {
+        const unsigned m = __ballot_sync(kFull, t == k);
+        if ((threadIdx.x & 31) == 0 && m) atomicAdd(&c[k], (uint32_t)__popc(m));
     }
-    const IT total = __shfl_sync(kFull, incl, 31);
-    const IT lo = (IT)(f_lo > at ? (f_lo - at < (int64_t)total ? f_lo - at : (int64_t)total) : 0);
-    const IT hi = (IT)(f_hi - at < (int64_t)total ? f_hi - at : (int64_t)total);
-    const uint32_t wmask = (1u << p.wlg) - 1u;
-    for (IT b0 = lo; b0 < hi; b0 += 32 * kBinUnroll) {
-        uint32_t bv[kBinUnroll], base[kBinUnroll];
-        int tv[kBinUnroll];
-        bool ok[kBinUnroll];
-#pragma unroll
-        for (int q = 0; q < kBinUnroll; ++q) {
-            const IT pos = b0 + 32 * q + lane;
-            int r = 0;  // the first member whose running sum exceeds pos
-#pragma unroll
-            for (int st = 16; st > 0; st >>= 1) {
-                const IT v = __shfl_sync(kFull, incl, r + st - 1);
-                if (v <= pos) r += st;
-            }
-            const int64_t bur = __shfl_sync(kFull, bu, r);
-            const IT str = __shfl_sync(kFull, incl - len, r);
-            const int tur = __shfl_sync(kFull, tu, r);
-            ok[q] = false;
-            bv[q] = 0;
-            tv[q] = 0;
-            if (pos < hi) {
-                const uint32_t b = __ldg(p.adj + bur + (int64_t)(pos - str)) & TG_IDMASK;
-                if (b > a) {
-                    ok[q] = true;
-                    bv[q] = b;
-                    tv[q] = tur;
-                }
-            }
-        }
-        // runs of equal buckets among consecutive lanes (a member's list is
-        // sorted by (type, id), so consecutive wedges mostly share a window):
-        // the first lane of a run takes the run's slots with one add
-        int rs[kBinUnroll];
-#pragma unroll
-        for (int q = 0; q < kBinUnroll; ++q) {
-            const int key = ok[q] ? (int)(bv[q] >> p.wlg) : -1;
-            const int prev = __shfl_up_sync(kFull, key, 1);
-            const unsigned heads = __ballot_sync(kFull, lane == 0 || key != prev);
-            const unsigned upto = heads & ((2u << lane) - 1u);  // heads at or below this lane
-            rs[q] = 31 - __clz(upto);
-            const unsigned above = heads & ~((2u << lane) - 1u);
-            const int re = above ? __ffs(above) - 1 : 32;
-            base[q] = 0u;
-            if (key >= 0 && rs[q] == lane) {
-                if (kFill)
-                    base[q] = atomicAdd(cb + key, (uint32_t)(re - lane));
-                else
-                    atomicAdd(cb + key, (uint32_t)(re - lane));
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < kBinUnroll; ++q) {
-            if (kFill) {
-                const uint32_t bb = __shfl_sync(kFull, base[q], rs[q]);
-                if (ok[q])
-                    p.bins[bb + (uint32_t)(lane - rs[q])] =
-                        (uint16_t)((bv[q] & wmask) | ((uint32_t)tv[q] << p.wlg));
-            } else if (ok[q]) {
-                ++wk;
-            }
-        }
-    }
-    return (int64_t)total;
+    __syncthreads();
+    if (threadIdx.x < L) cnt[threadIdx.x * nblk + blockIdx.x] = c[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0) cnt[L * nblk] = 0u;
 }
 
-// The count (kFill = false) or fill pass of a binned wave: one warp per unit.
+// base[t]: first far-end number of type t, padded to multiples of 2^lg; one warp
+__global__ void k_bin_bases(const uint32_t *scan, int64_t nblk, int L, int lg, uint32_t *base) {
+    if (threadIdx.x != 0) return;
+    uint32_t at = 0;
+    for (int t = 0; t < L; ++t) {
+        base[t] = at;
+        const uint32_t c = scan[(t + 1) * nblk] - scan[t * nblk];
+        at += ((c + (1u << lg) - 1u) >> lg) << lg;
+    }
+    base[L] = at;
+}
+
+__global__ void __launch_bounds__(kRankBlock) k_bin_numbers(const uint8_t *ntype, int64_t n, int64_t nblk,
+                                                            int L, const uint32_t *scan,
+                                                            const uint32_t *base, uint32_t *num) {
+    __shared__ uint32_t c[kRankBlock / 32][TG_MAX_TYPES];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t v = blockIdx.x * (int64_t)kRankBlock + threadIdx.x;
+    const int t = v < n ? (int)ntype[v] : -1;
+    uint32_t rank = 0;
+    for (int k = 0; k < L; ++k) {
+        const unsigned m = __ballot_sync(kFull, t == k);
+        if (t == k) rank = (uint32_t)__popc(m & ((1u << lane) - 1u));
+        if (lane == 0) c[warp][k] = (uint32_t)__popc(m);
+    }
+    __syncthreads();
+    if (t < 0) return;
+    for (int w = 0; w < warp; ++w) rank += c[w][t];
+    num[v] = base[t] + (scan[t * nblk + blockIdx.x] - scan[t * nblk]) + rank;
+}
+
+__global__ void k_bin_entries(const uint32_t *adj, int64_t entries, const uint32_t *num, uint32_t *badj) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < entries;
+         x += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t w = __ldg(adj + x);
+        badj[x] = (w & ~TG_IDMASK) | __ldg(num + (w & TG_IDMASK));
+    }
+}
+
+// thr[q L + t]: base[t] plus the nodes of type t with ids up to anchor q's; one
+// warp per anchor.
+__global__ void k_bin_thresholds(const uint32_t *heavy, int64_t na, const uint8_t *ntype, int64_t nblk,
+                                 int L, const uint32_t *scan, const uint32_t *base, uint32_t *thr,
+                                 uint8_t *htype) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < na; q += nw) {
+        const int64_t a = heavy[q], blk = a / kRankBlock;
+        uint32_t c = lane < L ? base[lane] + (scan[lane * nblk + blk] - scan[lane * nblk]) : 0u;
+        for (int64_t v0 = blk * kRankBlock; v0 <= a; v0 += 32) {
+            const int t = v0 + lane <= a ? (int)ntype[v0 + lane] : -1;
+            for (int k = 0; k < L; ++k) {
+                const unsigned m = __ballot_sync(kFull, t == k);
+                if (lane == k) c += (uint32_t)__popc(m);
+            }
+        }
+        if (lane < L) thr[q * L + lane] = c;
+        if (lane == 0) htype[q] = ntype[a];
+    }
+}
+
+constexpr int kBinUnroll = 4;              // batches of 32 positions in flight
+constexpr int kBinFill = 32;            // default: binned when a walk averages this many wedges per window
+constexpr size_t kBinTable = 64 * 1024;  // bytes of the dense far-end table
+constexpr int kBinRun = 16;              // anchors of one type taken together, at most
+
+// 32 consecutive positions of a walk, one per lane (entry w of a list in far-end
+// numbers; in: the position belongs to the unit; tu: the type of its member): the
+// entries ranked below the anchor (from their type's threshold on; lane t holds
+// type t's) go to their buckets cb[window].  Runs of one bucket among consecutive
+// lanes take their places with one add; the fill pass writes the entries.
+template <bool kFill>
+__device__ __forceinline__ void bin_put(const C4Bin &p, uint32_t *cb, uint32_t thr, uint32_t w, bool in,
+                                        int tu, unsigned long long &wk) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t from = __shfl_sync(kFull, thr, (int)(w >> TG_TSHIFT));
+    const uint32_t b = w & TG_IDMASK;
+    const bool ok = in && b >= from;
+    const int key = ok ? (int)(b >> p.wlg) : -1;
+    const int prev = __shfl_up_sync(kFull, key, 1);
+    const bool head = lane == 0 || key != prev;
+    const unsigned heads = __ballot_sync(kFull, head);
+    const unsigned upto = (2u << lane) - 1u;
+    uint32_t base = 0;
+    if (head && ok) {
+        const unsigned above = heads & ~upto;
+        const uint32_t len = (uint32_t)((above ? __ffs(above) - 1 : 32) - lane);
+        if (kFill)
+            base = atomicAdd(cb + key, len);
+        else
+            atomicAdd(cb + key, len);
+        if (!kFill) wk += len;
+    }
+    if (kFill) {
+        const int rs = 31 - __clz(heads & upto);  // the run's first lane
+        base = __shfl_sync(kFull, base, rs);
+        if (ok)
+            p.bins[base + (uint32_t)(lane - rs)] =
+                (uint16_t)(((b & ((1u << p.wlg) - 1u)) << p.tlg) | (uint32_t)tu);
+    }
+}
+
+// The count (kFill = false) or fill pass of a binned wave: one warp per unit.  A
+// member's list of kBinLong entries or more is taken by the whole warp, kBinUnroll
+// batches of 32 in flight, without the search that maps positions to members;
+// shorter lists are taken as one sequence by the unit in which they begin.
+constexpr int kBinLong = 64;
+
 template <bool kFill>
 __global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_bin_walk(C4Bin p) {
     const int lane = threadIdx.x & 31;
@@ -1003,11 +1049,12 @@ __global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_bin_walk(C4Bin p) {
         const int64_t ba = p.rowptr[a];
         const int da = (int)(p.rowptr[a + 1] - ba);
         uint32_t *cb = p.cnt + (un.q - p.q0) * p.W;
+        const uint32_t thr = lane < p.L ? p.thr[(int64_t)un.q * p.L + lane] : 0u;
         int64_t at = p.mprefix[p.pbase[un.q] + un.m];
         for (int m = un.m; m < da && at < un.hi; m += 32) {
             const int x = m + lane;
-            int64_t len = 0, bu = 0;
-            int tu = 0;
+            int64_t bu = 0;
+            int len = 0, tu = 0;
             if (x < da) {
                 const uint32_t wu = __ldg(p.adj + ba + x);
                 const uint32_t u = wu & TG_IDMASK;
@@ -1015,15 +1062,64 @@ __global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_bin_walk(C4Bin p) {
                     bu = p.rowptr[u];
                     const int64_t du = p.rowptr[u + 1] - bu;
                     if (du > 1) {
-                        len = du;
+                        len = (int)du;
                         tu = (int)(wu >> TG_TSHIFT);
                     }
                 }
             }
-            if (__all_sync(kFull, len < ((int64_t)1 << 26)))
-                at += c4_chunk_bin<kFill, int>(p, a, cb, len, bu, tu, at, un.lo, un.hi, wk);
-            else
-                at += c4_chunk_bin<kFill, int64_t>(p, a, cb, len, bu, tu, at, un.lo, un.hi, wk);
+            int64_t incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int64_t first = at + incl - len;  // walk position of this member's list
+            at += __shfl_sync(kFull, incl, 31);
+            // long lists, the part [q0, q1) inside the unit
+            const int64_t q0 = un.lo > first ? un.lo - first : 0;
+            const int64_t q1 = un.hi - first < len ? un.hi - first : len;
+            for (unsigned todo = __ballot_sync(kFull, len >= kBinLong && q0 < q1); todo; todo &= todo - 1u) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t *list = p.badj + __shfl_sync(kFull, bu + q0, src);
+                const int cnt = (int)__shfl_sync(kFull, q1 - q0, src), t = __shfl_sync(kFull, tu, src);
+                for (int c = lane; c - lane < cnt; c += 32 * kBinUnroll) {
+                    uint32_t w[kBinUnroll];
+#pragma unroll
+                    for (int z = 0; z < kBinUnroll; ++z) w[z] = c + 32 * z < cnt ? __ldg(list + c + 32 * z) : 0u;
+#pragma unroll
+                    for (int z = 0; z < kBinUnroll; ++z) bin_put<kFill>(p, cb, thr, w[z], c + 32 * z < cnt, t, wk);
+                }
+            }
+            // short lists that begin inside the unit
+            const int ls = len < kBinLong && first >= un.lo && first < un.hi ? len : 0;
+            int si = ls;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(kFull, si, o);
+                if (lane >= o) si += y;
+            }
+            const int total = __shfl_sync(kFull, si, 31);
+            const int64_t org = bu - (si - ls);
+            for (int c = 0; c < total; c += 32 * kBinUnroll) {
+                uint32_t w[kBinUnroll];
+                int t[kBinUnroll];
+#pragma unroll
+                for (int z = 0; z < kBinUnroll; ++z) {
+                    const int pos = c + 32 * z + lane;
+                    int r = 0;  // the member whose list holds pos
+#pragma unroll
+                    for (int st = 16; st > 0; st >>= 1) {
+                        const int v = __shfl_sync(kFull, si, r + st - 1);
+                        if (v <= pos) r += st;
+                    }
+                    const int64_t e = __shfl_sync(kFull, org, r) + pos;
+                    t[z] = __shfl_sync(kFull, tu, r);
+                    w[z] = pos < total ? __ldg(p.badj + e) : 0u;
+                }
+#pragma unroll
+                for (int z = 0; z < kBinUnroll; ++z)
+                    bin_put<kFill>(p, cb, thr, w[z], c + 32 * z + lane < total, t[z], wk);
+            }
         }
     }
     if (!kFill && p.work) {
@@ -1033,148 +1129,308 @@ __global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_bin_walk(C4Bin p) {
     }
 }
 
-// The buckets of a binned wave.  A CTA takes runs of kBinRun consecutive
-// buckets (consecutive windows of one anchor, mostly) from a queue.  A bucket
-// (anchor a of type ta, window w) has its entries counted by (b, t) in the
-// dense table (16-bit halves when the wave's anchors have fewer than 2^16
-// neighbours, else 32-bit counts); the first entry of a far end puts it on a
-// list (a bit per far end keeps it there once).  Then one thread per listed
-// far end reads its counts, clears them, and for the types it has (usually
-// few) adds C(c_t, 2) and c_t c_t' to the CTA's table acc[type of b][pair]
-// in shared memory (atomic adds), which goes into the histogram under
-// {ta, tb, t, t'} when the anchor changes.  1024-thread CTAs, two per SM.  Types beyond kBinAccL use c4_add
-// straight into a shared histogram instead.
-constexpr int kBinPairThreads = 1024;
-constexpr int kBinRun = 16;
-constexpr int kBinAccL = 8;
+// Counts of a far-end row of k_c4_bin_gram (a power of two from L on; L <= 8), 0
+// for more types (k_c4_bin_pairs).
+__host__ __device__ constexpr int bin_lanes(int L) { return L <= 2 ? 2 : L <= 4 ? 4 : L <= 8 ? 8 : 0; }
 
-__device__ __forceinline__ void bin_flush(unsigned long long *acc, unsigned long long *h4, int L,
-                                          int P, int ta) {
-    for (int k = threadIdx.x; k < L * P; k += blockDim.x) {
-        const unsigned long long v = acc[k];
-        if (!v) continue;
-        acc[k] = 0ull;
-        int t, u;
-        unpair(L, k % P, t, u);
-        k4_hist_add(h4, ta, k / P, t, u, v);
-    }
+// Type of window w.
+__device__ __forceinline__ int bin_type(const C4Bin &p, int64_t w) {
+    int t = 0;
+    while (t + 1 < p.L && (int64_t)(p.tbase[t + 1] >> p.wlg) <= w) ++t;
+    return t;
 }
 
-__global__ void __launch_bounds__(kBinPairThreads) k_c4_bin_pairs(C4Bin p) {
+constexpr int kGramThreads = 512;
+
+__device__ __forceinline__ void ldsm_t4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// d += x^T y over 16 far ends: x0, y0 hold the counts of far ends 0..7 in the
+// transposed ldmatrix layout (lane: type lane / 4, far ends 2 (lane % 4) and the
+// next), x1, y1 those of far ends 8..15; d: types (lane / 4, 2 (lane % 4) and the
+// next).  A's other eight rows are zero.
+__device__ __forceinline__ void gram16(float (&d)[2], uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1) {
+    float z0 = 0.f, z1 = 0.f;
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(z0), "+f"(z1)
+        : "r"(x0), "r"(0u), "r"(x1), "r"(0u), "r"(y0), "r"(y1));
+}
+
+// Two counts below 1024 in 16-bit halves as two fp16 values: 0x6400 is 1024 and
+// its last place 1.
+__device__ __forceinline__ uint32_t counts_f16(uint32_t x) {
+    uint32_t r;
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x | 0x64006400u), "r"(0x64006400u));
+    return r;
+}
+
+// Buckets of a binned wave, L <= 8 types.  A CTA takes an item (anchors of one
+// type, one window): bucket after bucket it counts the entries in the table (a row
+// of counts per far end), then sums c_t c_t' over the far ends and clears it.  With
+// eight 16-bit counts a row (5 to 8 types) the sums are X^T X of the table X on the
+// tensor cores: a row is a row of an 8 x 8 matrix of 16-bit values, so one ldmatrix
+// gives 32 far ends in the layout of both operands, and counts up to 255 are exact
+// as fp16, their sums over 128 far ends (two of them in the cross terms) below 2^24
+// in fp32, which are then added to 64-bit sums.  Where a count is larger its high and low bytes take the place of
+// it: 65536 H^T H + 256 (H^T L + L^T H) + L^T L.  The other row widths sum the rows
+// with two middles or more in groups of G lanes, lane a holding sum c_a c_b for every
+// b.  No add to shared memory is made until the item's end.
+template <int G, bool kHalf>
+__global__ void __launch_bounds__(kGramThreads, 2) k_c4_bin_gram(C4Bin p) {
+    constexpr int RW = kHalf ? G / 2 : G;  // words of a row
+    constexpr bool kMma = kHalf && G == 8;
+    constexpr int kSums = kMma ? 2 : G;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int tid = threadIdx.x;
-    const int L = p.L, Lp = L + (L & 1), P = L * (L + 1) / 2;
-    const bool acc_mode = L <= kBinAccL;
+    __shared__ unsigned long long s_item;
+    __shared__ uint32_t s_off[2 * kBinRun];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nfar = 1 << p.wlg;
-    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem);
-    size_t off = ((size_t)p.n4 * 8 + 15) & ~(size_t)15;
-    unsigned long long *acc = reinterpret_cast<unsigned long long *>(smem + off);  // one per CTA
-    if (acc_mode) off += ((size_t)L * P * 8 + 15) & ~(size_t)15;
-    uint32_t *tab = reinterpret_cast<uint32_t *>(smem + off);
-    const int twords = p.half ? nfar * (Lp >> 1) : nfar * L;
-    uint32_t *tbits = tab + twords;                                      // nfar / 32 words
-    uint16_t *flist = reinterpret_cast<uint16_t *>(tbits + nfar / 32);  // touched far ends
-    const volatile uint32_t *vtab = tab;
-    __shared__ unsigned long long s_run;
-    __shared__ uint32_t s_nl;
-    for (int64_t q = tid; q < p.n4; q += blockDim.x) h4[q] = 0ull;
-    if (acc_mode)
-        for (int q = tid; q < L * P; q += blockDim.x) acc[q] = 0ull;
-    for (int q = tid; q < twords + nfar / 32; q += blockDim.x) tab[q] = 0u;
-    if (tid == 0) s_nl = 0u;
-    const uint32_t wmask = (uint32_t)nfar - 1u;
-    int cur_ta = -1;
-    int64_t cur_row = -1;
+    uint32_t *tab = reinterpret_cast<uint32_t *>(smem);
+    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem + (size_t)nfar * RW * 4);
+    for (int q = tid; q < nfar * RW; q += kGramThreads) tab[q] = 0u;
+    for (int64_t q = tid; q < p.n4; q += kGramThreads) h4[q] = 0ull;
+    // this lane's type and its group (or first column)
+    const int ga = kMma ? lane / 4 : lane % G, gg = kMma ? lane % 4 : lane / G;
     for (;;) {
         __syncthreads();
-        if (tid == 0) s_run = atomicAdd(p.queue, (unsigned long long)kBinRun);
+        if (tid == 0) s_item = atomicAdd(p.queue, 1ull);
         __syncthreads();
-        const int64_t r0 = (int64_t)s_run;
-        if (r0 >= p.nb) break;
-        const int64_t r1 = r0 + kBinRun < p.nb ? r0 + kBinRun : p.nb;
-        for (int64_t item = r0; item < r1; ++item) {
-            const uint32_t c0 = p.offs[item], c1 = p.offs[item + 1];
-            if (c0 == c1) continue;  // uniform across the CTA
-            const int64_t row = item / p.W;
-            const int64_t wbase = (item % p.W) << p.wlg;
-            if (row != cur_row) {
-                if (acc_mode && cur_ta >= 0) bin_flush(acc, h4, L, P, cur_ta);
-                cur_row = row;
-                cur_ta = p.ntype[p.heavy[p.q0 + row]];
+        if (s_item >= (unsigned long long)p.nitems) break;
+        const int64_t w = (int64_t)s_item % p.W;
+        const int2 run = p.runs[(int64_t)s_item / p.W];
+        const int nr = run.y - run.x;
+        if (tid < nr) {
+            const int64_t b = (run.x + tid - p.q0) * p.W + w;
+            s_off[2 * tid] = p.offs[b];
+            s_off[2 * tid + 1] = p.offs[b + 1];
+        }
+        __syncthreads();
+        unsigned long long acc[kSums], one = 0;
+#pragma unroll
+        for (int b = 0; b < kSums; ++b) acc[b] = 0ull;
+        // four entries at 8-byte boundaries; those outside the bucket are left out
+        auto fetch = [&](uint32_t k, uint32_t c1) -> uint2 {
+            return k < c1 ? *reinterpret_cast<const uint2 *>(p.bins + k) : make_uint2(0u, 0u);
+        };
+        auto count = [&](uint2 e, uint32_t k, uint32_t c0, uint32_t c1) {
+            if (k >= c1) return;
+            const bool whole = k >= c0 && k + 4 <= c1;
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+                const uint32_t x = ((z < 2 ? e.x : e.y) >> (16 * (z & 1))) & 0xffffu;
+                if (!whole && (k + z < c0 || k + z >= c1)) continue;
+                if (kHalf)
+                    atomicAdd(tab + (x >> 1), 1u << (16 * (x & 1u)));
+                else
+                    atomicAdd(tab + x, 1u);
             }
-            const int ta = cur_ta;
-            // count the entries by (far end, type); a far end's first entry
-            // puts it on the list
-            for (uint32_t k0 = c0 + tid; k0 < c1; k0 += 4 * blockDim.x) {
-                uint32_t ev[4];
+        };
+        uint32_t k0 = (s_off[0] & ~3u) + 4u * tid;
+        uint2 ahead = fetch(k0, s_off[1]);
+        for (int r = 0; r < nr; ++r) {
+            const uint32_t c0 = s_off[2 * r], c1 = s_off[2 * r + 1];
+            for (uint32_t k = k0; k < c1; k += 4 * kGramThreads) {
+                const uint2 e = ahead;
+                ahead = fetch(k + 4 * kGramThreads, c1);
+                count(e, k, c0, c1);
+            }
+            if (r + 1 < nr) {  // the next bucket's first entries, before the rows are taken
+                k0 = (s_off[2 * r + 2] & ~3u) + 4u * tid;
+                ahead = fetch(k0, s_off[2 * r + 3]);
+            }
+            if (c0 == c1) continue;  // uniform across the CTA
+            __syncthreads();
+            if (kMma) {
+                // a warp takes 128 rows at a time
+                for (int r0 = 128 * warp; r0 < nfar; r0 += 128 * (kGramThreads / 32)) {
+                    uint32_t x[4][4], big = 0;
+                    const uint32_t base = (uint32_t)__cvta_generic_to_shared(tab + (r0 + lane) * RW);
 #pragma unroll
-                for (int z = 0; z < 4; ++z) {
-                    const uint32_t k = k0 + (uint32_t)z * blockDim.x;
-                    ev[z] = k < c1 ? (uint32_t)p.bins[k] : 0xffffffffu;
-                }
-#pragma unroll
-                for (int z = 0; z < 4; ++z) {
-                    if (ev[z] == 0xffffffffu) continue;
-                    const uint32_t bl = ev[z] & wmask;
-                    const int t = (int)(ev[z] >> p.wlg);
-                    bool first;
-                    if (p.half) {
-                        const uint32_t idx = bl * (uint32_t)Lp + (uint32_t)t;
-                        const int sh = (int)(idx & 1u) * 16;
-                        const uint32_t old = atomicAdd(tab + (idx >> 1), 1u << sh);
-                        first = ((old >> sh) & 0xffffu) == 0u;
-                    } else {
-                        first = atomicAdd(tab + bl * (uint32_t)L + (uint32_t)t, 1u) == 0u;
+                    for (int z = 0; z < 4; ++z) {
+                        ldsm_t4(base + z * 32 * RW * 4, x[z]);
+                        big |= x[z][0] | x[z][1] | x[z][2] | x[z][3];
                     }
-                    if (first) {
-                        const uint32_t bit = 1u << (bl & 31u);
-                        if (!(atomicOr(tbits + (bl >> 5), bit) & bit)) flist[atomicAdd(&s_nl, 1u)] = (uint16_t)bl;
+                    big = __reduce_or_sync(kFull, big);
+                    if (big == 0u) continue;
+                    uint4 *row = reinterpret_cast<uint4 *>(tab) + r0 + lane;
+#pragma unroll
+                    for (int z = 0; z < 4; ++z) row[32 * z] = make_uint4(0u, 0u, 0u, 0u);
+                    const uint32_t ones = 0x3c003c00u;  // 1.0, 1.0
+                    float ll[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
+                    if (!(big & 0xff00ff00u)) {
+#pragma unroll
+                        for (int z = 0; z < 4; ++z)
+#pragma unroll
+                            for (int h = 0; h < 4; h += 2) {
+                                const uint32_t l0 = counts_f16(x[z][h]), l1 = counts_f16(x[z][h + 1]);
+                                gram16(ll, l0, l1, l0, l1);
+                                gram16(s1, l0, l1, ones, ones);
+                            }
+                    } else {
+                        float lh[2] = {0.f, 0.f}, hh[2] = {0.f, 0.f}, sh[2] = {0.f, 0.f};
+#pragma unroll
+                        for (int z = 0; z < 4; ++z)
+#pragma unroll
+                            for (int h = 0; h < 4; h += 2) {
+                                const uint32_t l0 = counts_f16(x[z][h] & 0x00ff00ffu);
+                                const uint32_t l1 = counts_f16(x[z][h + 1] & 0x00ff00ffu);
+                                const uint32_t h0 = counts_f16((x[z][h] >> 8) & 0x00ff00ffu);
+                                const uint32_t h1 = counts_f16((x[z][h + 1] >> 8) & 0x00ff00ffu);
+                                gram16(ll, l0, l1, l0, l1);
+                                gram16(lh, l0, l1, h0, h1);
+                                gram16(lh, h0, h1, l0, l1);
+                                gram16(hh, h0, h1, h0, h1);
+                                gram16(s1, l0, l1, ones, ones);
+                                gram16(sh, h0, h1, ones, ones);
+                            }
+#pragma unroll
+                        for (int b = 0; b < 2; ++b)
+                            acc[b % kSums] += 256ull * (uint32_t)lh[b] + 65536ull * (uint32_t)hh[b];
+                        one += 256ull * (uint32_t)sh[0];
+                    }
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) acc[b % kSums] += (uint32_t)ll[b];
+                    one += (uint32_t)s1[0];
+                }
+            } else {
+                for (int row = tid; row < nfar; row += kGramThreads) {
+                    uint32_t v[RW], any = 0, sum = 0;
+                    uint32_t *tr = tab + row * RW;
+#pragma unroll
+                    for (int z = 0; z < RW; ++z) {
+                        v[z] = tr[z];
+                        any |= v[z];
+                        sum += kHalf ? (v[z] & 0xffffu) + (v[z] >> 16) : v[z];
+                    }
+                    if (any) {
+#pragma unroll
+                        for (int z = 0; z < RW; ++z) tr[z] = 0u;
+                    }
+                    // one middle closes no cycle
+                    for (unsigned m = __ballot_sync(kFull, sum > 1u); m;) {
+                        unsigned mine = m;  // this group's row: the gg-th set bit
+#pragma unroll
+                        for (int z = 0; z < 32 / G; ++z) {
+                            if (z < gg) mine &= mine - 1u;
+                            m &= m - 1u;
+                        }
+                        const int src = mine ? __ffs(mine) - 1 : 0;
+                        uint32_t c[G], ca = 0;
+#pragma unroll
+                        for (int z = 0; z < RW; ++z) {
+                            const uint32_t y = __shfl_sync(kFull, v[z], src);
+                            if (kHalf) {
+                                c[2 * z] = y & 0xffffu;
+                                c[2 * z + 1] = y >> 16;
+                            } else {
+                                c[z] = y;
+                            }
+                        }
+#pragma unroll
+                        for (int b = 0; b < G; ++b)
+                            if (b == ga) ca = c[b];
+                        if (!mine) ca = 0u;
+                        one += ca;
+#pragma unroll
+                        for (int b = 0; b < kSums; ++b) acc[b] += (unsigned long long)ca * c[b];
                     }
                 }
             }
             __syncthreads();
-            // one far end per thread: its nonzero types, the pairs among them
+        }
+        // the item's sums over the groups of a warp, then into the histogram
+        if (!kMma) {
+#pragma unroll
+            for (int o = G; o < 32; o <<= 1) {
+                one += __shfl_xor_sync(kFull, one, o);
+#pragma unroll
+                for (int b = 0; b < kSums; ++b) acc[b] += __shfl_xor_sync(kFull, acc[b], o);
+            }
+        }
+        if ((kMma || gg == 0) && one) {
+            const int ta = p.htype[run.x], tb = bin_type(p, w);
+#pragma unroll
+            for (int b = 0; b < kSums; ++b) {
+                const int t = kMma ? 2 * gg + b : b;
+                if (t < ga) continue;
+                const unsigned long long x = t == ga ? (acc[b] - one) / 2 : acc[b];
+                if (x) k4_hist_add(h4, ta, tb, ga, t, x);
+            }
+        }
+    }
+    __syncthreads();
+    for (int64_t q = tid; q < p.n4; q += kGramThreads)
+        if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
+}
+
+// The same for more than 8 types: a far end's first entry puts it on a list; then
+// one thread per listed far end adds its pairs to a shared histogram (c4_add).
+constexpr int kBinPairThreads = 1024;
+
+__global__ void __launch_bounds__(kBinPairThreads) k_c4_bin_pairs(C4Bin p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int tid = threadIdx.x;
+    const int L = p.L, Lp = L + (L & 1);
+    const int nfar = 1 << p.wlg;
+    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(smem);
+    uint32_t *tab = reinterpret_cast<uint32_t *>(smem + (((size_t)p.n4 * 8 + 15) & ~(size_t)15));
+    const int twords = p.half ? nfar * (Lp >> 1) : nfar * L;
+    uint32_t *tbits = tab + twords;                                      // nfar / 32 words
+    uint16_t *flist = reinterpret_cast<uint16_t *>(tbits + nfar / 32);  // touched far ends
+    const volatile uint32_t *vtab = tab;
+    __shared__ unsigned long long s_item;
+    __shared__ uint32_t s_nl;
+    for (int64_t q = tid; q < p.n4; q += blockDim.x) h4[q] = 0ull;
+    for (int q = tid; q < twords + nfar / 32; q += blockDim.x) tab[q] = 0u;
+    if (tid == 0) s_nl = 0u;
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_item = atomicAdd(p.queue, 1ull);
+        __syncthreads();
+        if (s_item >= (unsigned long long)p.nitems) break;
+        const int64_t w = (int64_t)s_item % p.W;
+        const int2 run = p.runs[(int64_t)s_item / p.W];
+        const int ta = p.htype[run.x], tb = bin_type(p, w);
+        for (int r = run.x; r < run.y; ++r) {
+            const int64_t bucket = (r - p.q0) * p.W + w;
+            const uint32_t c0 = p.offs[bucket], c1 = p.offs[bucket + 1];
+            if (c0 == c1) continue;  // uniform across the CTA
+            for (uint32_t k = c0 + tid; k < c1; k += blockDim.x) {
+                const uint32_t ev = p.bins[k];
+                const uint32_t bl = ev >> p.tlg, t = ev & ((1u << p.tlg) - 1u);
+                bool first;
+                if (p.half) {
+                    const uint32_t idx = bl * (uint32_t)Lp + t;
+                    const int sh = (int)(idx & 1u) * 16;
+                    first = ((atomicAdd(tab + (idx >> 1), 1u << sh) >> sh) & 0xffffu) == 0u;
+                } else {
+                    first = atomicAdd(tab + bl * (uint32_t)L + t, 1u) == 0u;
+                }
+                if (first) {
+                    const uint32_t bit = 1u << (bl & 31u);
+                    if (!(atomicOr(tbits + (bl >> 5), bit) & bit)) flist[atomicAdd(&s_nl, 1u)] = (uint16_t)bl;
+                }
+            }
+            __syncthreads();
             const uint32_t nl = s_nl;
             for (uint32_t x = tid; x < nl; x += blockDim.x) {
                 const uint32_t bl = flist[x];
                 uint32_t c[TG_MAX_TYPES];
-                uint32_t sum = 0, mask = 0;
-                if (p.half) {
-                    const uint32_t w0 = bl * (uint32_t)(Lp >> 1);
-                    for (int q = 0; q < (Lp >> 1); ++q) {
-                        const uint32_t w = vtab[w0 + q];
-                        tab[w0 + q] = 0u;
-                        c[2 * q] = w & 0xffffu;
-                        if (2 * q + 1 < L) c[2 * q + 1] = w >> 16;
-                        sum += (w & 0xffffu) + (w >> 16);
-                        if (w & 0xffffu) mask |= 1u << (2 * q);
-                        if (w >> 16) mask |= 1u << (2 * q + 1);
-                    }
-                } else {
-                    for (int t = 0; t < L; ++t) {
-                        c[t] = vtab[bl * (uint32_t)L + t];
-                        tab[bl * (uint32_t)L + t] = 0u;
-                        sum += c[t];
-                        if (c[t]) mask |= 1u << t;
-                    }
+                uint32_t sum = 0;
+                for (int t = 0; t < L; ++t) {
+                    const uint32_t at = p.half ? (bl * (uint32_t)Lp + t) >> 1 : bl * (uint32_t)L + t;
+                    c[t] = p.half ? (vtab[at] >> (16 * (t & 1))) & 0xffffu : vtab[at];
+                    sum += c[t];
                 }
-                if (sum < 2) continue;
-                const int tb = (int)p.ntype[wbase + bl];
-                if (!acc_mode) {
-                    c4_add(h4, L, ta, tb, c);
-                    continue;
-                }
-                unsigned long long *ar = acc + (size_t)tb * P;
-                for (uint32_t mt = mask; mt; mt &= mt - 1u) {
-                    const int t = __ffs(mt) - 1;
-                    const unsigned long long ct = c[t];
-                    const int rowt = t * L - (t * (t - 1)) / 2;  // pair_index(L, t, u) = rowt + u - t
-                    if (ct > 1) atomicAdd(ar + rowt, ct * (ct - 1) / 2);
-                    for (uint32_t mu = mt & (mt - 1u); mu; mu &= mu - 1u) {
-                        const int u = __ffs(mu) - 1;
-                        atomicAdd(ar + rowt + (u - t), ct * c[u]);
-                    }
-                }
+                const int row = p.half ? Lp >> 1 : L;
+                for (int q = 0; q < row; ++q) tab[bl * (uint32_t)row + q] = 0u;
+                if (sum >= 2) c4_add(h4, L, ta, tb, c);
             }
             __syncthreads();
             for (int q = tid; q < nfar / 32; q += blockDim.x) tbits[q] = 0u;
@@ -1182,8 +1438,6 @@ __global__ void __launch_bounds__(kBinPairThreads) k_c4_bin_pairs(C4Bin p) {
             __syncthreads();
         }
     }
-    if (acc_mode && cur_ta >= 0) bin_flush(acc, h4, L, P, cur_ta);
-    __syncthreads();
     for (int64_t q = tid; q < p.n4; q += blockDim.x)
         if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
 }
@@ -1777,28 +2031,32 @@ int c4_walk_waves(const C4Params &p, const tg_graph *g, const uint32_t *list, in
     return TG_OK;
 }
 
-// Window bits of the binned waves: the largest window whose dense table
-// (16-bit counts when half, else 32-bit) fits kBinTable bytes, with room for
-// the type in a 16-bit entry.
+// Bits of the type in a bucket entry: an entry is the index of its count in a table
+// of 2^tlg counts a row.
+int bin_tlg(int L) { return L <= 2 ? 1 : L <= 4 ? 2 : L <= 8 ? 3 : 4; }
+
+// Window bits of the binned waves: the largest window whose dense table (16-bit
+// counts when half, else 32-bit) fits kBinTable bytes, with room for the type in
+// a 16-bit entry.
 int c4_bin_wlg(int L, int half) {
-    const int Lp = L + (L & 1);
-    const size_t per = half ? (size_t)Lp * 2 : (size_t)L * 4;
-    int tbits = 1;
-    while ((1 << tbits) < L) ++tbits;
+    const int G = bin_lanes(L), Lp = L + (L & 1);
+    const size_t per = G ? (size_t)G * (half ? 2 : 4) : half ? (size_t)Lp * 2 : (size_t)L * 4;
+    const int tbits = bin_tlg(L);
     int wlg = 5;
     while (wlg < 16 - tbits && ((size_t)1 << (wlg + 1)) * per <= kBinTable) ++wlg;
     return wlg;
 }
 
 // Global-mode binned waves of the anchors list[0 .. na) (degrees hdeg): walk
-// positions per anchor (k_c4_prefix), warp units (k_c4_units), then per wave
-// (anchors of one counter width, at most `ecap` walk positions in all) the
-// count pass, the bucket offsets, the fill pass and the bucket pairs.
+// positions per anchor (k_c4_prefix), warp units (k_c4_units), the far ends'
+// numbers, then per wave (anchors of one counter width, at most `ecap` walk
+// positions in all) the count pass, the bucket offsets, the fill pass and the
+// bucket pairs.  list is sorted by (counter width, type), types in ltype.
 int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
-                 const std::vector<int64_t> &hdeg, int64_t n4, unsigned long long *g4,
+                 const std::vector<int64_t> &hdeg, const std::vector<uint8_t> &ltype, int64_t n4, unsigned long long *g4,
                  unsigned long long *work, int64_t ecap, cudaStream_t s) {
     const int L = g->L;
-    const int64_t n = g->n;
+    const int64_t n = g->n_nonisolated;
     std::vector<int64_t> pb((size_t)na + 1, 0);
     for (int64_t q = 0; q < na; ++q) pb[q + 1] = pb[q] + hdeg[q];
     DevBuf<int64_t> dpb, dmp;
@@ -1807,6 +2065,29 @@ int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
     TG_TRY_CUDA(cudaMemcpyAsync(dpb.p, pb.data(), (na + 1) * 8, cudaMemcpyHostToDevice, s));
     k_c4_prefix<<<(unsigned)na, 256, 0, s>>>(list, dpb.p, g->rowptr, g->adj, dmp.p, dtot.p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
+    // far-end numbers, types padded to the windows of the 16-bit waves (those of
+    // the 32-bit ones divide them)
+    const int64_t nblk = (n + kRankBlock - 1) / kRankBlock;
+    DevBuf<uint32_t> tcnt, tbase, num, badj, thr;
+    DevBuf<uint8_t> htype;
+    if (!tcnt.alloc(L * nblk + 1, s) || !tbase.alloc(L + 1, s) || !num.alloc(n, s) ||
+        !badj.alloc(2 * g->M, s) || !thr.alloc(na * L, s) || !htype.alloc(na, s))
+        return TG_ENOMEM;
+    k_bin_hist<<<(unsigned)nblk, kRankBlock, 0, s>>>(g->ntype, n, nblk, L, tcnt.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    TG_TRY(tg_scan_u32(tcnt.p, tcnt.p, L * nblk + 1, s));
+    k_bin_bases<<<1, 32, 0, s>>>(tcnt.p, nblk, L, c4_bin_wlg(L, 1), tbase.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    k_bin_numbers<<<(unsigned)nblk, kRankBlock, 0, s>>>(g->ntype, n, nblk, L, tcnt.p, tbase.p, num.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    k_bin_entries<<<(unsigned)std::min<int64_t>((2 * g->M + 255) / 256, 65535LL * 16), 256, 0, s>>>(
+        g->adj, 2 * g->M, num.p, badj.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    k_bin_thresholds<<<(unsigned)std::min<int64_t>((na + 7) / 8, 65535), 256, 0, s>>>(
+        list, na, g->ntype, nblk, L, tcnt.p, tbase.p, thr.p, htype.p); tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
+    C4Bin pb0{};
+    TG_TRY_CUDA(cudaMemcpyAsync(pb0.tbase, tbase.p, (L + 1) * 4, cudaMemcpyDeviceToHost, s));
     std::vector<unsigned long long> tot_h((size_t)na);
     TG_TRY_CUDA(cudaMemcpyAsync(tot_h.data(), dtot.p, na * 8, cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
@@ -1823,7 +2104,7 @@ int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
     int64_t wmax = 0;
     for (int64_t q = 0; q < na;) {
         const int half = hdeg[q] < 65536 ? 1 : 0;
-        const int64_t W = (n + ((int64_t)1 << c4_bin_wlg(L, half)) - 1) >> c4_bin_wlg(L, half);
+        const int64_t W = (int64_t)pb0.tbase[L] >> c4_bin_wlg(L, half);
         int64_t e = q + 1;
         unsigned long long tot = tot_h[q];
         while (e < na && (hdeg[e] < 65536 ? 1 : 0) == half && tot + tot_h[e] <= (unsigned long long)ecap &&
@@ -1851,7 +2132,20 @@ int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
             us[q + 1] = us[q] + (int64_t)((tot_h[q] + tgt - 1) / tgt);
         }
     }
+    // runs of anchors of one type inside a wave
+    std::vector<int2> runs;
+    std::vector<int64_t> wr((size_t)nwaves + 1, 0);
+    for (int64_t w = 0; w < nwaves; ++w) {
+        for (int64_t q = wq0[w]; q < wq1[w];) {
+            int64_t e = q + 1;
+            while (e < wq1[w] && e - q < kBinRun && ltype[e] == ltype[q]) ++e;
+            runs.push_back(make_int2((int)q, (int)e));
+            q = e;
+        }
+        wr[w + 1] = (int64_t)runs.size();
+    }
     const int64_t nunits = us[na];
+    DevBuf<int2> druns;
     DevBuf<int64_t> dus, dtg;
     DevBuf<C4Unit> dun;
     DevBuf<unsigned long long> dq;
@@ -1859,8 +2153,9 @@ int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
     DevBuf<uint16_t> bins;
     if (!dus.alloc(na + 1, s) || !dtg.alloc(na, s) || !dun.alloc(nunits ? nunits : 1, s) ||
         !dq.alloc(3 * nwaves, s) || !cnt.alloc(wmax + 1, s) || !offs.alloc(wmax + 1, s) ||
-        !bins.alloc(wtmax ? wtmax : 1, s))
+        !bins.alloc(wtmax + 4, s) || !druns.alloc(runs.size(), s))
         return TG_ENOMEM;
+    TG_TRY_CUDA(cudaMemcpyAsync(druns.p, runs.data(), runs.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
     TG_TRY_CUDA(cudaMemcpyAsync(dus.p, us.data(), (na + 1) * 8, cudaMemcpyHostToDevice, s));
     TG_TRY_CUDA(cudaMemcpyAsync(dtg.p, tg.data(), na * 8, cudaMemcpyHostToDevice, s));
     TG_TRY_CUDA(cudaMemsetAsync(dq.p, 0, 3 * nwaves * 8, s));
@@ -1870,12 +2165,12 @@ int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
                                       dun.p); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
     }
-    C4Bin pb0{};
     pb0.rowptr = g->rowptr;
     pb0.adj = g->adj;
-    pb0.ntype = g->ntype;
+    pb0.badj = badj.p;
+    pb0.thr = thr.p;
+    pb0.htype = htype.p;
     pb0.L = L;
-    pb0.n = n;
     pb0.heavy = list;
     pb0.mprefix = dmp.p;
     pb0.pbase = dpb.p;
@@ -1885,44 +2180,48 @@ int c4_bin_waves(const tg_graph *g, const uint32_t *list, int64_t na,
     pb0.g4 = g4;
     pb0.n4 = n4;
     pb0.work = work;
-    TG_TRY(tg_allow_max_smem((const void *)k_c4_bin_pairs));
     for (int64_t w = 0; w < nwaves; ++w) {
         const int64_t q0 = wq0[w], q1 = wq1[w];
         C4Bin pw = pb0;
         pw.half = whalf[w];
         pw.wlg = c4_bin_wlg(L, pw.half);
-        pw.W = (n + ((int64_t)1 << pw.wlg) - 1) >> pw.wlg;
+        pw.tlg = bin_tlg(L);
+        pw.W = (int64_t)pw.tbase[L] >> pw.wlg;
         pw.q0 = q0;
-        pw.nb = (q1 - q0) * pw.W;
+        const int64_t nb = (q1 - q0) * pw.W;
         pw.units = dun.p + us[q0];
         pw.n_units = us[q1] - us[q0];
         if (pw.n_units == 0) continue;
         const int64_t need = (pw.n_units + kC4WalkWarps - 1) / kC4WalkWarps;
         const int64_t grid = std::min<int64_t>(walk_grid, need);
         // bucket sizes, then offsets (one more entry, zero, takes the total)
-        TG_TRY_CUDA(cudaMemsetAsync(cnt.p, 0, (pw.nb + 1) * 4, s));
+        TG_TRY_CUDA(cudaMemsetAsync(cnt.p, 0, (nb + 1) * 4, s));
         pw.queue = dq.p + 3 * w;
         k_c4_bin_walk<false><<<(unsigned)grid, kC4WalkWarps * 32, 0, s>>>(pw); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
-        TG_TRY(tg_scan_u32(cnt.p, offs.p, pw.nb + 1, s));
-        TG_TRY_CUDA(cudaMemcpyAsync(cnt.p, offs.p, pw.nb * 4, cudaMemcpyDeviceToDevice, s));
+        TG_TRY(tg_scan_u32(cnt.p, offs.p, nb + 1, s));
+        TG_TRY_CUDA(cudaMemcpyAsync(cnt.p, offs.p, nb * 4, cudaMemcpyDeviceToDevice, s));
         pw.queue = dq.p + 3 * w + 1;
         k_c4_bin_walk<true><<<(unsigned)grid, kC4WalkWarps * 32, 0, s>>>(pw); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
-        const int Lp = L + (L & 1);
-        const size_t nfar = (size_t)1 << pw.wlg;
-        const int P = L * (L + 1) / 2;
-        const size_t psmem = (((size_t)n4 * 8 + 15) & ~(size_t)15) +
-                             (L <= kBinAccL ? (((size_t)L * P * 8 + 15) & ~(size_t)15) : 0) +
-                             (pw.half ? nfar * (Lp >> 1) : nfar * L) * 4 + nfar / 32 * 4 + nfar * 2;
+        pw.runs = druns.p + wr[w];
+        pw.nitems = (wr[w + 1] - wr[w]) * pw.W;
+        const int G = bin_lanes(L), Lp = L + (L & 1);
+        const size_t nfar = (size_t)1 << pw.wlg, h4b = ((size_t)n4 * 8 + 15) & ~(size_t)15;
+        void (*const fn)(C4Bin) = G == 2   ? (pw.half ? k_c4_bin_gram<2, true> : k_c4_bin_gram<2, false>)
+                                  : G == 4 ? (pw.half ? k_c4_bin_gram<4, true> : k_c4_bin_gram<4, false>)
+                                  : G == 8 ? (pw.half ? k_c4_bin_gram<8, true> : k_c4_bin_gram<8, false>)
+                                           : k_c4_bin_pairs;
+        const int threads = G ? kGramThreads : kBinPairThreads;
+        const size_t psmem = h4b + (G ? nfar * G * (pw.half ? 2 : 4)
+                                      : (pw.half ? nfar * (Lp >> 1) : nfar * L) * 4 + nfar / 32 * 4 + nfar * 2);
+        TG_TRY(tg_allow_max_smem((const void *)fn));
         int pper = 0;
-        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pper, k_c4_bin_pairs,
-                                                                  kBinPairThreads, psmem));
+        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pper, fn, threads, psmem));
         if (pper < 1) pper = 1;
-        const int64_t pgrid =
-            std::min<int64_t>((int64_t)tg_num_sms() * pper, (pw.nb + kBinRun - 1) / kBinRun);
+        const int64_t pgrid = std::min<int64_t>((int64_t)tg_num_sms() * pper, pw.nitems);
         pw.queue = dq.p + 3 * w + 2;
-        k_c4_bin_pairs<<<(unsigned)pgrid, kBinPairThreads, psmem, s>>>(pw); tg_note_launch();
+        fn<<<(unsigned)pgrid, threads, psmem, s>>>(pw); tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
     }
     // the host vectors are read by the copies above before they go out of scope
@@ -2023,21 +2322,39 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
         // bucket entries of one wave: 2 bytes each, within an eighth of free memory
         const int64_t ecap = std::min<int64_t>((int64_t)1 << 31, (int64_t)(fb / 16));
         std::vector<uint32_t> lb, ls;
+        // far-end numbers, types padded to whole windows, have to fit an entry's id
+        const bool numbered = g->n_nonisolated + ((int64_t)L << c4_bin_wlg(L, 1)) <= (int64_t)TG_IDMASK;
         std::vector<int64_t> db, ds;
+        std::vector<uint8_t> tyb;
+        std::vector<C4HeavyInfo> ib;
         for (int64_t q = 0; q < nheavy; ++q) {
             const int half = hdeg[q] < 65536 ? 1 : 0;
             const int wlg = c4_bin_wlg(L, half);
-            const int64_t span = ((n - 1) >> wlg) - ((int64_t)heavy[q] >> wlg) + 1;
-            const bool bin = global && t.unroll != 1 && info[q].cost >= (unsigned long long)bin_fill * span &&
+            const int64_t span = ((g->n_nonisolated - 1) >> wlg) - ((int64_t)heavy[q] >> wlg) + 1;
+            const bool bin = global && numbered && t.unroll != 1 && info[q].cost >= (unsigned long long)bin_fill * span &&
                              info[q].cost <= (unsigned long long)ecap;
-            (bin ? lb : ls).push_back(heavy[q]);
-            (bin ? db : ds).push_back(hdeg[q]);
+            if (bin) {
+                ib.push_back(info[q]);
+                continue;
+            }
+            ls.push_back(heavy[q]);
+            ds.push_back(hdeg[q]);
+        }
+        // binned anchors by counter width, then type
+        std::stable_sort(ib.begin(), ib.end(), [](const C4HeavyInfo &x, const C4HeavyInfo &y) {
+            const bool xw = x.degree < 65536, yw = y.degree < 65536;
+            return xw != yw ? yw : x.type < y.type;
+        });
+        for (const C4HeavyInfo &x : ib) {
+            lb.push_back(x.a);
+            db.push_back(x.degree);
+            tyb.push_back((uint8_t)x.type);
         }
         DevBuf<uint32_t> dlb, dls;
         if (!dlb.alloc(lb.size() + 1, s) || !dls.alloc(ls.size() + 1, s)) return TG_ENOMEM;
         if (!lb.empty()) {
             TG_TRY_CUDA(cudaMemcpyAsync(dlb.p, lb.data(), lb.size() * 4, cudaMemcpyHostToDevice, s));
-            TG_TRY(c4_bin_waves(g, dlb.p, (int64_t)lb.size(), db, n4, g4, work, ecap, s));
+            TG_TRY(c4_bin_waves(g, dlb.p, (int64_t)lb.size(), db, tyb, n4, g4, work, ecap, s));
         }
         if (!ls.empty()) {
             TG_TRY_CUDA(cudaMemcpyAsync(dls.p, ls.data(), ls.size() * 4, cudaMemcpyHostToDevice, s));

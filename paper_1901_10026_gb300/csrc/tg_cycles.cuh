@@ -12,7 +12,7 @@ enum { kC4Warp = 0, kC4Cta, kC4CtaLarge, kC4Slot, kC4Split, kC4Classes };
 struct C4HeavyInfo {
     unsigned long long cost;
     int64_t degree;
-    uint32_t a, pad;
+    uint32_t a, type;
 };
 
 struct C4Lists {
