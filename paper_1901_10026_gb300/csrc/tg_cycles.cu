@@ -879,7 +879,7 @@ __device__ __forceinline__ void k4_hist_add(unsigned long long *h4, int a, int b
 //
 // With windows over the node ids (types mixed) a far end's pairs went, one 64-bit
 // shared add each, to a table by (type of b, pair).  4-cycle phase, before -> now:
-// R-MAT-21 (1.43e10 wedges, L = 8) 316 -> 184 ms, CL-1M (9.1e8, L = 5) 33.5 -> 20.9
+// R-MAT-21 (1.43e10 wedges, L = 8) 316 -> 166 ms, CL-1M (9.1e8, L = 5) 33.5 -> 19.0
 // ms, CL-100K (5.8e7) 4.1 -> 2.5 ms.
 struct C4Bin {
     const int64_t *rowptr;
@@ -1149,36 +1149,39 @@ __device__ __forceinline__ void ldsm_t4(uint32_t addr, uint32_t (&r)[4]) {
                  : "memory");
 }
 
-// d += x^T y over 16 far ends: x0, y0 hold the counts of far ends 0..7 in the
+// d[0..1] += x^T y over 16 far ends: x0, y0 hold the counts of far ends 0..7 in the
 // transposed ldmatrix layout (lane: type lane / 4, far ends 2 (lane % 4) and the
-// next), x1, y1 those of far ends 8..15; d: types (lane / 4, 2 (lane % 4) and the
-// next).  A's other eight rows are zero.
-__device__ __forceinline__ void gram16(float (&d)[2], uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1) {
-    float z0 = 0.f, z1 = 0.f;
+// next), x1, y1 those of far ends 8..15; d[0..1]: types (lane / 4, 2 (lane % 4) and
+// the next).  Row 8 of A is `row8` (lanes 0..3): with ones there, d[2..3] of lanes
+// 0..3 are the sums of y.
+__device__ __forceinline__ void gram16(float (&d)[4], uint32_t x0, uint32_t x1, uint32_t row8, uint32_t y0,
+                                       uint32_t y1) {
     asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %5}, {%7, %8}, "
         "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(z0), "+f"(z1)
-        : "r"(x0), "r"(0u), "r"(x1), "r"(0u), "r"(y0), "r"(y1));
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(x0), "r"(row8), "r"(x1), "r"(y0), "r"(y1));
 }
 
-// Two counts below 1024 in 16-bit halves as two fp16 values: 0x6400 is 1024 and
-// its last place 1.
-__device__ __forceinline__ uint32_t counts_f16(uint32_t x) {
-    uint32_t r;
-    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x | 0x64006400u), "r"(0x64006400u));
-    return r;
-}
+// A count c below 1024 read as an fp16 value is the subnormal c 2^-24, so products
+// of two counts are exact multiples of 2^-48 and sums of counts of 2^-24.
+constexpr float kGramScale = 281474976710656.f, kSumScale = 16777216.f;
 
 // Buckets of a binned wave, L <= 8 types.  A CTA takes an item (anchors of one
 // type, one window): bucket after bucket it counts the entries in the table (a row
 // of counts per far end), then sums c_t c_t' over the far ends and clears it.  With
 // eight 16-bit counts a row (5 to 8 types) the sums are X^T X of the table X on the
 // tensor cores: a row is a row of an 8 x 8 matrix of 16-bit values, so one ldmatrix
-// gives 32 far ends in the layout of both operands, and counts up to 255 are exact
-// as fp16, their sums over 128 far ends (two of them in the cross terms) below 2^24
-// in fp32, which are then added to 64-bit sums.  Where a count is larger its high and low bytes take the place of
-// it: 65536 H^T H + 256 (H^T L + L^T H) + L^T L.  The other row widths sum the rows
+// gives 32 far ends in the layout of both operands, and the counts are used as they
+// stand, as fp16 subnormals.  The fp32 sums hold integers below 2^24 (times a power
+// of two) and are exact: a warp adds them to its 64-bit sums before the blocks of 128
+// far ends since then could pass it (33 blocks of counts up to 63, or one of counts
+// up to 255 and 16 of those).  Where a count is larger its high and low bytes take
+// its place: 65536 H^T H + 256 (H^T L + L^T H) + L^T L.  On R-MAT-18 the kernel takes
+// 2.5 ms (5.7 with the sums in integer registers, 3.0 with the counts converted and a
+// second product for sum c); the reads and clears of the 64 KB table (1,024 shared
+// wavefronts a bucket) and the two barriers a bucket bound it.  Two CTAs per SM: three
+// need spills (R-MAT-21 174 against 166 ms).  The other row widths sum the rows
 // with two middles or more in groups of G lanes, lane a holding sum c_a c_b for every
 // b.  No add to shared memory is made until the item's end.
 template <int G, bool kHalf>
@@ -1211,9 +1214,23 @@ __global__ void __launch_bounds__(kGramThreads, 2) k_c4_bin_gram(C4Bin p) {
             s_off[2 * tid + 1] = p.offs[b + 1];
         }
         __syncthreads();
-        unsigned long long acc[kSums], one = 0;
+        unsigned long long acc[kSums], one[2] = {0ull, 0ull};
 #pragma unroll
         for (int b = 0; b < kSums; ++b) acc[b] = 0ull;
+        // kMma: the fp32 sums since the last settling (row 8, lanes 0..3: sums of the
+        // counts of types 2 gg and the next), and the blocks in them by weight
+        float ll[4] = {0.f, 0.f, 0.f, 0.f};
+        int spent = 0;
+        const uint32_t row8 = lane < 4 ? 0x3c003c00u : 0u;  // 1.0, 1.0
+        auto settle = [&]() {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                acc[b % kSums] += (uint32_t)(ll[b] * kGramScale);
+                one[b] += (uint32_t)(ll[2 + b] * kSumScale);
+                ll[b] = ll[2 + b] = 0.f;
+            }
+            spent = 0;
+        };
         // four entries at 8-byte boundaries; those outside the bucket are left out
         auto fetch = [&](uint32_t k, uint32_t c1) -> uint2 {
             return k < c1 ? *reinterpret_cast<const uint2 *>(p.bins + k) : make_uint2(0u, 0u);
@@ -1261,42 +1278,38 @@ __global__ void __launch_bounds__(kGramThreads, 2) k_c4_bin_gram(C4Bin p) {
                     uint4 *row = reinterpret_cast<uint4 *>(tab) + r0 + lane;
 #pragma unroll
                     for (int z = 0; z < 4; ++z) row[32 * z] = make_uint4(0u, 0u, 0u, 0u);
-                    const uint32_t ones = 0x3c003c00u;  // 1.0, 1.0
-                    float ll[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
                     if (!(big & 0xff00ff00u)) {
+                        const int weight = big & 0xffc0ffc0u ? 17 : 1;
+                        if (spent + weight > 33) settle();
+                        spent += weight;
 #pragma unroll
-                        for (int z = 0; z < 4; ++z)
-#pragma unroll
-                            for (int h = 0; h < 4; h += 2) {
-                                const uint32_t l0 = counts_f16(x[z][h]), l1 = counts_f16(x[z][h + 1]);
-                                gram16(ll, l0, l1, l0, l1);
-                                gram16(s1, l0, l1, ones, ones);
-                            }
+                        for (int z = 0; z < 4; ++z) {
+                            gram16(ll, x[z][0], x[z][1], row8, x[z][0], x[z][1]);
+                            gram16(ll, x[z][2], x[z][3], row8, x[z][2], x[z][3]);
+                        }
                     } else {
-                        float lh[2] = {0.f, 0.f}, hh[2] = {0.f, 0.f}, sh[2] = {0.f, 0.f};
+                        settle();
+                        float lh[4] = {0.f, 0.f, 0.f, 0.f}, hh[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int z = 0; z < 4; ++z)
 #pragma unroll
                             for (int h = 0; h < 4; h += 2) {
-                                const uint32_t l0 = counts_f16(x[z][h] & 0x00ff00ffu);
-                                const uint32_t l1 = counts_f16(x[z][h + 1] & 0x00ff00ffu);
-                                const uint32_t h0 = counts_f16((x[z][h] >> 8) & 0x00ff00ffu);
-                                const uint32_t h1 = counts_f16((x[z][h + 1] >> 8) & 0x00ff00ffu);
-                                gram16(ll, l0, l1, l0, l1);
-                                gram16(lh, l0, l1, h0, h1);
-                                gram16(lh, h0, h1, l0, l1);
-                                gram16(hh, h0, h1, h0, h1);
-                                gram16(s1, l0, l1, ones, ones);
-                                gram16(sh, h0, h1, ones, ones);
+                                const uint32_t l0 = x[z][h] & 0x00ff00ffu, l1 = x[z][h + 1] & 0x00ff00ffu;
+                                const uint32_t h0 = (x[z][h] >> 8) & 0x00ff00ffu;
+                                const uint32_t h1 = (x[z][h + 1] >> 8) & 0x00ff00ffu;
+                                gram16(ll, l0, l1, row8, l0, l1);
+                                gram16(lh, l0, l1, 0u, h0, h1);
+                                gram16(lh, h0, h1, 0u, l0, l1);
+                                gram16(hh, h0, h1, row8, h0, h1);
                             }
 #pragma unroll
-                        for (int b = 0; b < 2; ++b)
-                            acc[b % kSums] += 256ull * (uint32_t)lh[b] + 65536ull * (uint32_t)hh[b];
-                        one += 256ull * (uint32_t)sh[0];
+                        for (int b = 0; b < 2; ++b) {
+                            acc[b % kSums] += 256ull * (uint32_t)(lh[b] * kGramScale) +
+                                              65536ull * (uint32_t)(hh[b] * kGramScale);
+                            one[b] += 256ull * (uint32_t)(hh[2 + b] * kSumScale);
+                        }
+                        settle();
                     }
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) acc[b % kSums] += (uint32_t)ll[b];
-                    one += (uint32_t)s1[0];
                 }
             } else {
                 for (int row = tid; row < nfar; row += kGramThreads) {
@@ -1336,7 +1349,7 @@ __global__ void __launch_bounds__(kGramThreads, 2) k_c4_bin_gram(C4Bin p) {
                         for (int b = 0; b < G; ++b)
                             if (b == ga) ca = c[b];
                         if (!mine) ca = 0u;
-                        one += ca;
+                        one[0] += ca;
 #pragma unroll
                         for (int b = 0; b < kSums; ++b) acc[b] += (unsigned long long)ca * c[b];
                     }
@@ -1344,22 +1357,28 @@ __global__ void __launch_bounds__(kGramThreads, 2) k_c4_bin_gram(C4Bin p) {
             }
             __syncthreads();
         }
-        // the item's sums over the groups of a warp, then into the histogram
-        if (!kMma) {
+        // the item's sums over the groups of a warp, then into the histogram; `own`:
+        // the sum of the counts of this lane's type
+        unsigned long long own = one[0];
+        if (kMma) {
+            settle();
+            const unsigned long long s0 = __shfl_sync(kFull, one[0], ga / 2), s1 = __shfl_sync(kFull, one[1], ga / 2);
+            own = ga & 1 ? s1 : s0;
+        } else {
 #pragma unroll
             for (int o = G; o < 32; o <<= 1) {
-                one += __shfl_xor_sync(kFull, one, o);
+                own += __shfl_xor_sync(kFull, own, o);
 #pragma unroll
                 for (int b = 0; b < kSums; ++b) acc[b] += __shfl_xor_sync(kFull, acc[b], o);
             }
         }
-        if ((kMma || gg == 0) && one) {
+        if ((kMma || gg == 0) && own) {
             const int ta = p.htype[run.x], tb = bin_type(p, w);
 #pragma unroll
             for (int b = 0; b < kSums; ++b) {
                 const int t = kMma ? 2 * gg + b : b;
                 if (t < ga) continue;
-                const unsigned long long x = t == ga ? (acc[b] - one) / 2 : acc[b];
+                const unsigned long long x = t == ga ? (acc[b] - own) / 2 : acc[b];
                 if (x) k4_hist_add(h4, ta, tb, ga, t, x);
             }
         }
