@@ -995,6 +995,7 @@ static void sched_dfree(tg_sched *sc, cudaStream_t s) {
     tg_dfree(sc->lists.uadj, 0, s);
     tg_dfree(sc->lists.ueid, 0, s);
     tg_dfree(sc->lists.order, 0, s);
+    tg_dfree(sc->lists.other, 0, s);
     tg_dfree(sc->sorted, 0, s);
     tg_dfree(sc->s, 0, s);
 }
@@ -1191,8 +1192,8 @@ static int launch_cta_u(const CountParams &p, const CtaParams &cp, int threads, 
 }
 
 // Launch the counting kernel over `count` edges (order[item] or e0 + item);
-// full_order is the grouped order of the whole graph.
-static int launch_count(const tg_graph *g, int k, int level, const uint32_t *full_order,
+// lists holds the grouped order of the whole graph.
+static int launch_count(const tg_graph *g, int k, int level, const tg_lists &lists,
                         const uint32_t *order, int64_t e0, int64_t count, uint64_t *rows,
                         int64_t width, unsigned long long *hist, cudaStream_t s) {
     if (count <= 0) return TG_OK;
@@ -1201,7 +1202,7 @@ static int launch_count(const tg_graph *g, int k, int level, const uint32_t *ful
         if ((t0.kernel == TG_KERNEL_AUTO || t0.kernel == TG_KERNEL_REUSE ||
              t0.kernel == TG_KERNEL_CYCLES) &&
             order)
-            return tg_reuse_count(g, k, level, full_order, order, count, rows, width, hist, t0, s);
+            return tg_reuse_count(g, k, level, lists, order, count, rows, width, hist, t0, s);
     }
     DevBuf<unsigned long long> queue;
     if (!queue.alloc(1, s)) return TG_ENOMEM;
@@ -1238,11 +1239,11 @@ static int sums_impl(const tg_graph *g, int k, int64_t e0, int64_t e1,
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
     if (e0 == 0 && e1 == g->M)
-        return launch_count(g, k, TG_GRAPHLET, sc->lists.order, sc->lists.order, 0, g->M, nullptr, 0, dsums,
+        return launch_count(g, k, TG_GRAPHLET, sc->lists, sc->lists.order, 0, g->M, nullptr, 0, dsums,
                             s);
     DevBuf<uint32_t> order;
     TG_TRY(grouped_order(g, e0, e1 - e0, s, order));
-    return launch_count(g, k, TG_GRAPHLET, sc->lists.order, order.p, 0, e1 - e0, nullptr, 0, dsums, s);
+    return launch_count(g, k, TG_GRAPHLET, sc->lists, order.p, 0, e1 - e0, nullptr, 0, dsums, s);
 }
 extern "C" int tg_count_global(const tg_graph *g, int32_t k, uint64_t *out, void *stream) {
     TG_TRY(check_counts(g, k));
@@ -1372,14 +1373,14 @@ extern "C" int tg_count_shard(const tg_graph *g, int32_t k, int32_t shard, int32
             part.index = shard;
             part.count = nshards;
             if (k == 4)
-                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists.order, sc->sorted + q[0], q[1] - q[0],
+                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], q[1] - q[0],
                                       nullptr, 0, dsums, t, s, part));
             else if (q[1] > q[0])
-                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists.order, sc->sorted + q[0], q[1] - q[0],
+                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], q[1] - q[0],
                                       nullptr, 0, dsums, t, s));
         } else if (q[1] > q[0]) {
             // the per-edge kernels need nothing beyond the slice's edges
-            TG_TRY(launch_count(g, k, TG_GRAPHLET, sc->lists.order, sc->sorted + q[0], 0, q[1] - q[0],
+            TG_TRY(launch_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], 0, q[1] - q[0],
                                 nullptr, 0, dsums, s));
         }
     }
@@ -1398,13 +1399,13 @@ extern "C" int tg_count_per_edge(const tg_graph *g, int32_t k, int32_t level, ui
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
     if (tg_is_device_ptr(rows)) {
-        TG_TRY(launch_count(g, k, level, sc->lists.order, sc->lists.order, 0, g->M, rows, width, nullptr, s));
+        TG_TRY(launch_count(g, k, level, sc->lists, sc->lists.order, 0, g->M, rows, width, nullptr, s));
         TG_TRY_CUDA(cudaStreamSynchronize(s));
         return TG_OK;
     }
     DevBuf<uint64_t> d;
     if (!d.alloc((size_t)g->M * width, s)) return TG_ENOMEM;
-    TG_TRY(launch_count(g, k, level, sc->lists.order, sc->lists.order, 0, g->M, d.p, width, nullptr, s));
+    TG_TRY(launch_count(g, k, level, sc->lists, sc->lists.order, 0, g->M, d.p, width, nullptr, s));
     TG_TRY_CUDA(cudaMemcpyAsync(rows, d.p, (size_t)g->M * width * 8, cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
     return TG_OK;
@@ -1415,7 +1416,7 @@ int tg_rows_device(const tg_graph *g, int k, int level, uint64_t *rows, cudaStre
     if (g->M == 0) return TG_OK;
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
-    return launch_count(g, k, level, sc->lists.order, sc->lists.order, 0, g->M, rows,
+    return launch_count(g, k, level, sc->lists, sc->lists.order, 0, g->M, rows,
                         tg_slots(g->L, k, level), nullptr, s);
 }
 
@@ -1428,7 +1429,7 @@ int tg_rows_mapped(const tg_graph *g, int k, int level, uint64_t *const *rowmap,
     if (g->M > 0) {
         tg_sched *sc = nullptr;
         TG_TRY(get_sched(g, s, &sc));
-        TG_TRY(tg_reuse_count(g, k, level, sc->lists.order, sc->lists.order, g->M, nullptr,
+        TG_TRY(tg_reuse_count(g, k, level, sc->lists, sc->lists.order, g->M, nullptr,
                               tg_slots(g->L, k, level), nullptr, t, s, tg_part(), rowmap));
     }
     *done = true;

@@ -285,14 +285,13 @@ __global__ void __launch_bounds__(kDirThreads) k_dir3(DirParams p) {
 // over the edges of one type and adds them to the sums once.
 //
 // Before, one warp per edge searched every member of the shorter list in the
-// longer one and evaluated 13 L slots per edge: 84.4 -> 25.0 ms on R-MAT-20 (15.7M
-// edges, L = 8), of which the heavy units take 22.5 ms, bound by the reads of
-// Gamma_i (entries and arc bits) and the shared-memory adds of the hits.
+// longer one and evaluated 13 L slots per edge: 84.4 -> 19.0 ms on R-MAT-20 (15.7M
+// edges, L = 8), of which the heavy units take 16.4 ms (22.5 with one edge at a time),
+// bound by the shared-memory adds of the hits and the reads of Gamma_i.
 struct TriParams {
     DirParams d;
-    const uint32_t *eid;
     const uint8_t *est;      // state of edge e seen from its smaller id
-    const uint32_t *order, *ustart, *ulist;
+    const uint32_t *order, *other, *ustart, *ulist;
     uint32_t nunits;
     int64_t nbits;           // ids below it are in the shared map (heavy units)
     int32_t hist_smem;
@@ -331,39 +330,85 @@ __device__ __forceinline__ void tri_flush(const DirParams &p, unsigned long long
     }
 }
 
-constexpr int kTriUnroll = 4;
+constexpr int kTriUnroll = 4;  // chunks of 32 entries tested and in flight per warp
 
-// One edge's scan of Gamma_i: state(id, entry) is the state of (j, w) or 0.
+// The edges q0, q0 + stride, ... (nb <= 32 of them, the same in every lane) of a
+// unit of j (type tj) by one warp, as tau_batch of tg_reuse.cu: lane k reads edge k's
+// id, state, end and list bounds, and the next edge's first chunks are read before
+// the current edge's are tested.  state(id, entry): the state of (j, w), or 0; pj: j's
+// packed entry (j is no neighbour of itself).  Counts wait in cnt while the type of
+// i stays ti (any: there are some).
 template <class State>
-__device__ __forceinline__ bool tri_scan(const DirParams &p, int64_t bi, int di, uint32_t j,
-                                         uint32_t *cnt, State state) {
-    const int lane = threadIdx.x & 31, L = p.L;
-    bool any = false;
-    for (int c0 = 0; c0 < di; c0 += 32 * kTriUnroll) {
-        uint32_t w[kTriUnroll];
-        int siw[kTriUnroll];
+__device__ __forceinline__ void tri_batch(const TriParams &p, unsigned long long *h, uint32_t *cnt,
+                                          uint32_t q0, uint32_t stride, int nb, int tj, uint32_t pj,
+                                          int &ti, bool &any, State state) {
+    const int lane = threadIdx.x & 31, L = p.d.L;
+    int sij = 0, d = 0, t = 0;
+    int64_t b = 0;
+    if (lane < nb) {
+        const uint32_t w = __ldg(p.other + q0 + lane * stride);
+        sij = swap_state(__ldg(p.est + __ldg(p.order + q0 + lane * stride)));
+        t = (int)(w >> TG_TSHIFT);
+        b = __ldg(p.d.rowptr + (w & TG_IDMASK));
+        d = (int)(__ldg(p.d.rowptr + (w & TG_IDMASK) + 1) - b);
+    }
+    uint32_t wv[kTriUnroll];
+    int sv[kTriUnroll];
+    int64_t bk = __shfl_sync(kFull, b, 0);
+    int dk = __shfl_sync(kFull, d, 0);
 #pragma unroll
-        for (int u = 0; u < kTriUnroll; ++u) {
-            const int x = c0 + 32 * u + lane;
-            w[u] = x < di ? __ldg(p.adj + bi + x) : j;  // j itself is no triangle node
-            siw[u] = x < di ? (int)__ldg(p.adir + bi + x) : 0;
+    for (int u = 0; u < kTriUnroll; ++u) {
+        const int x = 32 * u + lane;
+        wv[u] = x < dk ? __ldg(p.d.adj + bk + x) : pj;
+        sv[u] = x < dk ? (int)__ldg(p.d.adir + bk + x) : 1;
+    }
+    for (int k = 0; k < nb; ++k) {
+        const int tk = __shfl_sync(kFull, t, k);
+        if (tk != ti) {
+            __syncwarp();
+            if (__any_sync(kFull, any)) tri_flush(p.d, h, cnt, ti, tj);
+            __syncwarp();
+            any = false;
+            ti = tk;
         }
+        uint32_t *ck = cnt + (__shfl_sync(kFull, sij, k) - 1) * 9 * L;
+        const int64_t bn = __shfl_sync(kFull, b, k + 1 < nb ? k + 1 : k);
+        const int dn = k + 1 < nb ? __shfl_sync(kFull, d, k + 1) : 0;
+        for (int c0 = 0; c0 < dk; c0 += 32 * kTriUnroll) {
+            const bool more = c0 + 32 * kTriUnroll < dk;
+            const int64_t nb0 = more ? bk : bn;
+            const int from = more ? c0 + 32 * kTriUnroll : 0, to = more ? dk : dn;
+            uint32_t nw[kTriUnroll];
+            int ns[kTriUnroll];
 #pragma unroll
-        for (int u = 0; u < kTriUnroll; ++u) {
-            const uint32_t id = w[u] & TG_IDMASK;
-            if (id == j) continue;
-            const int sjw = state(id, w[u]);
-            if (sjw) {
-                atomicAdd(cnt + ((siw[u] - 1) * 3 + sjw - 1) * L + (int)(w[u] >> TG_TSHIFT), 1u);
-                any = true;
+            for (int u = 0; u < kTriUnroll; ++u) {
+                const int x = from + 32 * u + lane;
+                nw[u] = x < to ? __ldg(p.d.adj + nb0 + x) : pj;
+                ns[u] = x < to ? (int)__ldg(p.d.adir + nb0 + x) : 1;
+            }
+#pragma unroll
+            for (int u = 0; u < kTriUnroll; ++u) {
+                if (u > 0 && c0 + 32 * u >= dk) break;
+                const int sjw = state(wv[u] & TG_IDMASK, wv[u]);
+                if (sjw) {
+                    atomicAdd(ck + ((sv[u] - 1) * 3 + sjw - 1) * L + (int)(wv[u] >> TG_TSHIFT), 1u);
+                    any = true;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kTriUnroll; ++u) {
+                wv[u] = nw[u];
+                sv[u] = ns[u];
             }
         }
+        bk = bn;
+        dk = dn;
     }
-    return __any_sync(kFull, any);
 }
 
 constexpr int kTriThreads = 1024;
 
+template <bool kAll>  // every id that occurs is in the map
 __global__ void __launch_bounds__(kTriThreads) k_tri_heavy(TriParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_unit;
@@ -413,35 +458,22 @@ __global__ void __launch_bounds__(kTriThreads) k_tri_heavy(TriParams p) {
         }
         int ti = -1;
         bool any = false;
-        for (uint32_t q = p0 + warp; q < p1; q += W) {
-            const uint32_t e = p.order[q];
-            const int2 ab = p.d.edges[e];
-            const int i = max(ab.x, ab.y);
-            const int t = p.d.ntype[i];
-            if (t != ti) {
-                __syncwarp();
-                if (any) tri_flush(p.d, h, cnt, ti, tj);
-                __syncwarp();
-                any = false;
-                ti = t;
-            }
-            const int sij = swap_state(p.est[e]);
-            const int64_t bi = p.d.rowptr[i];
-            const int di = (int)(p.d.rowptr[i + 1] - bi);
-            any |= tri_scan(p.d, bi, di, (uint32_t)j, cnt + (sij - 1) * 9 * L, [&](uint32_t id, uint32_t w) -> int {
-                if ((int64_t)id < p.nbits) return (int)((map[id >> 4] >> (2 * (id & 15u))) & 3u);
-                // beyond the map: the shorter of the two lists is searched
-                const int64_t by = p.d.rowptr[id];
-                if (p.d.rowptr[id + 1] - by < dj) {
-                    const int k = find_pos(p.d.adj, by, p.d.toff + (int64_t)id * (L + 1), pj);
-                    return k < 0 ? 0 : swap_state(p.d.adir[by + k]);
-                }
-                const int k = find_pos(p.d.adj, bj, toj, w);
-                return k < 0 ? 0 : (int)p.d.adir[bj + k];
-            });
-        }
+        for (uint32_t q = p0 + warp; q < p1; q += 32 * W)
+            tri_batch(p, h, cnt, q, (uint32_t)W, (int)min(32u, (p1 - q + W - 1) / W), tj, pj, ti, any,
+                      [&](uint32_t id, uint32_t w) -> int {
+                          if (kAll || id < (uint32_t)p.nbits) return (int)((map[id >> 4] >> (2 * (id & 15u))) & 3u);
+                          if (id == (uint32_t)j) return 0;
+                          // beyond the map: the shorter of the two lists is searched
+                          const int64_t by = p.d.rowptr[id];
+                          if (p.d.rowptr[id + 1] - by < dj) {
+                              const int k = find_pos(p.d.adj, by, p.d.toff + (int64_t)id * (L + 1), pj);
+                              return k < 0 ? 0 : swap_state(p.d.adir[by + k]);
+                          }
+                          const int k = find_pos(p.d.adj, bj, toj, w);
+                          return k < 0 ? 0 : (int)p.d.adir[bj + k];
+                      });
         __syncwarp();
-        if (any) tri_flush(p.d, h, cnt, ti, tj);
+        if (__any_sync(kFull, any)) tri_flush(p.d, h, cnt, ti, tj);
         __syncwarp();
     }
     if (p.hist_smem) {
@@ -479,6 +511,7 @@ __global__ void __launch_bounds__(kTriLightWarps * 32) k_tri_light(TriParams p) 
         const int64_t bj = p.d.rowptr[j];
         const int dj = (int)(p.d.rowptr[j + 1] - bj);
         const int tj = p.d.ntype[j];
+        const uint32_t pj = ((uint32_t)tj << TG_TSHIFT) | (uint32_t)j;
         int lg = 5;
         while ((1 << lg) < 2 * dj) ++lg;  // at most TG_LIGHT_LG
         const uint32_t mask = (1u << lg) - 1u;
@@ -493,33 +526,19 @@ __global__ void __launch_bounds__(kTriLightWarps * 32) k_tri_light(TriParams p) 
         __syncwarp();
         int ti = -1;
         bool any = false;
-        for (uint32_t q = p0; q < p1; ++q) {
-            const uint32_t e = p.order[q];
-            const int2 ab = p.d.edges[e];
-            const int i = max(ab.x, ab.y);
-            const int t = p.d.ntype[i];
-            if (t != ti) {
-                __syncwarp();
-                if (any) tri_flush(p.d, h, cnt, ti, tj);
-                __syncwarp();
-                any = false;
-                ti = t;
-            }
-            const int sij = swap_state(p.est[e]);
-            const int64_t bi = p.d.rowptr[i];
-            const int di = (int)(p.d.rowptr[i + 1] - bi);
-            any |= tri_scan(p.d, bi, di, (uint32_t)j, cnt + (sij - 1) * 9 * L, [&](uint32_t id, uint32_t) -> int {
-                uint32_t s = hset_slot(id, lg);
-                for (;;) {  // ends at an empty slot: the set is at most half full
-                    const uint32_t v = set[s];
-                    if (v == 0u) return 0;
-                    if ((v >> 2) == id) return (int)(v & 3u);
-                    s = (s + 1u) & mask;
-                }
-            });
-        }
+        for (uint32_t q = p0; q < p1; q += 32)
+            tri_batch(p, h, cnt, q, 1u, (int)min(32u, p1 - q), tj, pj, ti, any,
+                      [&](uint32_t id, uint32_t) -> int {
+                          uint32_t s = hset_slot(id, lg);
+                          for (;;) {  // ends at an empty slot: the set is at most half full
+                              const uint32_t v = set[s];
+                              if (v == 0u) return 0;
+                              if ((v >> 2) == id) return (int)(v & 3u);
+                              s = (s + 1u) & mask;
+                          }
+                      });
         __syncwarp();
-        if (any) tri_flush(p.d, h, cnt, ti, tj);
+        if (__any_sync(kFull, any)) tri_flush(p.d, h, cnt, ti, tj);
         __syncwarp();
     }
     if (p.hist_smem) {
@@ -621,6 +640,7 @@ int dir_totals(const tg_graph *g, const DirParams &d, cudaStream_t s) {
     TG_TRY(tg_edge_units(g, lists->order, M, s, un));
     p.est = est.p;
     p.order = lists->order;
+    p.other = lists->other;
     p.ustart = un.ustart.p;
     const int64_t sms = tg_num_sms();
     if (un.nheavy > 0) {
@@ -636,10 +656,11 @@ int dir_totals(const tg_graph *g, const DirParams &d, cudaStream_t s) {
         p.nunits = un.nheavy;
         p.queue = queue.p;
         const size_t smem = fixed + (size_t)((nbits + 15) / 16) * 4;
-        TG_TRY(tg_allow_max_smem((const void *)k_tri_heavy));
+        const auto fn = nbits >= g->n_nonisolated ? k_tri_heavy<true> : k_tri_heavy<false>;
+        TG_TRY(tg_allow_max_smem((const void *)fn));
         int per = 0;
-        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_tri_heavy, threads, smem));
-        k_tri_heavy<<<(unsigned)std::min<int64_t>(sms * std::max(per, 1), un.nheavy), threads, smem, s>>>(p);
+        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem));
+        fn<<<(unsigned)std::min<int64_t>(sms * std::max(per, 1), un.nheavy), threads, smem, s>>>(p);
         tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
     }

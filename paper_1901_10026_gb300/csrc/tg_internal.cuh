@@ -25,11 +25,12 @@ struct tg_sched;  // per-graph counting schedule (tg_count.cu)
 // Oriented lists of a graph (tg_lists.cu): the up list of node v, its neighbours
 // of smaller id sorted by (type, id), is uadj[uoff[v] .. uoff[v + 1]) with edge
 // ids ueid and type offsets utoff[v (L + 1) ..]; order holds the M edge ids
-// grouped by their end of smaller id j, in j's list order.
+// grouped by their end of smaller id j, in j's list order, and other the packed
+// entries of their other ends.
 struct tg_lists {
     int64_t *uoff = nullptr;
     int32_t *utoff = nullptr;
-    uint32_t *uadj = nullptr, *ueid = nullptr, *order = nullptr;
+    uint32_t *uadj = nullptr, *ueid = nullptr, *order = nullptr, *other = nullptr;
 };
 
 struct tg_graph {
@@ -213,13 +214,13 @@ int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t 
                   const uint32_t *dlow, const unsigned long long *c4w, const unsigned long long *k4,
                   unsigned long long *hist, cudaStream_t s);
 
-// Counts through Alg. 1's typed triangle counts (tg_reuse.cu).  full_order is
+// Counts through Alg. 1's typed triangle counts (tg_reuse.cu).  lists.order is
 // the grouped order of all M edges; order[0..count) the edges to count.  With
 // TG_KERNEL_CYCLES (or AUTO) the per-edge pass is tg_cyc_*, else k_count_reuse.
 // With part.count > 1 (global sums only, k = 4), the call is one share of a
 // split count: order[0..count) is its slice of the edges, and the 4-cycle and
 // 4-clique totals (with their correction of the sums) are the part's own.
-int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_order,
+int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
                    const uint32_t *order, int64_t count, uint64_t *rows, int64_t width,
                    unsigned long long *hist, const tg_tune &t, cudaStream_t s,
                    const tg_part &part = tg_part(), uint64_t *const *rowmap = nullptr);

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) k_oriented_fill(const int64_t *rowptr, co
                                                        const uint32_t *eid, const int32_t *toff,
                                                        const int32_t *utoff, const int64_t *uoff,
                                                        int64_t n, int64_t total, int L, uint32_t *uadj,
-                                                       uint32_t *ueid, uint32_t *order) {
+                                                       uint32_t *ueid, uint32_t *order, uint32_t *other) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; c * kFillChunk < total;
@@ -111,7 +111,9 @@ __global__ void __launch_bounds__(256) k_oriented_fill(const int64_t *rowptr, co
                 ueid[ub + u0 + in] = id;
             } else {
                 const int u1 = __ldg(utoff + w * (L + 1) + t + 1);
-                order[(rb - ub) + (to - u0) + in - (u1 - u0)] = id;
+                const int64_t at = (rb - ub) + (to - u0) + in - (u1 - u0);
+                order[at] = id;
+                other[at] = e;
             }
         }
     }
@@ -124,9 +126,9 @@ int tg_build_lists(const tg_graph *g, tg_lists &out, cudaStream_t s) {
     const int L = g->L;
     DevBuf<int64_t> utot, uoff;
     DevBuf<int32_t> utoff;
-    DevBuf<uint32_t> uadj, ueid, order;
+    DevBuf<uint32_t> uadj, ueid, order, other;
     if (!utot.alloc(n + 1, s) || !uoff.alloc(n + 1, s) || !utoff.alloc((size_t)n * (L + 1), s) ||
-        !uadj.alloc(M, s) || !ueid.alloc(M, s) || !order.alloc(M, s))
+        !uadj.alloc(M, s) || !ueid.alloc(M, s) || !order.alloc(M, s) || !other.alloc(M, s))
         return TG_ENOMEM;
     const int G = L <= 4 ? 4 : L <= 8 ? 8 : 16;
     const unsigned cg = (unsigned)std::min<int64_t>(n / (256 / G) + 1, (int64_t)tg_num_sms() * 64);
@@ -139,7 +141,7 @@ int tg_build_lists(const tg_graph *g, tg_lists &out, cudaStream_t s) {
         const unsigned fg = (unsigned)std::min<int64_t>((2 * M + 8 * kFillChunk - 1) / (8 * kFillChunk),
                                                         (int64_t)tg_num_sms() * 64);
         k_oriented_fill<<<fg, 256, 0, s>>>(g->rowptr, g->adj, g->eid, g->toff, utoff.p, uoff.p, n, 2 * M, L,
-                                           uadj.p, ueid.p, order.p);
+                                           uadj.p, ueid.p, order.p, other.p);
         tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
     }
@@ -148,5 +150,6 @@ int tg_build_lists(const tg_graph *g, tg_lists &out, cudaStream_t s) {
     out.uadj = uadj.release();
     out.ueid = ueid.release();
     out.order = order.release();
+    out.other = other.release();
     return TG_OK;
 }

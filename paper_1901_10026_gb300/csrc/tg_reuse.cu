@@ -30,6 +30,7 @@
 // g4, g5, g9, g11 then follow from Sec. "Combinatorial Relationships" as in
 // the paper.  The counts equal those of Alg. 1-3 exactly; the work drops from
 // sum over w in S_i u S_j u T of d_w to the small side's enumerations.
+#include <algorithm>
 #include <mutex>
 #include <new>
 
@@ -39,7 +40,6 @@ using namespace tgd;
 
 namespace {
 
-constexpr int kTauUnit = 256;  // edges per work unit of the tau kernel
 constexpr int kTCap = 1024;    // T members kept in shared memory for probing
 constexpr int kProbeFactor = 4;
 
@@ -124,25 +124,97 @@ __global__ void k_unit_lists(const uint32_t *flag, const uint32_t *pos, uint32_t
 // Gamma_i \ {j} against it by type.
 // Bits [lo, hi) of a 32-bit word, the range clamped to the word.
 __device__ __forceinline__ uint32_t word_bits(int lo, int hi) {
-    lo = lo < 0 ? 0 : lo;
-    hi = hi > 32 ? 32 : hi;
-    if (lo >= hi) return 0u;
-    const uint32_t up = hi == 32 ? 0xffffffffu : ((1u << hi) - 1u);
-    return up & ~((1u << lo) - 1u);
+    lo = max(lo, 0);
+    uint32_t m;
+    asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(lo), "r"(max(min(hi, 32) - lo, 0)));
+    return m;
 }
 
-constexpr int kTauUnroll = 8;       // chunks of 32 entries in flight per warp
+// A warp takes up to 32 edges of a unit at a time, as far apart as the CTA has warps
+// (neighbouring edges have lists of similar length, the longest first in each type):
+// lane k reads edge k's id, its end i and i's list bounds, so the chain of dependent
+// reads behind an edge is paid once per batch, and the first kTauUnroll chunks of
+// the next edge's list are read before the current edge's are tested.
+// Alg. 1 phase, one edge at a time -> batches (and the tiny edges' kernel below):
+// R-MAT-21 48.7 -> 27.3 ms (5.75e9 entries), CL-1M 6.1 -> 2.9 ms, ER 1M/5M 0.81 ->
+// 0.30 ms.  With consecutive edges in a batch a warp got the longest lists of a type
+// together and R-MAT-21 took 103 ms.  Now bound by instructions (a mask, a shared
+// read and a ballot per 32 entries) and, on small units, by the barriers around them.
+constexpr int kTauUnroll = 8;       // chunks of 32 entries tested and in flight per warp
 constexpr int kTauThreads = 1024;   // one CTA per SM holds the bitmap: 32 warps share it
 
+// Counts the edges q0, q0 + stride, ... (nb <= 32 of them, the same in every lane):
+// test(w) tells whether the entry w of Gamma_i lies in Gamma_j; `none` is an entry
+// for which it does not.
+template <int U, class Test>
+__device__ __forceinline__ void tau_batch(const int64_t *rowptr, const uint32_t *adj, const int32_t *toff,
+                                          const uint32_t *order, const uint32_t *other, uint32_t q0,
+                                          uint32_t stride, int nb, int L, uint32_t none,
+                                          uint32_t *tau, Test test) {
+    const int lane = threadIdx.x & 31;
+    uint32_t e = 0, i = 0;
+    int64_t b = 0;
+    int d = 0;
+    if (lane < nb) {
+        e = __ldg(order + q0 + lane * stride);
+        i = __ldg(other + q0 + lane * stride) & TG_IDMASK;
+        b = __ldg(rowptr + i);
+        d = (int)(__ldg(rowptr + i + 1) - b);
+    }
+    uint32_t wv[U];
+    int64_t bk = __shfl_sync(kFull, b, 0);
+    int dk = __shfl_sync(kFull, d, 0);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int x = 32 * u + lane;
+        wv[u] = x < dk ? __ldg(adj + bk + x) : none;
+    }
+    for (int k = 0; k < nb; ++k) {
+        // lane t < L keeps the count of type t: Gamma_i is sorted by type, so the
+        // hits of type t are the ballot's bits in t's position range
+        const int32_t *toi = toff + (int64_t)__shfl_sync(kFull, i, k) * (L + 1);
+        const int ts0 = lane < L ? __ldg(toi + lane) : 0, ts1 = lane < L ? __ldg(toi + lane + 1) : 0;
+        const int64_t bn = __shfl_sync(kFull, b, k + 1 < nb ? k + 1 : k);
+        const int dn = k + 1 < nb ? __shfl_sync(kFull, d, k + 1) : 0;
+        unsigned mine = 0;
+        for (int c0 = 0; c0 < dk; c0 += 32 * U) {
+            // the next chunks: of this list, or of the next edge's
+            const bool more = c0 + 32 * U < dk;
+            const int64_t nb0 = more ? bk : bn;
+            const int from = more ? c0 + 32 * U : 0, to = more ? dk : dn;
+            uint32_t nx[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int x = from + 32 * u + lane;
+                nx[u] = x < to ? __ldg(adj + nb0 + x) : none;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int cb = c0 + 32 * u;
+                if (u > 0 && cb >= dk) break;
+                const unsigned hm = __ballot_sync(kFull, test(wv[u]));
+                if (lane < L) mine += __popc(hm & word_bits(ts0 - cb, ts1 - cb));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) wv[u] = nx[u];
+        }
+        const int64_t ek = __shfl_sync(kFull, e, k);
+        if (lane < L) tau[ek * L + lane] = mine;
+        bk = bn;
+        dk = dn;
+    }
+}
+
+template <bool kAll>
 __global__ void __launch_bounds__(kTauThreads) k_tau(const int64_t *rowptr, const uint32_t *adj,
                                              const int32_t *toff, const uint8_t *ntype,
-                                             const int2 *edges,
-                                             const uint32_t *order, const uint32_t *ustart,
+                                             const int2 *edges, const uint32_t *order,
+                                             const uint32_t *other, const uint32_t *ustart,
                                              const uint32_t *ulist, uint32_t nunits, int32_t L,
                                              int64_t nbits, unsigned long long *queue,
                                              uint32_t *tau) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, W = blockDim.x >> 5;
     const int64_t bwords = (nbits + 31) >> 5;
     uint32_t *bm = reinterpret_cast<uint32_t *>(smem);
     unsigned long long *s_unit =
@@ -180,41 +252,20 @@ __global__ void __launch_bounds__(kTauThreads) k_tau(const int64_t *rowptr, cons
             cur_dj = dj;
             __syncthreads();
         }
-        for (uint32_t p = p0 + warp; p < p1; p += W) {
-            const uint32_t e = order[p];
-            const int2 ab = edges[e];
-            const int i = max(ab.x, ab.y);
-            const int64_t bi = rowptr[i];
-            const int di = (int)(rowptr[i + 1] - bi);
-            // lane t < L keeps the count of type t: Gamma_i is sorted by type, so
-            // the hits of type t are the ballot's bits in t's position range
-            const int32_t *toi = toff + (int64_t)i * (L + 1);
-            const int ts0 = lane < L ? __ldg(toi + lane) : 0, ts1 = lane < L ? __ldg(toi + lane + 1) : 0;
-            unsigned mine = 0;
-            // kTauUnroll chunks of 32 entries in flight per warp
-            for (int c0 = 0; c0 < di; c0 += 32 * kTauUnroll) {
-                uint32_t wv[kTauUnroll];
-#pragma unroll
-                for (int u = 0; u < kTauUnroll; ++u) {
-                    const int x = c0 + 32 * u + lane;
-                    wv[u] = x < di ? __ldg(adj + bi + x) : 0xffffffffu;
-                }
-#pragma unroll
-                for (int u = 0; u < kTauUnroll; ++u) {
-                    bool hit = false;
-                    const uint32_t w = wv[u];
-                    if (w != 0xffffffffu) {
-                        const uint32_t id = w & TG_IDMASK;
-                        if ((int)id != j)
-                            hit = (int64_t)id < nbits ? bm_test(bm, id)
-                                                      : adjacent(rowptr, adj, toff, L, bj, dj, toj, pj, w);
-                    }
-                    const unsigned hm = __ballot_sync(kFull, hit);
-                    const int cb = c0 + 32 * u;
-                    if (lane < L) mine += __popc(hm & word_bits(ts0 - cb, ts1 - cb));
-                }
-            }
-            if (lane < L) tau[(int64_t)e * L + lane] = mine;
+        // j is no neighbour of itself, so its own entry stands for no entry
+        const uint32_t bits = (uint32_t)nbits;
+        for (uint32_t q = p0 + warp; q < p1; q += 32 * W) {
+            const int nb = (int)min(32u, (p1 - q + W - 1) / W);
+            if (kAll)  // every id that occurs has its bit
+                tau_batch<kTauUnroll>(rowptr, adj, toff, order, other, q, (uint32_t)W, nb, L, pj, tau,
+                                      [&](uint32_t w) -> bool { return bm_test(bm, w & TG_IDMASK); });
+            else
+                tau_batch<kTauUnroll>(rowptr, adj, toff, order, other, q, (uint32_t)W, nb, L, pj, tau,
+                                      [&](uint32_t w) -> bool {
+                                          const uint32_t id = w & TG_IDMASK;
+                                          return id < bits ? bm_test(bm, id)
+                                                           : id != (uint32_t)j && adjacent(rowptr, adj, toff, L, bj, dj, toj, pj, w);
+                                      });
         }
     }
 }
@@ -232,11 +283,13 @@ __global__ void k_tau_adj(const uint32_t *eid, const uint32_t *tau, int64_t entr
 
 // Light units: one warp per unit, Gamma_j (at most TG_LIGHT_DEGREE entries)
 // in a per-warp hash set, the unit's edges one after the other; no CTA barrier.
+// The edges of a j with at most kTauTiny neighbours are left to k_tau_tiny.
 constexpr int kLightWarps = 8;
+constexpr int kTauTiny = 64;
 
 __global__ void __launch_bounds__(kLightWarps * 32) k_tau_light(
     const int64_t *rowptr, const uint32_t *adj, const int32_t *toff, const int2 *edges,
-    const uint32_t *order,
+    const uint32_t *order, const uint32_t *other,
     const uint32_t *ustart, const uint32_t *ulist, uint32_t nlist, int32_t L,
     unsigned long long *queue, uint32_t *tau) {
     __shared__ uint32_t keys[kLightWarps][1 << TG_LIGHT_LG];
@@ -253,18 +306,20 @@ __global__ void __launch_bounds__(kLightWarps * 32) k_tau_light(
         const int j = min(ab0.x, ab0.y);
         const int64_t bj = rowptr[j];
         const int dj = (int)(rowptr[j + 1] - bj);
-        for (int q = lane; q < (1 << TG_LIGHT_LG); q += 32) hk[q] = 0u;
+        int lg = 5;
+        while ((1 << lg) < 2 * dj) ++lg;  // at most TG_LIGHT_LG
+        if (dj <= kTauTiny) break;  // k_tau_tiny's, like all units after it
+        for (int q = lane; q < (1 << lg); q += 32) hk[q] = 0u;
         __syncwarp();
-        for (int x = lane; x < dj; x += 32) hset_put(hk, TG_LIGHT_LG, __ldg(adj + bj + x) & TG_IDMASK);
+        for (int x = lane; x < dj; x += 32) hset_put(hk, lg, __ldg(adj + bj + x) & TG_IDMASK);
         __syncwarp();
         for (uint32_t p = p0; p < p1; ++p) {
             const uint32_t e = order[p];
-            const int2 ab = edges[e];
-            const int i = max(ab.x, ab.y);
+            const int64_t i = __ldg(other + p) & TG_IDMASK;
             const int64_t bi = rowptr[i];
             const int di = (int)(rowptr[i + 1] - bi);
             // lane t < L keeps the count of type t (hits in t's position range)
-            const int32_t *toi = toff + (int64_t)i * (L + 1);
+            const int32_t *toi = toff + i * (L + 1);
             const int ts0 = lane < L ? __ldg(toi + lane) : 0, ts1 = lane < L ? __ldg(toi + lane + 1) : 0;
             unsigned mine = 0;
             for (int c0 = 0; c0 < di; c0 += 32) {
@@ -272,7 +327,7 @@ __global__ void __launch_bounds__(kLightWarps * 32) k_tau_light(
                 bool hit = false;
                 if (x < di) {
                     const uint32_t id = __ldg(adj + bi + x) & TG_IDMASK;
-                    hit = (int)id != j && hset_has(hk, TG_LIGHT_LG, id);
+                    hit = (int)id != j && hset_has(hk, lg, id);
                 }
                 const unsigned hm = __ballot_sync(kFull, hit);
                 if (lane < L) mine += __popc(hm & word_bits(ts0 - c0, ts1 - c0));
@@ -281,6 +336,103 @@ __global__ void __launch_bounds__(kLightWarps * 32) k_tau_light(
         }
         __syncwarp();
     }
+}
+
+// Edges whose end j has at most kTauTiny neighbours: they are the last of the
+// grouped order (ids are degree-ordered).  A warp takes 32 edges, whatever their j,
+// and walks the lists Gamma_i as one sequence, a lane per entry searching the typed
+// range of Gamma_j (a few reads that hit L1); hits are counted in shared memory.
+// With one warp per j and a hash set, the set's build and one 32-lane step per edge
+// were most of the work on lists of ten entries.
+constexpr int kTinyWarps = 8;
+
+__global__ void __launch_bounds__(kTinyWarps * 32) k_tau_tiny(const int64_t *rowptr, const uint32_t *adj,
+                                                              const int32_t *toff, const int2 *edges,
+                                                              const uint32_t *order, const uint32_t *other,
+                                                              const uint32_t *first, int64_t M, int L,
+                                                              uint32_t *tau) {
+    extern __shared__ uint32_t tiny_cnt[];  // [warps][32 L]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *cnt = tiny_cnt + warp * 32 * L;
+    for (int q = lane; q < 32 * L; q += 32) cnt[q] = 0u;
+    __syncwarp();
+    const int64_t p0 = *first, nw = (int64_t)gridDim.x * kTinyWarps;
+    for (int64_t c = (int64_t)blockIdx.x * kTinyWarps + warp; p0 + c * 32 < M; c += nw) {
+        const int64_t p = p0 + c * 32 + lane;
+        uint32_t e = 0;
+        int64_t bi = 0, bj = 0;
+        int di = 0, j = 0;
+        if (p < M) {
+            e = __ldg(order + p);
+            const uint32_t i = __ldg(other + p) & TG_IDMASK;
+            const int2 ab = edges[e];
+            j = min(ab.x, ab.y);
+            bi = __ldg(rowptr + i);
+            di = (int)(__ldg(rowptr + i + 1) - bi);
+            bj = __ldg(rowptr + j);
+        }
+        int incl = di;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int total = __shfl_sync(kFull, incl, 31);
+        const int64_t org = bi - (incl - di);
+        bool any = false;
+        for (int c0 = 0; c0 < total; c0 += 64) {
+            uint32_t w[2];
+            int r[2], jr[2];
+            int64_t by[2];
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                const int pos = c0 + 32 * z + lane;
+                r[z] = 0;  // the edge whose list holds pos
+#pragma unroll
+                for (int st = 16; st > 0; st >>= 1) {
+                    const int v = __shfl_sync(kFull, incl, r[z] + st - 1);
+                    if (v <= pos) r[z] += st;
+                }
+                const int64_t x = __shfl_sync(kFull, org, r[z]) + pos;
+                by[z] = __shfl_sync(kFull, bj, r[z]);
+                jr[z] = __shfl_sync(kFull, j, r[z]);
+                w[z] = pos < total ? __ldg(adj + x) : (uint32_t)jr[z];
+            }
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                if ((int)(w[z] & TG_IDMASK) == jr[z]) continue;
+                if (contains(adj, by[z], toff + (int64_t)jr[z] * (L + 1), w[z])) {
+                    atomicAdd(cnt + r[z] * L + (int)(w[z] >> TG_TSHIFT), 1u);
+                    any = true;
+                }
+            }
+        }
+        any = __any_sync(kFull, any);
+        __syncwarp();
+        const int rows = (int)min((int64_t)32, M - (p0 + c * 32));
+        for (int q = lane; q - lane < rows * L; q += 32) {
+            const int r = min(q / L, 31);
+            const int64_t er = __shfl_sync(kFull, e, r);
+            if (q >= rows * L) continue;
+            tau[er * L + (q - r * L)] = any ? cnt[q] : 0u;
+            if (any) cnt[q] = 0u;
+        }
+        __syncwarp();
+    }
+}
+
+// first[0]: the first position of the grouped order whose j has at most kTauTiny
+// neighbours
+__global__ void k_tau_first(const int64_t *rowptr, const int64_t *uoff, int64_t n, uint32_t *first) {
+    int64_t lo = 0, hi = n;  // the first node of degree <= kTauTiny
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (rowptr[mid + 1] - rowptr[mid] > kTauTiny)
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    first[0] = (uint32_t)(rowptr[lo] - uoff[lo]);
 }
 
 // --------------------------------------------------- per-node aggregates ----
@@ -1023,13 +1175,14 @@ int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStrea
 
 // Runs Alg. 1 for every edge (tau), the per-node sums, then the per-edge
 // counts for the edges order[0..count) (grouped by their high-degree end).
-int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_order,
+int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
                    const uint32_t *order, int64_t count, uint64_t *rows, int64_t width,
                    unsigned long long *hist, const tg_tune &t, cudaStream_t s,
                    const tg_part &part, uint64_t *const *rowmap) {
     if (count <= 0 && part.count <= 1) return TG_OK;  // a share of a split count still enumerates
     const int L = g->L, L2 = L * L;
     const int64_t M = g->M, n = g->n;
+    const uint32_t *const full_order = lists.order;
     unsigned long long *work = nullptr;
     TG_TRY(timing_begin(s, &work));
     // tau for every edge of the graph (the identities need tau of edges
@@ -1052,16 +1205,18 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
             const int64_t maxb = (int64_t)((avail - 64) / 16) * 128;
             if (nbits > maxb) nbits = maxb;
             const size_t smem = ((((size_t)((nbits + 31) >> 5)) * 4 + 15) & ~(size_t)15) + 16;
-            TG_TRY(tg_allow_max_smem((const void *)k_tau));
+            const bool all = nbits >= g->n_nonisolated;
+            const auto fn = all ? k_tau<true> : k_tau<false>;
+            TG_TRY(tg_allow_max_smem((const void *)fn));
             int per_sm = 0;
-            TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tau, kTauThreads, smem));
+            TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kTauThreads, smem));
             if (per_sm < 1) per_sm = 1;
             int64_t grid = (int64_t)tg_num_sms() * per_sm;
             if (grid > (int64_t)un.nheavy) grid = un.nheavy;
             if (grid < 1) grid = 1;
-            k_tau<<<(unsigned)grid, kTauThreads, smem, s>>>(g->rowptr, g->adj, g->toff, g->ntype, g->edges, ord,
-                                                    un.ustart.p, un.heavy.p, un.nheavy, L, nbits,
-                                                    q.p, tau.p); tg_note_launch();
+            fn<<<(unsigned)grid, kTauThreads, smem, s>>>(g->rowptr, g->adj, g->toff, g->ntype, g->edges, ord,
+                                                         lists.other, un.ustart.p, un.heavy.p, un.nheavy, L, nbits,
+                                                         q.p, tau.p); tg_note_launch();
             TG_TRY_CUDA(cudaGetLastError());
         }
         if (un.nlight > 0) {
@@ -1073,8 +1228,25 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const uint32_t *full_ord
             const int64_t need = ((int64_t)un.nlight + kLightWarps - 1) / kLightWarps;
             if (grid > need) grid = need;
             k_tau_light<<<(unsigned)grid, kLightWarps * 32, 0, s>>>(
-                g->rowptr, g->adj, g->toff, g->edges, ord, un.ustart.p, un.light.p, un.nlight, L,
+                g->rowptr, g->adj, g->toff, g->edges, ord, lists.other, un.ustart.p, un.light.p, un.nlight, L,
                 q.p + 1, tau.p); tg_note_launch();
+            TG_TRY_CUDA(cudaGetLastError());
+        }
+    }
+    {
+        DevBuf<uint32_t> first;
+        if (!first.alloc(1, s)) return TG_ENOMEM;
+        k_tau_first<<<1, 1, 0, s>>>(g->rowptr, lists.uoff, n, first.p); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+        const size_t smem = (size_t)kTinyWarps * 32 * L * 4;
+        int per_sm = 0;
+        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tau_tiny, kTinyWarps * 32, smem));
+        const int64_t grid = std::min<int64_t>((int64_t)tg_num_sms() * std::max(per_sm, 1),
+                                               (M + 32 * kTinyWarps - 1) / (32 * kTinyWarps));
+        if (M > 0) {
+            k_tau_tiny<<<(unsigned)grid, kTinyWarps * 32, smem, s>>>(g->rowptr, g->adj, g->toff, g->edges,
+                                                                     lists.order, lists.other, first.p, M, L,
+                                                                     tau.p); tg_note_launch();
             TG_TRY_CUDA(cudaGetLastError());
         }
     }
