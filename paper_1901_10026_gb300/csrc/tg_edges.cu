@@ -14,11 +14,12 @@
 //   G6 = S6 - TSi^T, Y and Z as in tg_reuse.cu; g12 = sym(Q)/2,
 //   g10 = sym(TSi + TSj), g7 = sym(SiSi + SjSj)/2, g6 = sym(G6), g3 = sym(Y),
 //   g8 = sym(Z).
-// k_cyc_edge<true> (units of one j, Gamma_j as a shared-memory bitmap) and
-// k_cyc_tsum_light (light units, Gamma_j in a per-warp hash map) store B, C,
-// DT per edge; k_cyc_finish evaluates the identities per edge from a per-warp
-// table of their L x L terms.  k_cyc_edge<false> does both in one kernel when
-// the T sums would not fit in a quarter of free memory.
+// k_cyc_edge<true> (heavy units of one j, Gamma_j as a shared-memory bitmap)
+// stores B, C, DT per edge.  Rows are finished by k_cyc_rows, which takes the T
+// sums of light edges itself.  Sums over a range of edges go through k_cyc_finish,
+// with k_cyc_tsum_light (light units, Gamma_j in a per-warp hash map) before it.
+// k_cyc_edge<false> does all in one kernel when the T sums would not fit in a
+// quarter of free memory.
 #include <algorithm>
 #include <vector>
 
@@ -665,6 +666,250 @@ __global__ void __launch_bounds__(256) k_cyc_finish(EdgeParams p, int64_t count)
 }
 
 
+// The identities are linear in their ordered L x L terms but for a final halving, and
+// every result takes a term at (t, u) and (u, t) alike, so k_cyc_rows keeps only these
+// combinations: TSi + TSj; SSi + SSj less those; S6 - TSi; Y without the transposed
+// S6 terms that the sum over both orders restores; Z.  Q is the clique row itself.
+enum { RT_TS = 0, RT_SS, RT_G6, RT_Y, RT_Z, RT_N };
+
+__host__ __device__ inline size_t rows_warp_bytes(int LP, int L, size_t term) {
+    const size_t terms = (size_t)((RT_N * L * L + 1) & ~1) * term;
+    return (terms + (size_t)3 * L * L * 8 + (4 * LP + 1) * 4 + 15) & ~(size_t)15;
+}
+
+// Rows of the order positions [p.qbase, p.qbase + count): one warp per edge.  For an
+// edge whose j has at most light_max neighbours the T sums are taken here, from the
+// lists: a lane per entry of Gamma_i searches the typed range of Gamma_j (which the
+// CTA's other edges of j keep in L1), and groups of lanes add the members' three rows
+// to 32-bit sums in shared memory; they fit while a degree is below 2^24.  Edges of a
+// larger j have theirs from k_cyc_edge<true>.
+//
+// Terms are 32-bit (S) while hubs have at most 8,192 neighbours.  Edges of a j beyond
+// 256 neighbours are left to the bitmap of k_cyc_edge<true>: searched as well, the
+// rows of a 960,000-edge power law (hub 36,182, L = 8) took 7.4 ms and not 3.5.
+//
+// Bound by instructions (issue slots 66% busy) and the row stores.  Before, light edges
+// went through a hash map per j, and 3 L^2 64-bit sums per edge were written and read
+// back.  240,000 edges, L = 8, orbit rows (722 MB): 0.675 -> 0.225 ms (3.2 TB/s of
+// rows); the power law's light edges and rows: 1.84 -> 0.95 ms.
+template <int LP, typename S>
+__global__ void __launch_bounds__(256, LP <= 8 ? 3 : 1) k_cyc_rows(EdgeParams p, int64_t count, int light_max) {
+    constexpr int kM = (LP * LP + 31) / 32, kP = (LP * (LP + 1) / 2 + 31) / 32;
+    constexpr int G = LP < 8 ? LP : LP == 8 ? 8 : 16;  // lanes of a member's group
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int L = p.L, P = p.P, L2 = L * L;
+    // per warp: the term table, the T sums (64-bit, or 32-bit when taken here), then
+    // typed degrees of i and j, tau of the edge and the type offsets of j's list
+    S *const xt = reinterpret_cast<S *>(smem + warp * rows_warp_bytes(LP, L, sizeof(S)));
+    unsigned long long *const sum64 = reinterpret_cast<unsigned long long *>(xt + ((RT_N * L2 + 1) & ~1));
+    uint32_t *const sum32 = reinterpret_cast<uint32_t *>(sum64);
+    int *sdi = reinterpret_cast<int *>(sum64 + 3 * L2), *sdj = sdi + LP, *stn = sdj + LP, *soj = stn + LP;
+    constexpr bool kEarly = LP <= 8;  // operands in registers; 6 x 8 entries a lane would spill
+    constexpr int kV = kEarly ? kM : 1;
+    uint32_t mk[kM], pk[kP];  // a | b << 8 | pair << 16 and t | u << 8 of the lane's entries
+#pragma unroll
+    for (int z = 0; z < kM; ++z) {
+        const int a = (lane + 32 * z) / L, b = (lane + 32 * z) % L;
+        mk[z] = a < L ? (uint32_t)(a | b << 8 | pair_index(L, a, b) << 16) : 0u;
+    }
+#pragma unroll
+    for (int z = 0; z < kP; ++z) {
+        int t = 0, u = 0;
+        if (lane + 32 * z < P) unpair(L, lane + 32 * z, t, u);
+        pk[z] = (uint32_t)(t | u << 8);
+    }
+    const int grp = lane / G, gb = lane % G;
+    unsigned long long wk_gamma = 0, wk_t = 0;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    // A lane fetches the ids, types and list bounds of one of the warp's next 32 edges:
+    // three dependent reads once per 32 edges and not before each.
+    int qe = 0, qi = 0, qj = 0, qt = 0, qdi = 0, qdj = 0;
+    int64_t qbi = 0, qbj = 0;
+    int at_lane = 32;
+    for (int64_t r = r0; r < count; r += nw, ++at_lane) {
+        if (at_lane == 32) {
+            at_lane = 0;
+            const int64_t rl = r + lane * nw;
+            if (rl < count) {
+                qe = (int)p.order[p.qbase + rl];
+                const int2 ab = p.edges[qe];
+                qj = min(ab.x, ab.y);
+                qi = max(ab.x, ab.y);
+                qt = p.ntype[qi] | p.ntype[qj] << 8;
+                qbi = p.rowptr[qi];
+                qbj = p.rowptr[qj];
+                qdi = (int)(p.rowptr[qi + 1] - qbi);
+                qdj = (int)(p.rowptr[qj + 1] - qbj);
+            }
+        }
+        const int64_t e = (uint32_t)__shfl_sync(kFull, qe, at_lane);
+        const int i = __shfl_sync(kFull, qi, at_lane), j = __shfl_sync(kFull, qj, at_lane);
+        const int tij = __shfl_sync(kFull, qt, at_lane), ti = tij & 255, tj = tij >> 8;
+        const int64_t bi = __shfl_sync(kFull, qbi, at_lane), bj = __shfl_sync(kFull, qbj, at_lane);
+        const int di = __shfl_sync(kFull, qdi, at_lane), dj = __shfl_sync(kFull, qdj, at_lane);
+        const uint32_t *thi = p.theta + (int64_t)i * L2, *thj = p.theta + (int64_t)j * L2;
+        const uint32_t *dvi = p.dsum + (int64_t)i * L2, *dvj = p.dsum + (int64_t)j * L2;
+        // operands of the terms, in flight while the T sums are taken
+        uint32_t vhi[kV], vhj[kV], vdi[kV], vdj[kV];
+        unsigned long long vq[kV], vc4[kV];
+        if (kEarly && p.k == 4) {
+#pragma unroll
+            for (int z = 0; z < kV; ++z) {
+                const int m = lane + 32 * z;
+                const bool in = m < L2;
+                vhi[z] = in ? __ldg(thi + m) : 0u;
+                vhj[z] = in ? __ldg(thj + m) : 0u;
+                vdi[z] = in ? __ldg(dvi + m) : 0u;
+                vdj[z] = in ? __ldg(dvj + m) : 0u;
+                vc4[z] = in ? __ldg(p.c4e + e * L2 + m) : 0ull;
+                vq[z] = in ? __ldg(p.k4e + e * P + (mk[z] >> 16)) : 0ull;
+            }
+        }
+        uint32_t tn = 0;
+        if (lane < L) {
+            const int32_t *oi = p.toff + (int64_t)i * (L + 1) + lane, *oj = p.toff + (int64_t)j * (L + 1) + lane;
+            const int j0 = __ldg(oj), j1 = __ldg(oj + 1);
+            tn = __ldg(p.tau + e * L + lane);
+            sdi[lane] = __ldg(oi + 1) - __ldg(oi);
+            sdj[lane] = j1 - j0;
+            stn[lane] = (int)tn;
+            soj[lane] = j0;
+            if (lane == L - 1) soj[L] = j1;
+        }
+        uint64_t *const row = p.rowmap ? p.rowmap[e] : p.rows + e * p.width;
+        if (lane < L) {
+            const int64_t si = (int64_t)sdi[lane] - tn - (lane == tj), sj = (int64_t)sdj[lane] - tn - (lane == ti);
+            row[lane] = (uint64_t)(si + sj);
+            row[L + lane] = tn;
+        }
+        if (p.k != 4) continue;
+        const bool light = dj <= light_max;
+        if (light) {
+            for (int x = lane; x < 3 * L2; x += 32) sum32[x] = 0u;
+            int need = (int)__reduce_add_sync(kFull, tn);  // T members left to find
+            __syncwarp();
+            for (int c0 = 0; c0 < di && need > 0; c0 += 32) {
+                const int x = c0 + lane;
+                uint32_t w = 0, at = 0;
+                bool isT = false;
+                if (x < di) {
+                    w = __ldg(p.adj + bi + x);
+                    const int t = (int)(w >> TG_TSHIFT);
+                    if (stn[t] > 0) {  // j itself is not in its own list
+                        int lo = soj[t], hi = soj[t + 1];
+                        const int end = hi;
+                        while (lo < hi) {
+                            const int mid = (lo + hi) >> 1;
+                            if (__ldg(p.adj + bj + mid) < w)
+                                lo = mid + 1;
+                            else
+                                hi = mid;
+                        }
+                        isT = lo < end && __ldg(p.adj + bj + lo) == w;
+                        at = (uint32_t)lo;
+                    }
+                }
+                unsigned tb = __ballot_sync(kFull, isT);
+                need -= __popc(tb);
+                if (lane == 0) {
+                    wk_gamma += min(32, di - c0);
+                    wk_t += __popc(tb);
+                }
+                while (tb) {
+                    // group grp takes the grp-th remaining member
+                    unsigned m = tb;
+#pragma unroll
+                    for (int k = 0; k < 32 / G; ++k) {
+                        if (k < grp) m &= m - 1u;
+                        tb &= tb - 1u;
+                    }
+                    const int src = m ? __ffs(m) - 1 : 0;
+                    const uint32_t wy = __shfl_sync(kFull, w, src), ay = __shfl_sync(kFull, at, src);
+                    if (m && gb < L) {
+                        const int32_t *ty = p.toff + (int64_t)(wy & TG_IDMASK) * (L + 1) + gb;
+                        const uint32_t vb = __ldg(p.tau_adj + (bj + ay) * L + gb);
+                        const uint32_t vc = __ldg(p.tau_adj + (bi + c0 + src) * L + gb);
+                        const uint32_t vd = (uint32_t)(__ldg(ty + 1) - __ldg(ty));
+                        const int k = (int)(wy >> TG_TSHIFT) * L + gb;
+                        if (vb) atomicAdd(sum32 + k, vb);
+                        if (vc) atomicAdd(sum32 + L2 + k, vc);
+                        if (vd) atomicAdd(sum32 + 2 * L2 + k, vd);
+                    }
+                }
+            }
+        } else {
+            const unsigned long long *src = p.tsum + r * 3 * L2;
+            for (int x = lane; x < 3 * L2; x += 32) sum64[x] = __ldg(src + x);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int z = 0; z < kM; ++z) {
+            const int m = lane + 32 * z, a = mk[z] & 255u, b = mk[z] >> 8 & 255u;
+            if (m >= L2) continue;
+            const S Bv = light ? (S)sum32[m] : (S)sum64[m];
+            const S Cv = light ? (S)sum32[L2 + m] : (S)sum64[L2 + m];
+            const S Dv = light ? (S)sum32[2 * L2 + m] : (S)sum64[2 * L2 + m];
+            S q = (S)(kEarly ? vq[z % kV] : __ldg(p.k4e + e * P + (mk[z] >> 16)));
+            if (a == b) q *= 2;
+            const S na = stn[a], nb = stn[b];
+            const S tsi = Cv - q - (b == tj ? na : 0), tsj = Bv - q - (b == ti ? na : 0);
+            const S ss = (S)(kEarly ? vhi[z % kV] : __ldg(thi + m)) - Cv - (a == tj ? nb : 0) +
+                         (S)(kEarly ? vhj[z % kV] : __ldg(thj + m)) - Bv - (a == ti ? nb : 0);
+            const S ds = (S)(kEarly ? vdi[z % kV] : __ldg(dvi + m)) + (S)(kEarly ? vdj[z % kV] : __ldg(dvj + m)) -
+                         2 * Dv - (a == tj ? sdj[b] : 0) - (a == ti ? sdi[b] : 0);
+            const S sia = sdi[a] - na - (a == tj), sja = sdj[a] - na - (a == ti);
+            const S g6 = (S)(kEarly ? vc4[z % kV] : __ldg(p.c4e + e * L2 + m)) - Bv + (b == ti ? na : 0) - tsi;
+            xt[RT_TS * L2 + m] = tsi + tsj;
+            xt[RT_SS * L2 + m] = ss - tsi - tsj;
+            xt[RT_G6 * L2 + m] = g6;
+            xt[RT_Y * L2 + m] = ds - (b == ti ? sia : 0) - (b == tj ? sja : 0) - ss - 2 * g6;
+            xt[RT_Z * L2 + m] = Dv - na * ((b == ti) + (b == tj)) - q - tsi - tsj;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int z = 0; z < kP; ++z) {
+            const int pr = lane + 32 * z, t = pk[z] & 255u, u = pk[z] >> 8;
+            if (pr >= P) continue;
+            const int m = t * L + u, mt = u * L + t;
+            auto sym = [&](int x) -> S { return t == u ? xt[x * L2 + m] : xt[x * L2 + m] + xt[x * L2 + mt]; };
+            const S tt = stn[t], tu = stn[u];
+            const S sit = sdi[t] - tt - (t == tj), siu = sdi[u] - tu - (u == tj);
+            const S sjt = sdj[t] - tt - (t == ti), sju = sdj[u] - tu - (u == ti);
+            const S g3 = sym(RT_Y), g6 = sym(RT_G6), g7 = sym(RT_SS) / 2, g8 = sym(RT_Z), g10 = sym(RT_TS);
+            const S g12 = (S)__ldg(p.k4e + e * P + pr);
+            S g4, g5, g9, g11;
+            if (t == u) {
+                g4 = sit * sjt - g6;
+                g5 = (sit * (sit - 1) + sjt * (sjt - 1)) / 2 - g7;
+                g9 = tt * (sit + sjt) - g10;
+                g11 = tt * (tt - 1) / 2 - g12;
+            } else {
+                g4 = sit * sju + siu * sjt - g6;
+                g5 = sit * siu + sjt * sju - g7;
+                g9 = tt * (siu + sju) + tu * (sit + sjt) - g10;
+                g11 = tt * tu - g12;
+            }
+            uint64_t *o = row + 2 * L + pr;
+            if (p.level == TG_ORBIT) {
+                const S g[10] = {g3, g4, g5, g6, g7, g8, g9, g10, g11, g12};
+#pragma unroll
+                for (int x = 0; x < 10; ++x) o[x * P] = (uint64_t)g[x];
+            } else {
+                const S g[6] = {g3 + g4, g5, g6, g7 + g8 + g9, g10 + g11, g12};
+#pragma unroll
+                for (int x = 0; x < 6; ++x) o[x * P] = (uint64_t)g[x];
+            }
+        }
+        __syncwarp();  // the warp's tables are rewritten by the next edge
+    }
+    if (p.work && lane == 0) {
+        if (wk_gamma) atomicAdd(p.work + 0, wk_gamma);
+        if (wk_t) atomicAdd(p.work + 3, wk_t);
+    }
+}
+
 int num_sms_e() {
     int dev = 0, sms = 0;
     (void)cudaGetDevice(&dev);
@@ -751,8 +996,34 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
     const size_t row_bytes = (size_t)3 * L2 * 8;
     size_t free_b = 0, total_b = 0;
     TG_TRY_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    // rows (k = 4 from per-edge counters): k_cyc_rows finishes the edges and takes the
+    // T sums of light ones; without T sums (k = 3) it needs nothing before it
+    const bool row_mode = (rows || rowmap) && t.edge_pass != TG_EDGE_PASS_FUSED;
+    const int light_max = row_mode && g->max_degree < ((int64_t)1 << 24) ? TG_LIGHT_DEGREE : -1;
+    const bool narrow = g->max_degree <= 8192;  // every term below 8 x 8192^2 < 2^31
+    void (*const rows_fn)(EdgeParams, int64_t, int) =
+        L <= 4   ? (narrow ? k_cyc_rows<4, int> : k_cyc_rows<4, long long>)
+        : L <= 8 ? (narrow ? k_cyc_rows<8, int> : k_cyc_rows<8, long long>)
+                 : (narrow ? k_cyc_rows<16, int> : k_cyc_rows<16, long long>);
+    const size_t rsmem = 8 * rows_warp_bytes(L <= 4 ? 4 : L <= 8 ? 8 : 16, L, narrow ? 4 : 8);
+    int rper = 0;
+    if (row_mode) {
+        TG_TRY(tg_allow_max_smem((const void *)rows_fn));
+        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rper, rows_fn, 256, rsmem));
+        if (rper < 1) rper = 1;
+    }
+    auto launch_rows = [&](const EdgeParams &rp, int64_t nq) -> int {
+        int64_t rgrid = std::min<int64_t>((int64_t)num_sms_e() * rper, (nq + 7) / 8);
+        if (t.grid_limit > 0 && rgrid > t.grid_limit) rgrid = t.grid_limit;
+        if (rgrid < 1) rgrid = 1;
+        rows_fn<<<(unsigned)rgrid, 256, rsmem, s>>>(rp, nq, light_max); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+        return TG_OK;
+    };
+    if (row_mode && k != 4) return launch_rows(p, count);
     bool split = k == 4 && t.edge_pass != TG_EDGE_PASS_FUSED;
-    int64_t qcap = std::min<int64_t>(count, (int64_t)(free_b / 4 / row_bytes));
+    const bool sums = un.nheavy > 0 || light_max < 0;  // some sums go through memory
+    int64_t qcap = sums ? std::min<int64_t>(count, (int64_t)(free_b / 4 / row_bytes)) : count;
     if (t.edge_batch > 0 && qcap > t.edge_batch) qcap = t.edge_batch;
     // batches [bu[x], bu[x + 1]) of units, with their heavy and light sub-lists
     std::vector<uint32_t> bu{0u, un.nunits}, bh{0u, un.nheavy}, bl{0u, un.nlight};
@@ -813,7 +1084,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
     const size_t smem = fixed + ((((size_t)((nbits + 31) >> 5)) * 4 + 15) & ~(size_t)15);
     DevBuf<unsigned long long> queue, tsum;
     if (!queue.alloc(2, s)) return TG_ENOMEM;
-    if (split && !tsum.alloc((size_t)(bu.size() > 2 ? qcap : count) * 3 * L2, s)) return TG_ENOMEM;
+    if (split && sums && !tsum.alloc((size_t)(bu.size() > 2 ? qcap : count) * 3 * L2, s)) return TG_ENOMEM;
     p.tsum = tsum.p;
     const void *kfn = split ? (const void *)k_cyc_edge<true> : (const void *)k_cyc_edge<false>;
     TG_TRY(tg_allow_max_smem(kfn));
@@ -875,7 +1146,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
         lp.hist_smem = 0;
         lp.ulist = un.light.p + bl[x];
         lp.nunits = bl[x + 1] - bl[x];
-        if (lp.nunits > 0) {
+        if (lp.nunits > 0 && light_max < 0) {
             TG_TRY_CUDA(cudaMemsetAsync(queue.p + 1, 0, 8, s));
             lp.queue = queue.p + 1;
             int64_t lgrid = (int64_t)num_sms_e() * lper;
@@ -886,6 +1157,10 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
             TG_TRY_CUDA(cudaGetLastError());
         }
         // finishing pass: warp per edge
+        if (row_mode) {
+            TG_TRY(launch_rows(p, nq));
+            continue;
+        }
         EdgeParams fp = p;
         fp.hist_smem = hist_smem;
         int64_t fgrid = (int64_t)num_sms_e() * fper;
