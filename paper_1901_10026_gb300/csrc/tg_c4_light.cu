@@ -167,18 +167,18 @@ struct LightParams {
 // anchor a: op(ok, entry b of u's list, its position, member x of Gamma_a,
 // entry u), called by all lanes, ok where b ranks below a; kWalkBatch batches
 // of 32 positions in flight.
-constexpr int kWalkBatch = 2;
+constexpr int kWalkBatch = 4;
 
 template <class Op>
 __device__ __forceinline__ void light_walk(const LightParams &p, uint32_t a, int64_t ba, int da,
-                                           int m0, int stride, Op op) {
+                                           int m0, int stride, int step, Op op) {
     const int lane = threadIdx.x & 31;
     for (int m = m0; m < da; m += stride) {
         const int x = m + lane;
         uint32_t wu = 0;
         int64_t bu = 0;
         int len = 0;
-        if (x < da) {
+        if (lane < step && x < da) {
             wu = __ldg(p.adj + ba + x);
             const uint32_t u = wu & TG_IDMASK;
             if (u > a) {
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kLightWarps * 32) k_c4_warp(LightParams p) {
             int lg = 5;
             while ((1ull << lg) <= ca) ++lg;  // at most lg_max: cost < 2^lg_max
             int nl = 0;  // claimed slots
-            light_walk(p, a, ba, da, 0, 32, [&](bool ok, uint32_t wb, int64_t, int, uint32_t wu) {
+            light_walk(p, a, ba, da, 0, 32, 32, [&](bool ok, uint32_t wb, int64_t, int, uint32_t wu) {
                 bool isnew = false;
                 int h = 0;
                 if (ok) {
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kLightWarps * 32) k_c4_warp(LightParams p) {
             });
             __syncwarp();
             if (kEdge) {
-                light_walk(p, a, ba, da, 0, 32, [&](bool ok, uint32_t wb, int64_t at, int x, uint32_t wu) {
+                light_walk(p, a, ba, da, 0, 32, 32, [&](bool ok, uint32_t wb, int64_t at, int x, uint32_t wu) {
                     if (ok) wedge_edges(p, tab, lg, ta, ba, wb, at, x, wu);
                 });
                 __syncwarp();
@@ -417,6 +417,7 @@ __global__ void __launch_bounds__(1024) k_c4_cta(LightParams p) {
     tab.place(smem + (kEdge ? 0 : ((size_t)p.n4 * 8 + 15) & ~(size_t)15), L, p.lg_max);
     for (int q = tid; q < (1 + tab.words) << p.lg_max; q += blockDim.x) tab.keys[q] = 0u;
     unsigned long long wk = 0;
+    const int nwarps = blockDim.x >> 5;
     for (;;) {
         __syncthreads();
         if (tid == 0) {
@@ -431,9 +432,10 @@ __global__ void __launch_bounds__(1024) k_c4_cta(LightParams p) {
         const int da = (int)(p.rowptr[a + 1] - ba);
         const int ta = p.ntype[a];
         const unsigned long long ca = p.cost[a];
+        const int step = max(4, min(32, (da + nwarps - 1) / nwarps));  // members a warp takes at once
         int lg = 5;
         while ((1ull << lg) <= ca) ++lg;
-        light_walk(p, a, ba, da, 32 * warp, blockDim.x, [&](bool ok, uint32_t wb, int64_t, int, uint32_t wu) {
+        light_walk(p, a, ba, da, step * warp, step * nwarps, step, [&](bool ok, uint32_t wb, int64_t, int, uint32_t wu) {
             bool isnew = false;
             int h = 0;
             if (ok) {
@@ -450,7 +452,7 @@ __global__ void __launch_bounds__(1024) k_c4_cta(LightParams p) {
         });
         __syncthreads();
         if (kEdge) {
-            light_walk(p, a, ba, da, 32 * warp, blockDim.x,
+            light_walk(p, a, ba, da, step * warp, step * nwarps, step,
                        [&](bool ok, uint32_t wb, int64_t at, int x, uint32_t wu) {
                            if (ok) wedge_edges(p, tab, lg, ta, ba, wb, at, x, wu);
                        });
