@@ -438,13 +438,11 @@ __global__ void k_tau_first(const int64_t *rowptr, const int64_t *uoff, int64_t 
 // --------------------------------------------------- per-node aggregates ----
 // Theta_v[a][b] = sum over w in Gamma_v^a of tau_vw[b]; D_v[a][b] = sum of
 // d_w^b, or (kLow, for the whole-graph totals of tg_sums.cu) the sum of
-// d_w^b - [b = phi_v] over the w of larger id only.  Nodes of degree up to dsmall: one thread per node, its 2 L^2 sums in
-// a private column of shared memory (k_node_aggr_small).  Larger nodes: their
+// d_w^b - [b = phi_v] over the w of larger id only.  Nodes of degree up to
+// dsmall: a group of lanes per typed range (k_node_aggr_small).  Larger nodes: their
 // typed ranges are cut into chunks of at most kAggrChunk entries, one warp per
 // chunk, whose sums are added to the (zeroed) rows (k_node_aggr).
-constexpr int kAggrSmall = 64;        // degree bound of the one-thread nodes
-constexpr int kAggrSmallMaxL = 8;     // types up to which they are used
-constexpr int kAggrSmallThreads = 128;
+constexpr int kAggrSmall = 64;  // degree bound of the lane groups
 constexpr int kAggrChunk = 2048;
 
 // chunks of node v's typed ranges (0 for a node left to the one-thread kernel)
@@ -461,37 +459,50 @@ __global__ void k_aggr_chunks(const int64_t *rowptr, const int32_t *toff, int64_
     }
 }
 
-template <bool kLow>
-__global__ void __launch_bounds__(kAggrSmallThreads)
+// A group of G >= L lanes per node and type a, lane b on column b: the entries of the
+// typed range are read four at a time, their tau and offset rows side by side, and the
+// sums stay in registers.  Rows of larger nodes are set to zero.
+//
+// Bound by the latency of the gathers.  Before, a thread per node kept its 2 L^2 sums in
+// a column of shared memory, one entry at a time (and L > 8 took a warp per node):
+// ER 100K/1M (L = 5) 0.268 -> 0.053 ms, an 8M-edge power law's small nodes 1.2 -> 0.37.
+template <int G, bool kLow>
+__global__ void __launch_bounds__(256)
     k_node_aggr_small(const int64_t *rowptr, const uint32_t *adj, const uint32_t *eid,
                       const int32_t *toff, const uint8_t *ntype, const uint32_t *tau, int64_t n,
                       int32_t L, int dsmall, uint32_t *theta, uint32_t *dsum) {
-    extern __shared__ uint32_t col[];  // [2 L^2][blockDim.x]
-    const int tid = threadIdx.x, bd = blockDim.x;
-    const int L2 = L * L;
-    for (int64_t v = blockIdx.x * (int64_t)bd + tid; v < n; v += (int64_t)gridDim.x * bd) {
-        const int64_t rb = rowptr[v], re = rowptr[v + 1];
-        if (re - rb > dsmall) continue;  // a warp of k_node_aggr takes it
-        for (int q = 0; q < 2 * L2; ++q) col[q * bd + tid] = 0u;
-        const int tv = kLow ? ntype[v] : -1;
-        for (int64_t x = rb; x < re; ++x) {
-            const uint32_t wu = __ldg(adj + x);
-            const int a = (int)(wu >> TG_TSHIFT);
-            const bool deg = !kLow || (int64_t)(wu & TG_IDMASK) > v;
-            const uint32_t *tw = tau + (int64_t)__ldg(eid + x) * L;
-            const int32_t *ow = toff + (int64_t)(wu & TG_IDMASK) * (L + 1);
-            int prev = __ldg(ow);
-            for (int b = 0; b < L; ++b) {
-                const int nx = __ldg(ow + b + 1);
-                col[(a * L + b) * bd + tid] += __ldg(tw + b);
-                if (deg) col[(L2 + a * L + b) * bd + tid] += (uint32_t)(nx - prev - (kLow && b == tv));
-                prev = nx;
+    const int b = threadIdx.x % G;
+    const int64_t items = n * L, ng = (int64_t)gridDim.x * (256 / G);
+    if (b >= L) return;
+    for (int64_t it = (int64_t)blockIdx.x * (256 / G) + threadIdx.x / G; it < items; it += ng) {
+        const uint32_t v = (uint32_t)it / (uint32_t)L;  // n < 2^28 and L <= 16
+        const int a = (int)((uint32_t)it - v * (uint32_t)L);
+        const int64_t rb = __ldg(rowptr + v);
+        const int32_t *tv = toff + (int64_t)v * (L + 1) + a;
+        const int deg = (int)(__ldg(rowptr + v + 1) - rb);
+        const int s0 = __ldg(tv), s1 = deg > dsmall ? s0 : __ldg(tv + 1);
+        const bool own = kLow && b == __ldg(ntype + v);
+        uint32_t st = 0, sd = 0;
+        for (int x = s0; x < s1; x += 4) {
+            uint32_t w[4], e[4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int64_t at = rb + min(x + y, s1 - 1);
+                w[y] = __ldg(adj + at) & TG_IDMASK;
+                e[y] = __ldg(eid + at);
+            }
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const int32_t *ow = toff + (int64_t)w[y] * (L + 1) + b;
+                const uint32_t tw = __ldg(tau + (int64_t)e[y] * L + b);
+                const uint32_t dw = (uint32_t)(__ldg(ow + 1) - __ldg(ow)) - own;
+                if (x + y >= s1) continue;
+                st += tw;
+                if (!kLow || w[y] > v) sd += dw;
             }
         }
-        for (int q = 0; q < L2; ++q) {
-            theta[v * L2 + q] = col[q * bd + tid];
-            dsum[v * L2 + q] = col[(L2 + q) * bd + tid];
-        }
+        theta[it * L + b] = st;
+        dsum[it * L + b] = sd;
     }
 }
 
@@ -1081,24 +1092,19 @@ int timing_begin(cudaStream_t s, unsigned long long **work) {
 template <bool kLow>
 int node_sums(const tg_graph *g, const uint32_t *tau, uint32_t *theta, uint32_t *dsum,
               cudaStream_t s) {
-    const int L = g->L, L2 = L * L;
+    const int L = g->L, dsmall = kAggrSmall;
     const int64_t n = g->n;
-    const int dsmall = L <= kAggrSmallMaxL ? kAggrSmall : -1;
-    // rows of the chunked nodes start at zero
-    TG_TRY_CUDA(cudaMemsetAsync(theta, 0, (size_t)n * L2 * 4, s));
-    TG_TRY_CUDA(cudaMemsetAsync(dsum, 0, (size_t)n * L2 * 4, s));
-    if (dsmall >= 0) {
-        const size_t asmem = (size_t)2 * L2 * kAggrSmallThreads * 4;
-        TG_TRY(tg_allow_max_smem((const void *)k_node_aggr_small<kLow>));
-        int per = 0;
-        TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_node_aggr_small<kLow>,
-                                                                  kAggrSmallThreads, asmem));
-        const int64_t ag = std::min<int64_t>((int64_t)tg_num_sms() * (per > 0 ? per : 1),
-                                             (n + kAggrSmallThreads - 1) / kAggrSmallThreads);
-        k_node_aggr_small<kLow><<<(unsigned)std::max<int64_t>(ag, 1), kAggrSmallThreads, asmem, s>>>(
-            g->rowptr, g->adj, g->eid, g->toff, g->ntype, tau, n, L, dsmall, theta, dsum); tg_note_launch();
-        TG_TRY_CUDA(cudaGetLastError());
-    }
+    const int G = L == 1 ? 1 : L == 2 ? 2 : L <= 4 ? 4 : L <= 8 ? 8 : 16;
+    auto small = G == 1   ? k_node_aggr_small<1, kLow>
+                 : G == 2 ? k_node_aggr_small<2, kLow>
+                 : G == 4 ? k_node_aggr_small<4, kLow>
+                 : G == 8 ? k_node_aggr_small<8, kLow>
+                          : k_node_aggr_small<16, kLow>;
+    const int64_t ag = std::min<int64_t>((int64_t)tg_num_sms() * 64, (n * L * G + 255) / 256);
+    small<<<(unsigned)std::max<int64_t>(ag, 1), 256, 0, s>>>(g->rowptr, g->adj, g->eid, g->toff, g->ntype, tau, n,
+                                                             L, dsmall, theta, dsum);
+    tg_note_launch();
+    TG_TRY_CUDA(cudaGetLastError());
     DevBuf<uint32_t> nch, cpos;
     if (!nch.alloc(n, s) || !cpos.alloc(n, s)) return TG_ENOMEM;
     k_aggr_chunks<<<grid_r(n), 256, 0, s>>>(g->rowptr, g->toff, n, L, dsmall, nch.p); tg_note_launch();

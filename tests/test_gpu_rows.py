@@ -7,6 +7,7 @@ import pytest
 
 import oracle
 import paper_1901_10026_gb300 as tg
+from oracle import o2
 
 pytestmark = pytest.mark.gpu
 
@@ -19,6 +20,7 @@ def _built():
     from paper_1901_10026_gb300 import build
     build.build()
     oracle.build()
+    o2.build()
     yield
     tg.tg_set_tune(reset=True)
 
@@ -53,4 +55,26 @@ def test_rows_against_fused_and_oracle(deg, L):
             bad = np.argwhere(got != want)
             assert bad.shape[0] == 0, (k, level, tune, bad[:5])
         assert np.array_equal(got[e], og.per_edge(k, name, edges=e))
+    tg.tg_set_tune(reset=True)
+
+
+def _star_of_types(deg, L):
+    """A node with `deg` neighbours spread over L types, joined in a ring."""
+    ring = np.arange(1, deg + 1)
+    src = np.concatenate([np.zeros(deg, np.int64), ring[:-1]]).astype(np.int32)
+    dst = np.concatenate([ring, ring[1:]]).astype(np.int32)
+    return deg + 1, src, dst, (np.arange(deg + 1) * 7 % 11 % L).astype(np.uint8)
+
+
+@pytest.mark.parametrize("L", [1, 2, 3, 4, 5, 8, 9, 16])
+@pytest.mark.parametrize("deg", [3, 31, 63, 64, 65, 300])
+def test_node_sums_around_the_degree_bound(deg, L):
+    """Theta and D by lane groups up to 64 neighbours, by warps beyond (global and rows)."""
+    n, src, dst, types = _star_of_types(deg, L)
+    g = tg.tg_build_csr(n, src, dst, types, L)
+    og = oracle.OracleGraph(n, src, dst, types, L)
+    tg.tg_set_tune(kernel=tg.TG_KERNEL_CYCLES)
+    rows = tg.tg_count_per_edge(g, 4, tg.TG_ORBIT)
+    assert np.array_equal(rows, og.per_edge(4, "orbit"))
+    assert np.array_equal(tg.tg_count_global(g, 4), o2.global_counts(n, src, dst, types, L, 4))
     tg.tg_set_tune(reset=True)
