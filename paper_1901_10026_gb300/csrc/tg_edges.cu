@@ -938,6 +938,13 @@ __global__ void k_typed_degrees(const int32_t *toff, int64_t n, uint32_t *tdeg) 
 }
 }  // namespace
 
+// Rows need units for heavy edges, and to cut batches of edges; sums over a range and
+// the fused kernel run on units throughout.
+bool tg_cyc_edges_units(const tg_graph *g, int64_t count, bool rows, const tg_tune &t) {
+    return !rows || t.edge_pass == TG_EDGE_PASS_FUSED || g->max_degree > TG_LIGHT_DEGREE ||
+           (t.edge_batch > 0 && t.edge_batch < count);
+}
+
 int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int64_t count,
                  const tg_units &un, uint64_t *rows, int64_t width,
                  unsigned long long *hist, const uint32_t *tau, const uint32_t *tau_adj,
@@ -945,7 +952,7 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
                  const uint32_t *dsum, const unsigned long long *c4e,
                  const unsigned long long *k4e, unsigned long long *work, const tg_tune &t,
                  cudaStream_t s, uint64_t *const *rowmap) {
-    if (un.nunits == 0 || count <= 0) return TG_OK;
+    if (count <= 0) return TG_OK;
     const int L = g->L, L2 = L * L;
     if (g->max_degree >= ((int64_t)1 << 27)) return TG_EOVERFLOW;  // 32-lane uint32 sums
     EdgeParams p{};

@@ -199,6 +199,8 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
                    unsigned long long *work, const tg_tune &t, const tg_part &part, cudaStream_t s);
 int tg_cyc_correct(unsigned long long *hist, int L, const unsigned long long *c4w,
                    const unsigned long long *k4, cudaStream_t s);
+// whether tg_cyc_edges wants the units of its edges (an empty tg_units serves otherwise)
+bool tg_cyc_edges_units(const tg_graph *g, int64_t count, bool rows, const tg_tune &t);
 int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int64_t count,
                  const tg_units &un, uint64_t *rows, int64_t width,
                  unsigned long long *hist, const uint32_t *tau, const uint32_t *tau_adj,

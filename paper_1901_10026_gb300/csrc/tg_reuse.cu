@@ -88,34 +88,42 @@ __global__ void k_unit_flags(const uint32_t *order, const int2 *edges, int64_t c
     }
 }
 
-__global__ void k_unit_starts(const uint32_t *flag, const uint32_t *pos, int64_t count,
-                              uint32_t *ustart, uint32_t nunits) {
+// out: the number of units, and of heavy ones.  The order is ascending in j and ids
+// descend in degree, so the heavy units are a prefix: one warp finds the first edge
+// whose j has at most TG_LIGHT_DEGREE neighbours, 32 probes to a step.
+__global__ void k_unit_counts(const uint32_t *order, const int2 *edges, const int64_t *rowptr,
+                              int64_t count, const uint32_t *flag, const uint32_t *pos, uint32_t *out) {
+    const int lane = threadIdx.x;
+    int64_t lo = 0, hi = count;  // the edge lies in [lo, hi]
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) / 32, p = lo + lane * step;
+        bool heavy = false;
+        if (p < hi) {
+            const int2 ab = edges[order[p]];
+            const int j = min(ab.x, ab.y);
+            heavy = rowptr[j + 1] - rowptr[j] > TG_LIGHT_DEGREE;
+        }
+        const int k = __popc(__ballot_sync(kFull, heavy));  // heavy probes come first
+        hi = min(hi, lo + k * step);
+        lo = k ? lo + (k - 1) * step + 1 : hi;
+    }
+    if (lane == 0) {
+        out[0] = pos[count - 1] + flag[count - 1];
+        out[1] = lo < count ? pos[lo] : out[0];
+    }
+}
+
+__global__ void k_unit_lists(const uint32_t *flag, const uint32_t *pos, int64_t count, uint32_t nunits,
+                             uint32_t nheavy, uint32_t *ustart, uint32_t *heavy, uint32_t *light) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < count;
-         p += (int64_t)gridDim.x * blockDim.x)
+         p += (int64_t)gridDim.x * blockDim.x) {
         if (flag[p]) ustart[pos[p]] = (uint32_t)p;
+        if (p < nheavy)
+            heavy[p] = (uint32_t)p;
+        else if (p < nunits)
+            light[p - nheavy] = (uint32_t)p;
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) ustart[nunits] = (uint32_t)count;
-}
-
-// flag[u] = unit u's j has at most TG_LIGHT_DEGREE neighbours
-__global__ void k_unit_class(const uint32_t *order, const int2 *edges, const int64_t *rowptr,
-                             const uint32_t *ustart, uint32_t nunits, uint32_t *flag) {
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < nunits;
-         u += (int64_t)gridDim.x * blockDim.x) {
-        const int2 ab = edges[order[ustart[u]]];
-        const int j = min(ab.x, ab.y);
-        flag[u] = (rowptr[j + 1] - rowptr[j]) <= TG_LIGHT_DEGREE ? 1u : 0u;
-    }
-}
-
-__global__ void k_unit_lists(const uint32_t *flag, const uint32_t *pos, uint32_t nunits,
-                             uint32_t *light, uint32_t *heavy) {
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < nunits;
-         u += (int64_t)gridDim.x * blockDim.x) {
-        if (flag[u])
-            light[pos[u]] = (uint32_t)u;
-        else
-            heavy[u - pos[u]] = (uint32_t)u;
-    }
 }
 
 // ------------------------------------------------------------ tau (Alg. 1) --
@@ -356,7 +364,7 @@ __global__ void __launch_bounds__(kTinyWarps * 32) k_tau_tiny(const int64_t *row
     uint32_t *cnt = tiny_cnt + warp * 32 * L;
     for (int q = lane; q < 32 * L; q += 32) cnt[q] = 0u;
     __syncwarp();
-    const int64_t p0 = *first, nw = (int64_t)gridDim.x * kTinyWarps;
+    const int64_t p0 = first ? *first : 0, nw = (int64_t)gridDim.x * kTinyWarps;
     for (int64_t c = (int64_t)blockIdx.x * kTinyWarps + warp; p0 + c * 32 < M; c += nw) {
         const int64_t p = p0 + c * 32 + lane;
         uint32_t e = 0;
@@ -1137,7 +1145,10 @@ int launch_reuse_u(const ReuseParams &p, int threads, size_t smem, int grid_limi
 
 }  // namespace
 
-// Work units of the grouped order (see k_unit_flags), split by class.
+// Work units of the grouped order (see k_unit_flags), the heavy ones first.  Made only
+// for a graph or a pass that has use for them, with one wait for their number: with
+// the classes flagged, scanned and listed on the device, and a second wait, ER 1000
+// took 650 us and not 532, ER 1M/5M at k = 3 2.94 ms and not 2.54
 int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStream_t s,
                tg_units &un) {
     DevBuf<uint32_t> flag, pos, gs, ge;
@@ -1151,31 +1162,22 @@ int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStrea
     k_unit_flags<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, cnt, gs.p, ge.p, cum.p, flag.p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     TG_TRY(tg_scan_u32(flag.p, pos.p, cnt, s));
-    uint32_t lastp = 0, lastf = 0;
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastp, pos.p + cnt - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastf, flag.p + cnt - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaStreamSynchronize(s));
-    un.nunits = lastp + lastf;
-    if (!un.ustart.alloc((size_t)un.nunits + 1, s)) return TG_ENOMEM;
-    k_unit_starts<<<grid_r(cnt), 256, 0, s>>>(flag.p, pos.p, cnt, un.ustart.p, un.nunits); tg_note_launch();
+    DevBuf<uint32_t> num;
+    if (!num.alloc(2, s)) return TG_ENOMEM;
+    k_unit_counts<<<1, 32, 0, s>>>(ord, g->edges, g->rowptr, cnt, flag.p, pos.p, num.p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
-    // classes: light (one warp each) and heavy (one CTA each)
-    DevBuf<uint32_t> cflag, cpos;
-    if (!cflag.alloc(un.nunits, s) || !cpos.alloc(un.nunits, s) ||
-        !un.light.alloc(un.nunits, s) || !un.heavy.alloc(un.nunits, s))
+    uint32_t h[2] = {0, 0};
+    TG_TRY_CUDA(cudaMemcpyAsync(h, num.p, sizeof h, cudaMemcpyDeviceToHost, s));
+    TG_TRY_CUDA(cudaStreamSynchronize(s));
+    un.nunits = h[0];
+    un.nheavy = h[1];
+    un.nlight = h[0] - h[1];
+    if (!un.ustart.alloc((size_t)un.nunits + 1, s) || !un.light.alloc(un.nunits, s) ||
+        !un.heavy.alloc(un.nunits, s))
         return TG_ENOMEM;
-    k_unit_class<<<grid_r(un.nunits), 256, 0, s>>>(ord, g->edges, g->rowptr, un.ustart.p, un.nunits,
-                                                   cflag.p); tg_note_launch();
+    k_unit_lists<<<grid_r(cnt), 256, 0, s>>>(flag.p, pos.p, cnt, un.nunits, un.nheavy, un.ustart.p, un.heavy.p,
+                                             un.light.p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY(tg_scan_u32(cflag.p, cpos.p, un.nunits, s));
-    k_unit_lists<<<grid_r(un.nunits), 256, 0, s>>>(cflag.p, cpos.p, un.nunits, un.light.p,
-                                                   un.heavy.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastp, cpos.p + un.nunits - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaMemcpyAsync(&lastf, cflag.p + un.nunits - 1, 4, cudaMemcpyDeviceToHost, s));
-    TG_TRY_CUDA(cudaStreamSynchronize(s));
-    un.nlight = lastp + lastf;
-    un.nheavy = un.nunits - un.nlight;
     return TG_OK;
 }
 
@@ -1199,7 +1201,7 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
     {
         // tau of every edge, in the grouped order of the whole graph
         const uint32_t *ord = full_order;
-        TG_TRY(tg_edge_units(g, ord, M, s, un));
+        if (g->max_degree > kTauTiny) TG_TRY(tg_edge_units(g, ord, M, s, un));
         DevBuf<unsigned long long> q;
         if (!q.alloc(2, s)) return TG_ENOMEM;
         TG_TRY_CUDA(cudaMemsetAsync(q.p, 0, 16, s));
@@ -1240,10 +1242,12 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
         }
     }
     {
-        DevBuf<uint32_t> first;
-        if (!first.alloc(1, s)) return TG_ENOMEM;
-        k_tau_first<<<1, 1, 0, s>>>(g->rowptr, lists.uoff, n, first.p); tg_note_launch();
-        TG_TRY_CUDA(cudaGetLastError());
+        DevBuf<uint32_t> first;  // none: every edge is tiny
+        if (g->max_degree > kTauTiny) {
+            if (!first.alloc(1, s)) return TG_ENOMEM;
+            k_tau_first<<<1, 1, 0, s>>>(g->rowptr, lists.uoff, n, first.p); tg_note_launch();
+            TG_TRY_CUDA(cudaGetLastError());
+        }
         const size_t smem = (size_t)kTinyWarps * 32 * L * 4;
         int per_sm = 0;
         TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tau_tiny, kTinyWarps * 32, smem));
@@ -1303,8 +1307,9 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
         }
         tg_units un2;
         tg_units *ue = &un;
-        if (order != full_order || count != M) {
-            if (count > 0) TG_TRY(tg_edge_units(g, order, count, s, un2));
+        if (order != full_order || count != M || un.nunits == 0) {
+            if (count > 0 && tg_cyc_edges_units(g, count, rows || rowmap, t))
+                TG_TRY(tg_edge_units(g, order, count, s, un2));
             ue = &un2;
         }
         // triangle counts per adjacency entry, for the per-edge pass's reads
