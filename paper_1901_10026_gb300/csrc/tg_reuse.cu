@@ -48,12 +48,16 @@ constexpr int kProbeFactor = 4;
 // unit is a run of edges sharing j.  A CTA rebuilds its Gamma_j bitmap when it
 // takes a unit of another j, so a group is cut by cost, not by count: with
 // c_e = d_i + kUnitEdgeCost per edge and C_j the group's total, the units hold
-// about max(C_j / kUnitSplit, kUnitMinCost) each.  A hub's list is then built
+// about max(C_j / kUnitSplit, kUnitMinCost) each (kUnitMinLight for light units).  A hub's list is then built
 // about kUnitSplit times, and its heavy edges (first in the group) are spread
 // over as many units instead of filling one.
 constexpr int kUnitSplit = 8;
 constexpr int64_t kUnitEdgeCost = 16;
 constexpr int64_t kUnitMinCost = 8192;
+// Light units are one warp's work and their hash of Gamma_j is quickly made: with 8192
+// Alg. 1 waited for the longest of them (CL-100K 0.50 -> 0.33 ms, rows of CL-125K 0.52
+// -> 0.35, batch of 400 graphs 14.0 -> 12.8 in all; 2048: 0.35, 0.38, 13.0).
+constexpr int64_t kUnitMinLight = 1024;
 
 __global__ void k_group_bounds(const uint32_t *order, const int2 *edges, const int64_t *rowptr,
                                int64_t count, uint32_t *gs, uint32_t *ge, int64_t *cost) {
@@ -70,7 +74,7 @@ __global__ void k_group_bounds(const uint32_t *order, const int2 *edges, const i
 }
 
 // cum: exclusive prefix of the edge costs (count + 1 entries)
-__global__ void k_unit_flags(const uint32_t *order, const int2 *edges, int64_t count,
+__global__ void k_unit_flags(const uint32_t *order, const int2 *edges, const int64_t *rowptr, int64_t count,
                              const uint32_t *gs, const uint32_t *ge, const int64_t *cum,
                              uint32_t *flag) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < count;
@@ -83,7 +87,8 @@ __global__ void k_unit_flags(const uint32_t *order, const int2 *edges, int64_t c
             continue;
         }
         const int64_t base = cum[g0];
-        const int64_t ucost = max((cum[ge[j]] - base) / kUnitSplit, kUnitMinCost);
+        const int64_t least = rowptr[j + 1] - rowptr[j] > TG_LIGHT_DEGREE ? kUnitMinCost : kUnitMinLight;
+        const int64_t ucost = max((cum[ge[j]] - base) / kUnitSplit, least);
         flag[p] = (cum[p] - base) / ucost != (cum[p - 1] - base) / ucost ? 1u : 0u;
     }
 }
@@ -1148,7 +1153,7 @@ int launch_reuse_u(const ReuseParams &p, int threads, size_t smem, int grid_limi
 // Work units of the grouped order (see k_unit_flags), the heavy ones first.  Made only
 // for a graph or a pass that has use for them, with one wait for their number: with
 // the classes flagged, scanned and listed on the device, and a second wait, ER 1000
-// took 650 us and not 532, ER 1M/5M at k = 3 2.94 ms and not 2.54
+// took 650 us and not 532, ER 1M/5M at k = 3 2.94 ms and not 2.54.
 int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStream_t s,
                tg_units &un) {
     DevBuf<uint32_t> flag, pos, gs, ge;
@@ -1159,7 +1164,7 @@ int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStrea
     k_group_bounds<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, g->rowptr, cnt, gs.p, ge.p, cost.p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     TG_TRY(tg_scan_i64(cost.p, cum.p, cnt + 1, s));
-    k_unit_flags<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, cnt, gs.p, ge.p, cum.p, flag.p); tg_note_launch();
+    k_unit_flags<<<grid_r(cnt), 256, 0, s>>>(ord, g->edges, g->rowptr, cnt, gs.p, ge.p, cum.p, flag.p); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     TG_TRY(tg_scan_u32(flag.p, pos.p, cnt, s));
     DevBuf<uint32_t> num;
