@@ -91,3 +91,23 @@ def test_hub_rows(L):
     src = np.concatenate([u] + [h[0] for h in hubs]).astype(np.int32)
     dst = np.concatenate([v] + [h[1] for h in hubs]).astype(np.int32)
     _check(n, src, dst, synth.uniform_types(n, L, g), L)
+
+
+@pytest.mark.parametrize("L", [1, 5, 16])
+@pytest.mark.parametrize("low", [3, 4, 7, 8, 31, 32])
+def test_short_lists_of_members_with_long_lists(low, L):
+    """Lowest nodes of `low` members whose own up lists have 200 to 231 entries: the
+    members' lists are searched, not scanned, for even and odd numbers of members."""
+    core = 232
+    u, v = np.triu_indices(core, 1)
+    r = np.random.default_rng(low)
+    keep = r.random(u.shape[0]) < 0.97
+    src, dst = [u[keep]], [v[keep]]
+    for x in range(core, core + 40):
+        m = r.choice(core, low, replace=False)
+        src.append(np.full(low, x))
+        dst.append(m)
+    n = core + 40
+    src = np.concatenate(src).astype(np.int32)
+    dst = np.concatenate(dst).astype(np.int32)
+    _check(n, src, dst, r.integers(0, L, n).astype(np.uint8), L, sample=20)
