@@ -156,6 +156,99 @@ __global__ void k_fill_adj(const uint64_t *key, const uint32_t *val, int64_t tot
     }
 }
 
+// ---- lists of graphs without a node beyond kListMax neighbours
+// Both entries of every edge go to the next free place of their owner's list, then
+// each list is sorted by itself: two passes over the entries instead of one per digit
+// of (owner, type, id).  The order in which places are claimed does not matter, since a
+// list's words (type, id) are distinct.
+// Bound by the scattered 8-byte writes and their adds, then by instructions.  Against
+// keys, radix passes and a fill: ER 1M/5M 0.93 -> 0.27 ms (the k = 3 count 2.54 -> 1.89),
+// ER 100K/1M 0.22 -> 0.05 (1.70 -> 1.52), ER 1000 532 -> 486 us in all.
+constexpr int kListMax = 64;
+constexpr int kListLanes = 16;  // lanes of a list, up to 4 entries each
+
+// Edges are sorted by their end lo, so a warp claims the places of each run of equal
+// ends with one add.
+__global__ void k_scatter_arcs(const int32_t *lo, const int32_t *hi, int64_t M,
+                               const int32_t *old2new, const uint8_t *ntype, const int64_t *rowptr,
+                               uint32_t *used, uint2 *arcs, int2 *edges) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; c < M; c += step) {
+        const int64_t e = c + lane;
+        const bool in = e < M;
+        const int32_t l = in ? lo[e] : -1, h = in ? hi[e] : -1;
+        const int32_t prev = __shfl_up_sync(0xffffffffu, l, 1);
+        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || l != prev);
+        const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+        const unsigned after = heads & ~(0xffffffffu >> (31 - lane));
+        const int next = after ? __ffs(after) - 1 : 32;
+        int32_t a = 0, b = 0;
+        uint32_t pa = 0, pb = 0;
+        if (in) {
+            a = old2new[l];
+            b = old2new[h];
+            edges[e] = make_int2(a, b);
+            pb = atomicAdd(used + b, 1u);
+            if (lane == head) pa = atomicAdd(used + a, (uint32_t)(next - head));
+        }
+        pa = __shfl_sync(0xffffffffu, pa, head) + (uint32_t)(lane - head);
+        if (in) {
+            arcs[rowptr[a] + pa] = make_uint2((uint32_t)ntype[b] << TG_TSHIFT | (uint32_t)b, (uint32_t)e);
+            arcs[rowptr[b] + pb] = make_uint2((uint32_t)ntype[a] << TG_TSHIFT | (uint32_t)a, (uint32_t)e);
+        }
+    }
+}
+
+// One group of 16 lanes per list: an entry's place is the number of smaller words, each
+// word broadcast once; lane t counts the words of types below t, the typed offsets.
+__global__ void __launch_bounds__(256) k_sort_lists(const uint2 *arcs, const int64_t *rowptr, int64_t n,
+                                                    int32_t L, uint32_t *adj, uint32_t *eid, int32_t *toff) {
+    constexpr int E = kListMax / kListLanes;
+    const int q = threadIdx.x % kListLanes;
+    const int64_t step = (int64_t)gridDim.x * (256 / kListLanes);
+    // every lane of a warp makes the same number of steps
+    for (int64_t v0 = (int64_t)blockIdx.x * (256 / kListLanes); v0 < n; v0 += step) {
+        const int64_t v = v0 + threadIdx.x / kListLanes;
+        const int64_t b = v < n ? rowptr[v] : 0;
+        const int d = v < n ? (int)(rowptr[v + 1] - b) : 0;
+        const int dmax = __reduce_max_sync(0xffffffffu, d);
+        uint32_t w[E], id[E];
+        int at[E], below = 0;
+#pragma unroll
+        for (int z = 0; z < E; ++z) {
+            w[z] = 0xffffffffu;  // not below any word, and of no type below 15
+            at[z] = 0;
+            if (z * kListLanes + q < d) {
+                const uint2 x = arcs[b + z * kListLanes + q];
+                w[z] = x.x;
+                id[z] = x.y;
+            }
+        }
+#pragma unroll
+        for (int y = 0; y < E; ++y) {
+            const int stop = min(kListLanes, dmax - y * kListLanes);
+            for (int k = 0; k < stop; ++k) {
+                const uint32_t x = __shfl_sync(0xffffffffu, w[y], k, kListLanes);
+                below += (int)(x >> TG_TSHIFT) < q;
+#pragma unroll
+                for (int z = 0; z < E; ++z) at[z] += x < w[z];
+            }
+        }
+#pragma unroll
+        for (int z = 0; z < E; ++z)
+            if (z * kListLanes + q < d) {
+                adj[b + at[z]] = w[z];
+                eid[b + at[z]] = id[z];
+            }
+        if (v < n) {
+            int32_t *to = toff + v * (L + 1);
+            if (q < L) to[q] = below;
+            if (q == 0) to[L] = d;
+        }
+    }
+}
+
 int build_impl(int64_t n, int64_t m, const int32_t *src, const int32_t *dst,
                const uint8_t *type, int32_t L, uint32_t flags, cudaStream_t s, tg_graph **out) {
     if (!out) return TG_EINVAL;
@@ -300,8 +393,21 @@ int build_impl(int64_t n, int64_t m, const int32_t *src, const int32_t *dst,
     g->toff = (int32_t *)tg_dalloc(n * (L + 1) * 4, s);
     g->eid = (uint32_t *)tg_dalloc((total > 0 ? total : 1) * 4, s);
     if (!g->adj || !g->edges || !g->toff || !g->eid) return TG_ENOMEM;
-    TG_TRY_CUDA(cudaMemsetAsync(g->toff, 0, n * (L + 1) * 4, s));
-    if (M > 0) {
+    if (M > 0 && g->max_degree <= kListMax) {
+        DevBuf<uint2> arcs;
+        DevBuf<uint32_t> used;
+        if (!arcs.alloc(total, s) || !used.alloc(n, s)) return TG_ENOMEM;
+        TG_TRY_CUDA(cudaMemsetAsync(used.p, 0, n * 4, s));
+        k_scatter_arcs<<<grid_for(M), kThreads, 0, s>>>(lo.p, hi.p, M, old2new.p, g->ntype, g->rowptr, used.p,
+                                                        arcs.p, g->edges); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+        k_sort_lists<<<grid_for(n * kListLanes), 256, 0, s>>>(arcs.p, g->rowptr, n, L, g->adj, g->eid,
+                                                              g->toff); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+    } else {
+        TG_TRY_CUDA(cudaMemsetAsync(g->toff, 0, n * (L + 1) * 4, s));
+    }
+    if (M > 0 && g->max_degree > kListMax) {
         DevBuf<uint64_t> d1, d2;
         DevBuf<uint32_t> v1, v2;
         if (!d1.alloc(total, s) || !d2.alloc(total, s) || !v1.alloc(total, s) ||

@@ -5,6 +5,7 @@ repeated pairs, one hub (equal digits), and ids that need one more digit."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_1901_10026_gb300 as tg
 
 pytestmark = pytest.mark.gpu
@@ -17,6 +18,7 @@ def _built():
         pytest.skip("no CUDA device")
     from paper_1901_10026_gb300 import build
     build.build()
+    oracle.build()
 
 
 def _check(n, src, dst, L=3):
@@ -47,3 +49,20 @@ def test_hub_and_repeats():
     src = np.where(g.random(m) < 0.7, 17, g.integers(0, n, m)).astype(np.int32)
     dst = g.integers(0, 40, m).astype(np.int32) * 700
     _check(n, src, dst)
+
+
+@pytest.mark.parametrize("L", [1, 3, 16])
+@pytest.mark.parametrize("top", [1, 2, 15, 16, 17, 32, 33, 63, 64, 65, 66])
+def test_lists_around_the_degree_bound(top, L):
+    """Lists sorted by themselves (no node beyond 64 neighbours) and by the radix sort:
+    a node of `top` neighbours among random pairs of low degree, against the lists'
+    own counts; 31 to 33 edges of equal lower ends in a row among them."""
+    g = np.random.default_rng([top, L])
+    n = 500
+    src = np.concatenate([np.full(top, 3), g.integers(100, n, 300)]).astype(np.int32)
+    dst = np.concatenate([np.arange(top) + 5, g.integers(100, n, 300)]).astype(np.int32)
+    _check(n, src, dst, L)
+    types = (np.arange(n) * 7 % 11 % L).astype(np.uint8)
+    want = oracle.OracleGraph(n, src, dst, types, L).per_edge(4, "orbit")
+    got = tg.tg_count_per_edge(tg.tg_build_csr(n, src, dst, types, L), 4, tg.TG_ORBIT)
+    assert np.array_equal(got, want)
