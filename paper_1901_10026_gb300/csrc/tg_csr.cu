@@ -13,6 +13,7 @@
 //      every adjacency list sorted by (type, id); entries are stored packed
 //      as (type << 28) | id;
 //   5. per-node type offsets toff[v][t] (start of Gamma_v^t inside row v).
+#include <algorithm>
 #include <stdlib.h>
 
 #include "tg_internal.cuh"
@@ -351,7 +352,8 @@ int build_impl(int64_t n, int64_t m, const int32_t *src, const int32_t *dst,
     DevBuf<unsigned long long> stats;
     if (!stats.alloc(2, s)) return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemsetAsync(stats.p, 0, 2 * sizeof(unsigned long long), s));
-    k_max_deg<<<grid_for(n), kThreads, 0, s>>>(deg.p, n, stats.p, stats.p + 1); tg_note_launch();
+    // a few warps per SM: each ends with two adds to the same two words
+    k_max_deg<<<std::min<unsigned>(grid_for(n), (unsigned)tg_num_sms() * 2), kThreads, 0, s>>>(deg.p, n, stats.p, stats.p + 1); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     unsigned long long hstats[2] = {0, 0};
     TG_TRY_CUDA(cudaMemcpyAsync(hstats, stats.p, sizeof(hstats), cudaMemcpyDeviceToHost, s));

@@ -97,10 +97,12 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
     uint32_t *row = reinterpret_cast<uint32_t *>(ts + words) + warp * 32 * (LP + 1);
     for (int q = threadIdx.x; q < words; q += blockDim.x) ts[q] = 0ull;
     int pa[kSlots], pb[kSlots];
+    uint32_t nec[kSlots];  // edges of the lane's type pairs, added to ne at the end
 #pragma unroll
     for (int z = 0; z < kSlots; ++z) {
         const int q = lane + 32 * z;
         pa[z] = pb[z] = 0;
+        nec[z] = 0u;
         if (q < P) unpair(L, q, pa[z], pb[z]);
     }
     __syncthreads();
@@ -126,7 +128,9 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
             const int g = __shfl_sync(kFull, pt, __ffs(todo) - 1);
             unsigned grp = __ballot_sync(kFull, pt == g);
             todo &= ~grp;
-            if (lane == 0) atomicAdd(ne + g, (unsigned long long)__popc(grp));
+#pragma unroll
+            for (int z = 0; z < kSlots; ++z)
+                if (lane + 32 * z == g) nec[z] += (uint32_t)__popc(grp);
             if (!any) continue;
             unsigned long long acc[kSlots], st = 0;
 #pragma unroll
@@ -151,6 +155,9 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
         }
         __syncwarp();  // the rows are rewritten by the next chunk
     }
+#pragma unroll
+    for (int z = 0; z < kSlots; ++z)
+        if (nec[z]) atomicAdd(ne + lane + 32 * z, (unsigned long long)nec[z]);
     __syncthreads();
     unsigned long long *s_p3 = p.sums + p.e2, *s_h2 = s_p3 + p.n3, *s_p4 = s_h2 + p.n3;
     unsigned long long *s_d = s_p4 + 3 * p.n4;
@@ -187,6 +194,21 @@ constexpr int kNodeMin = 16;  // nodes of a team's range, at least
 // nodes whose rows are read before they are used: of an 8M-edge power law's sums (L = 5)
 // 1.88 ms become 1.63 with 2 and 1.67 with 4
 constexpr int kNodeBatch = 2;
+
+// C(x, 3), the factors 2 and 3 taken out before the product
+__device__ __forceinline__ unsigned long long c3(uint32_t x) {
+    const uint32_t m = x % 3u;
+    uint32_t p = x, q = x - 1u, r = x - 2u;
+    if (x < 3u) return 0ull;
+    if (m == 0u) p /= 3u;
+    if (m == 1u) q /= 3u;
+    if (m == 2u) r /= 3u;
+    if (x & 1u)
+        q >>= 1;
+    else
+        p >>= 1;
+    return (unsigned long long)p * q * r;
+}
 
 template <int LP>
 __global__ void __launch_bounds__(kNodeThreads) k_sum_nodes(SumParams p) {
@@ -276,8 +298,8 @@ __global__ void __launch_bounds__(kNodeThreads) k_sum_nodes(SumParams p) {
                         uint64_t w = 0;
                         if (ts[z] < 0)
                             w = 0;
-                        else if (ts[z] == tu[z])  // C(x0, 3), the factor 3 taken out before the product
-                            w = x0 < 3 ? 0 : x0 % 3 == 2 ? c2(x0) * ((x0 - 2) / 3) : c2(x0) / 3 * (x0 - 2);
+                        else if (ts[z] == tu[z])
+                            w = c3((uint32_t)x0);
                         else if (ts[z] == tt[z])
                             w = c2(x0) * x2;
                         else if (tt[z] == tu[z])
