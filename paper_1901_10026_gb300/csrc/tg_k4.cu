@@ -639,14 +639,23 @@ int launch_cliques(const unsigned long long (&size)[2 * kUpClasses], CliqueParam
         while ((1 << p.hlg) < 2 * dmax) ++p.hlg;
         const int wpl = k == kUpXL ? 4 : k == kUpL ? 2 : 1;
         const size_t rbytes = (size_t)dmax * up_words(dmax, p.L) * 4;
+        auto fixed = [&](int th) {  // shared memory besides the rows
+            return h4b + (size_t)9 * ((size_t)1 << p.hlg) + (size_t)(th / 32) * kPend * 8 +
+                   (kEdge ? 0 : (size_t)(th / 32) * p.L * 32 * wpl * 4);
+        };
+        // Rows in shared memory where a quarter of the class's threads or more leaves
+        // room for them, else in global memory with CTAs of up to 512.  The cliques of
+        // R-MAT-23, whose longest rows do not fit, take 725 ms when the threads are cut to
+        // 64 in vain, 410 with 1024, 382 with 512, 413 with 256; those of R-MAT-21, whose
+        // rows fit, 56 with 1024 and 60 with 512.
         int threads = kUpThreads[k];
-        size_t base = 0;
-        for (;; threads /= 2) {  // the columns of fewer warps where they would not fit
-            base = h4b + (size_t)9 * ((size_t)1 << p.hlg) + (size_t)(threads / 32) * kPend * 8 +
-                   (kEdge ? 0 : (size_t)(threads / 32) * p.L * 32 * wpl * 4);
-            if (threads == 64 || base + (k == kUpXL ? 0 : rbytes) <= avail) break;
+        while (threads > std::max(64, kUpThreads[k] / 4) && fixed(threads) + rbytes > avail) threads /= 2;
+        const bool sm = k != kUpXL && fixed(threads) + rbytes <= avail;
+        if (!sm) {
+            threads = std::min(kUpThreads[k], 512);
+            while (threads > 64 && fixed(threads) > avail) threads /= 2;
         }
-        const bool sm = k != kUpXL && base + rbytes <= avail;
+        const size_t base = fixed(threads);
         const size_t smem = base + (sm ? rbytes : 0);
         if (smem > avail) return TG_EINVAL;
         void (*fn)(CliqueParams) = k == kUpXL ? k_k4_rows<4, kEdge, false>

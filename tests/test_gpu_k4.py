@@ -111,3 +111,11 @@ def test_short_lists_of_members_with_long_lists(low, L):
     src = np.concatenate(src).astype(np.int32)
     dst = np.concatenate(dst).astype(np.int32)
     _check(n, src, dst, r.integers(0, L, n).astype(np.uint8), L, sample=20)
+
+
+@pytest.mark.parametrize("m", [1000, 1984])  # rows of up to 62 words, beyond shared memory
+def test_rows_in_global_memory(m):
+    inner = 7
+    n, src, dst = _bipartite(m, inner)
+    g = tg.tg_build_csr(n, src, dst, np.zeros(n, np.uint8), 1)
+    assert tg.tg_count_global(g, 4)[-1] == m * comb(inner, 3) + comb(inner, 4)
