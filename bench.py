@@ -189,10 +189,10 @@ def measured_peak_gbs():
 # sources each phase's kernels are built from; a recorded traffic figure
 # stands only while they are unchanged
 PHASE_SOURCES = {
-    "tau": ["tg_reuse.cu", "tg_device.cuh"],
-    "count": ["tg_edges.cu", "tg_device.cuh"],
-    "cycles": ["tg_cycles.cu", "tg_device.cuh"],
-    "cliques": ["tg_cycles.cu", "tg_device.cuh"],
+    "tau": ["tg_reuse.cu", "tg_lists.cu", "tg_device.cuh"],
+    "count": ["tg_sums.cu", "tg_edges.cu", "tg_device.cuh"],
+    "cycles": ["tg_cycles.cu", "tg_c4_light.cu", "tg_cycles.cuh", "tg_device.cuh"],
+    "cliques": ["tg_k4.cu", "tg_cycles.cu", "tg_cycles.cuh", "tg_device.cuh"],
 }
 
 
@@ -223,7 +223,7 @@ def phase_bytes(tm, L, M, sum_min_deg):
       tau     (Alg. 1) the shorter endpoint list of every edge (4 B an entry),
               the edge's endpoints (8 B) and its L typed triangle counts
               written (4L B);
-      count   (per-edge pass) 4 B per Gamma_i entry read, per T member its two
+      count   (per-edge pass; whole-graph sums: sums_bytes) 4 B per Gamma_i entry read, per T member its two
               edge ids, its tau rows toward i and j and its typed offsets
               (4(3L+3) B), per edge its order entry, endpoints, tau row,
               typed offsets, degrees and types of i and j and their Theta and
@@ -237,6 +237,13 @@ def phase_bytes(tm, L, M, sum_min_deg):
         "cycles": 4.0 * tm["wedges"],
         "cliques": None,
     }
+
+
+def sums_bytes(n, M, L):
+    """Algorithmic bytes of the count phase of a whole-graph global count, which has
+    no per-edge pass: per edge its endpoints and tau row (8 + 4L B), per node its type,
+    typed offsets, Theta and D rows (5 + 4L + 8L^2 B)."""
+    return (8.0 + 4.0 * L) * M + (5.0 + 4.0 * L + 8.0 * L * L) * n
 
 
 def oracle_sample(og, seconds, max_edges, seed):
@@ -673,7 +680,7 @@ def run_directed(args):
         "clocks": clk.summary(), "gpu_launches": int(launches),
         "roofline": {"bound": "hbm", "achieved": algo / (step / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                      "frac": algo / (step / 1e3) / 1e9 / peak, "traffic": None, "peak_kind": peak_kind,
-                     "kernel": "k_dir3 (+ k_dir_degrees, k_dir_finalize)", "algorithmic_bytes": algo,
+                     "kernel": "k_tri_heavy + k_tri_light + k_dir_paths", "algorithmic_bytes": algo,
                      "algorithmic_basis": "5 B per entry of the shorter endpoint list, 9 + 24 L B per edge"},
         "triads": {name: int(c) for name, c in zip(tg.TRIAD_NAMES, h)},
     }
@@ -820,6 +827,8 @@ def main():
     mean_ms = {ph: statistics.mean(t[f"{ph}_ms"] for t in timings)
                for ph in ("tau", "aggregate", "count", "cycles", "cliques")}
     pbytes = phase_bytes(tm, L, M, sum_min_deg)
+    if not tm["gamma_entries"] and not tm["t_members"]:  # no per-edge pass ran
+        pbytes["count"] = sums_bytes(G.n, M, L)
     phases = {}
     for ph in ("tau", "count", "cycles", "cliques"):
         ms = mean_ms[ph]
@@ -833,8 +842,8 @@ def main():
                               if phases[ph]["achieved_gbs"] is not None else None)
     dominant = max(("tau", "count", "cycles"), key=lambda ph: phases[ph]["ms"])
     kernels = {"tau": "k_tau (Alg. 1 typed triangle counts)",
-               "count": "per-edge pass: k_cyc_edge + k_cyc_tsum_light + k_cyc_finish",
-               "cycles": "4-cycle enumeration: k_c4_bin_walk + k_c4_bin_pairs + walk waves"}
+               "count": "whole-graph sums: k_sum_edges + k_sum_nodes (shards: per-edge pass)",
+               "cycles": "4-cycle enumeration: k_c4_bin_walk + k_c4_bin_gram + k_c4_cta"}
     d = phases[dominant]
     roofline = {
         "bound": "hbm", "achieved": d["achieved_gbs"], "peak": peak, "unit": "GB/s",
