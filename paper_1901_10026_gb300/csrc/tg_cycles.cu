@@ -24,13 +24,14 @@
 //     clear the counters.  Light anchors keep their counters in shared memory
 //     (tg_c4_light.cu); global mode walks costly ones in warp units over binned
 //     waves and waves of counter slots.
-//   4-cliques (k_k4): each 4-clique x0 < v < w < x (by rank) is met once from
+//   4-cliques (tg_k4.cu; lists beyond its rows: k_k4, k_k4_global): each 4-clique x0 < v < w < x (by rank) is met once from
 //     its lowest node along "up" lists (neighbours of higher rank) and adds one
 //     to each of its six edges, keyed by the unordered types of the two nodes
 //     off the edge.
 // The enumeration work is the number of degree-ordered wedges plus the
 // 4-clique search, instead of sum over w in S_i u S_j u T_ij of d_w per edge.
-// The per-edge pass (tg_edges.cu) then needs only Gamma_i n Gamma_j (the T
+// Whole-graph sums (tg_sums.cu) need only the totals; the per-edge pass
+// (tg_edges.cu) needs only Gamma_i n Gamma_j (the T
 // sums) and O(L^2) identity and closed-form arithmetic.
 #include <algorithm>
 #include <new>
