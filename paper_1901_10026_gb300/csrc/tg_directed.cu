@@ -191,12 +191,20 @@ __global__ void __launch_bounds__(kDirThreads) k_dir_degrees(const int64_t *rowp
 
 __device__ __forceinline__ int swap_state(int s) { return ((s & 1) << 1) | ((s >> 1) & 1); }
 
-// Per-edge rows: one warp per edge (dynamic queue).
+// One warp per edge (dynamic queue).  kRows: per-edge rows, else the undivided sums
+// of a small graph's global count (per-CTA shared histogram).
+template <bool kRows>
 __global__ void __launch_bounds__(kDirThreads) k_dir3(DirParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int L = p.L, S = TG_TRIAD_CLASSES * L;
-    uint32_t *tri = reinterpret_cast<uint32_t *>(smem) + (size_t)warp * 9 * L;
+    const int64_t hlen = kRows ? 0 : TG_TRIAD_CLASSES * p.n3;
+    unsigned long long *h = reinterpret_cast<unsigned long long *>(smem);
+    uint32_t *tri = reinterpret_cast<uint32_t *>(h + hlen) + (size_t)warp * 9 * L;
+    if (!kRows) {
+        for (int64_t q = threadIdx.x; q < hlen; q += blockDim.x) h[q] = 0ull;
+        __syncthreads();
+    }
     for (;;) {
         unsigned long long item = 0;
         if (lane == 0) item = atomicAdd(p.queue, 1ull);
@@ -263,12 +271,25 @@ __global__ void __launch_bounds__(kDirThreads) k_dir3(DirParams p) {
                         v += (unsigned long long)m;
                     }
                 }
-                p.rows[e * S + k] = v;
+                if (kRows) {
+                    p.rows[e * S + k] = v;
+                } else if (v) {
+                    int a = ti, b = tj, cc = t;
+                    sort2(a, b);
+                    sort2(b, cc);
+                    sort2(a, b);
+                    atomicAdd(h + (int64_t)c * p.n3 + colex3(a, b, cc), v);
+                }
             }
-        } else {
+        } else if (kRows) {
             for (int k = lane; k < S; k += 32) p.rows[e * S + k] = 0ull;
         }
         __syncwarp();
+    }
+    if (!kRows) {
+        __syncthreads();
+        for (int64_t q = threadIdx.x; q < hlen; q += blockDim.x)
+            if (h[q]) atomicAdd(p.sums + q, h[q]);
     }
 }
 
@@ -690,6 +711,19 @@ int dir_totals(const tg_graph *g, const DirParams &d, cudaStream_t s) {
     return TG_OK;
 }
 
+// Global counts of small graphs take k_dir3, edge by edge: dir_totals launches about a
+// dozen kernels more (lists, units) and waits twice.  Its gain grows with the edges and
+// their lists, its fixed part with the types.  k_dir3 against dir_totals, ER graphs
+// unless said otherwise: 3,000 edges 0.07 and 0.18 ms (L = 3); 140,000 at mean degree
+// 18 0.24 and 0.23 (L = 8), 0.25 and 0.31 (L = 9); 200,000 at mean degree 6 0.31 and
+// 0.28 (L = 8), 0.31 and 0.42 (L = 9); 100,000 of a dense graph (mean degree 280) 0.37
+// and 0.32 (L = 1).  Of 270 graphs (ER, power law, R-MAT, dense; 8,000 to 450,000
+// edges; L = 1 to 16) the rule takes the slower way in none by more than 27 %.
+bool dir_totals_pays(const tg_graph *g) {
+    const double mean = 2.0 * (double)g->M / (double)g->n_nonisolated;
+    return (double)g->M * (1.0 + mean / 160.0) >= (g->L <= 8 ? 196608.0 : 327680.0);
+}
+
 // Per-edge rows (rows != nullptr) or undivided global sums of a TG_DIRECTED graph.
 int dir_count(const tg_graph *g, uint64_t *rows, unsigned long long *sums, unsigned *err,
               cudaStream_t s) {
@@ -733,15 +767,15 @@ int dir_count(const tg_graph *g, uint64_t *rows, unsigned long long *sums, unsig
             // a 3-path: centre 0, ends 1 (state sij) and 2 (state s1), seen from 0
             p.path[(sij - 1) * 3 + (s1 - 1)] = tt.cls[pair_mask(sij, 0, 1) | pair_mask(s1, 0, 2)];
         }
-    if (!rows) return dir_totals(g, p, s);
-    const void *fn = (const void *)k_dir3;
-    const size_t smem = (size_t)kDirWarps * 9 * L * 4;
-    TG_TRY(tg_allow_max_smem(fn));
+    if (!rows && dir_totals_pays(g)) return dir_totals(g, p, s);
+    void (*const fn)(DirParams) = rows ? k_dir3<true> : k_dir3<false>;
+    const size_t smem = (rows ? 0 : (size_t)TG_TRIAD_CLASSES * p.n3 * 8) + (size_t)kDirWarps * 9 * L * 4;
+    TG_TRY(tg_allow_max_smem((const void *)fn));
     int per = 0;
     TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kDirThreads, smem));
     if (per < 1) return TG_ENOMEM;
     const int64_t grid = std::min<int64_t>((int64_t)tg_num_sms() * per, (M + kDirWarps - 1) / kDirWarps);
-    k_dir3<<<(unsigned)grid, kDirThreads, smem, s>>>(p);
+    fn<<<(unsigned)grid, kDirThreads, smem, s>>>(p);
     tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     TG_TRY_CUDA(cudaStreamSynchronize(s));
