@@ -2293,12 +2293,23 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
     // counter slots: one per CTA of k_c4, one per split anchor of a wave; all
     // within a quarter of free memory
     const bool walk_waves = t.hash_slots >= 64;
+    // Per-edge waves: kWaveMax costly anchors have about 2^20 walk positions or more; of
+    // cheaper ones (unroll 4 alone splits them) a wave takes as many as have that many, a
+    // wave being three launches.  With kWaveMax throughout, rows with unroll 4 took 63 ms
+    // and not 23 on a cycle of 300,000 nodes, 11.7 and not 4.8 on ER 50K/400K.
+    int64_t wave_max = kWaveMax;
+    if (!global && nheavy > 0) {
+        unsigned long long walk = 0;
+        for (const C4HeavyInfo &x : info) walk += x.cost;
+        const unsigned long long mean = std::max<unsigned long long>(1, walk / (unsigned long long)nheavy);
+        wave_max = std::max(kWaveMax, std::min(full_grid, (int64_t)((1ull << 20) / mean)));
+    }
     const int64_t slot_words = n * (L + 1) + (n + 31) / 32;
     const size_t slot_bytes = (size_t)slot_words * 4;
     int64_t want = 0;
     if (cls.size[kC4Slot] > 0) want = std::min<int64_t>(full_grid, cls.size[kC4Slot]);
     if (nheavy > 0)
-        want = std::max<int64_t>(want, std::min<int64_t>(walk_waves ? kWaveMax : full_grid, nheavy));
+        want = std::max<int64_t>(want, std::min<int64_t>(walk_waves ? wave_max : full_grid, nheavy));
     size_t free_b = 0, total_b = 0;
     TG_TRY_CUDA(cudaMemGetInfo(&free_b, &total_b));
     int64_t slots = std::min<int64_t>(want, (int64_t)(free_b / 4 / (slot_bytes ? slot_bytes : 1)));

@@ -1,5 +1,6 @@
 """Every 4-cycle anchor split over the grid (``unroll = 4``): more anchors than one CTA
-sorts and more than a wave holds, against the default classes and O1."""
+sorts and more than a wave holds, against the default classes and O1; and the launches
+that the waves of many cheap anchors take."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,16 @@ def test_many_split_anchors(n, m, hub, L, split_all):
     assert np.array_equal(split[1], tg.tg_count_per_edge(g, 4, tg.TG_ORBIT))
     e = np.unique(np.random.default_rng(1).integers(0, g.M, 50))
     assert np.array_equal(split[1][e], oracle.OracleGraph(*G).per_edge(4, "orbit", edges=e))
+
+
+def test_cheap_anchors_take_few_waves(split_all):
+    """Rows of a cycle: 40,000 anchors of one member each."""
+    n = 40000
+    v = np.arange(n, dtype=np.int32)
+    g = tg.tg_build_csr(n, v, ((v + 1) % n).astype(np.int32), np.zeros(n, np.uint8), 1)
+    tg.tg_count_per_edge(g, 4)
+    before = tg.tg_launch_count()
+    rows = tg.tg_count_per_edge(g, 4)
+    assert tg.tg_launch_count() - before < 300  # 128 anchors a wave: above 900
+    # two nodes off either end; induced 4-paths: the edge in the middle once, at an end twice
+    assert np.array_equal(rows, np.tile(np.array([2, 0, 3, 0, 0, 0, 0, 0], np.uint64), (n, 1)))
