@@ -319,14 +319,17 @@ struct TriParams {
     unsigned long long *queue;
 };
 
-// est[e]: the state of edge e seen from its end of smaller id
+// est[e]: the state of edge e seen from its end of smaller id.  Every entry carries an
+// arc; one that does not sets err, at which the kernels that index by the states leave.
 __global__ void k_edge_states(const uint32_t *adj, const uint32_t *eid, const uint8_t *adir,
-                              const int2 *edges, int64_t entries, uint8_t *est) {
+                              const int2 *edges, int64_t entries, uint8_t *est, unsigned *err) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < entries;
          x += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t e = __ldg(eid + x);
         const int2 ab = edges[e];
-        if ((int)(__ldg(adj + x) & TG_IDMASK) == max(ab.x, ab.y)) est[e] = adir[x];
+        const uint8_t st = adir[x];
+        if (st < 1 || st > 3) atomicOr(err, TG_DERR_BOUNDS);
+        if ((int)(__ldg(adj + x) & TG_IDMASK) == max(ab.x, ab.y)) est[e] = st;
     }
 }
 
@@ -431,6 +434,7 @@ constexpr int kTriThreads = 1024;
 
 template <bool kAll>  // every id that occurs is in the map
 __global__ void __launch_bounds__(kTriThreads) k_tri_heavy(TriParams p) {
+    if (*p.d.err) return;  // see k_edge_states
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_unit;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
@@ -507,6 +511,7 @@ __global__ void __launch_bounds__(kTriThreads) k_tri_heavy(TriParams p) {
 constexpr int kTriLightWarps = 8;
 
 __global__ void __launch_bounds__(kTriLightWarps * 32) k_tri_light(TriParams p) {
+    if (*p.d.err) return;  // see k_edge_states
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int L = p.d.L;
@@ -653,7 +658,7 @@ int dir_totals(const tg_graph *g, const DirParams &d, cudaStream_t s) {
     if (!est.alloc(M, s) || !queue.alloc(2, s)) return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemsetAsync(queue.p, 0, 16, s));
     k_edge_states<<<(unsigned)std::min<int64_t>((2 * M + 255) / 256, 65535LL * 16), 256, 0, s>>>(
-        g->adj, g->eid, g->adir, g->edges, 2 * M, est.p); tg_note_launch();
+        g->adj, g->eid, g->adir, g->edges, 2 * M, est.p, d.err); tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     const tg_lists *lists = nullptr;
     TG_TRY(tg_graph_lists(g, &lists, s));
