@@ -185,8 +185,8 @@ int tg_slot_config(int32_t L, int32_t k, int32_t level, int32_t phi_i, int32_t p
  * other TG_KERNEL_* choices run Alg. 2-3 per edge as the paper does.  The
  * counts are the same.  Errors: TG_EINVAL,
  * TG_EOVERFLOW (the graph is too large for the 32-bit per-edge counters:
- * 2M >= 2^31), TG_EINTERNAL (a sum not divisible by |E(H)|), TG_ENOMEM,
- * TG_ECUDA.
+ * 2M >= 2^31), TG_EINTERNAL (a sum not divisible by |E(H)|, or totals of the
+ * whole graph that contradict one another), TG_ENOMEM, TG_ECUDA.
  */
 int tg_count_global(const tg_graph *g, int32_t k, uint64_t *out, void *stream);
 
@@ -239,6 +239,7 @@ int tg_sparse_id(int32_t L, int32_t k, int32_t level, int64_t id, int32_t *motif
  * total to tg_global_finalize gives tg_count_global's result; this is the
  * unit of work one rank does when the edges are sharded across GPUs.
  *   sums  tg_global_len(L, k) uint64, host or device
+ * Errors as tg_count_global; TG_EINVAL for a range outside [0, M].
  */
 int tg_count_range(const tg_graph *g, int32_t k, int64_t e0, int64_t e1, uint64_t *sums,
                    void *stream);

@@ -1195,14 +1195,16 @@ static int launch_cta_u(const CountParams &p, const CtaParams &cp, int threads, 
 // lists holds the grouped order of the whole graph.
 static int launch_count(const tg_graph *g, int k, int level, const tg_lists &lists,
                         const uint32_t *order, int64_t e0, int64_t count, uint64_t *rows,
-                        int64_t width, unsigned long long *hist, cudaStream_t s) {
+                        int64_t width, unsigned long long *hist, cudaStream_t s,
+                        unsigned *err = nullptr) {
     if (count <= 0) return TG_OK;
     {
         const tg_tune t0 = tune_now();
         if ((t0.kernel == TG_KERNEL_AUTO || t0.kernel == TG_KERNEL_REUSE ||
              t0.kernel == TG_KERNEL_CYCLES) &&
             order)
-            return tg_reuse_count(g, k, level, lists, order, count, rows, width, hist, t0, s);
+            return tg_reuse_count(g, k, level, lists, order, count, rows, width, hist, t0, s, tg_part(),
+                                  nullptr, err);
     }
     DevBuf<unsigned long long> queue;
     if (!queue.alloc(1, s)) return TG_ENOMEM;
@@ -1232,15 +1234,16 @@ static int check_counts(const tg_graph *g, int k) {
     return TG_OK;
 }
 
+// err: device error bits, set where a whole graph's totals contradict one another
 static int sums_impl(const tg_graph *g, int k, int64_t e0, int64_t e1,
-                     unsigned long long *dsums, cudaStream_t s) {
+                     unsigned long long *dsums, unsigned *err, cudaStream_t s) {
     const int64_t len = tg_global_len(g->L, k);
     TG_TRY_CUDA(cudaMemsetAsync(dsums, 0, len * 8, s));
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));
     if (e0 == 0 && e1 == g->M)
         return launch_count(g, k, TG_GRAPHLET, sc->lists, sc->lists.order, 0, g->M, nullptr, 0, dsums,
-                            s);
+                            s, err);
     DevBuf<uint32_t> order;
     TG_TRY(grouped_order(g, e0, e1 - e0, s, order));
     return launch_count(g, k, TG_GRAPHLET, sc->lists, order.p, 0, e1 - e0, nullptr, 0, dsums, s);
@@ -1255,7 +1258,7 @@ extern "C" int tg_count_global(const tg_graph *g, int32_t k, uint64_t *out, void
     DevBuf<unsigned> err;
     if (!sums.alloc(len, s) || !err.alloc(1, s)) return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemsetAsync(err.p, 0, 4, s));
-    TG_TRY(sums_impl(g, k, 0, g->M, sums.p, s));
+    TG_TRY(sums_impl(g, k, 0, g->M, sums.p, err.p, s));
     const bool dev_out = tg_is_device_ptr(out);
     DevBuf<uint64_t> tmp;
     uint64_t *dst = out;
@@ -1281,17 +1284,19 @@ extern "C" int tg_count_range(const tg_graph *g, int32_t k, int64_t e0, int64_t 
     if (!sums || e0 < 0 || e1 < e0 || e1 > g->M) return TG_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t len = tg_global_len(g->L, k);
-    if (tg_is_device_ptr(sums)) {
-        TG_TRY(sums_impl(g, k, e0, e1, reinterpret_cast<unsigned long long *>(sums), s));
-        TG_TRY_CUDA(cudaStreamSynchronize(s));
-        return TG_OK;
-    }
     DevBuf<unsigned long long> d;
-    if (!d.alloc(len, s)) return TG_ENOMEM;
-    TG_TRY(sums_impl(g, k, e0, e1, d.p, s));
-    TG_TRY_CUDA(cudaMemcpyAsync(sums, d.p, len * 8, cudaMemcpyDeviceToHost, s));
+    DevBuf<unsigned> err;
+    unsigned long long *dsums = reinterpret_cast<unsigned long long *>(sums);
+    const bool dev_out = tg_is_device_ptr(sums);
+    if (!err.alloc(1, s) || (!dev_out && !d.alloc(len, s))) return TG_ENOMEM;
+    if (!dev_out) dsums = d.p;
+    TG_TRY_CUDA(cudaMemsetAsync(err.p, 0, 4, s));
+    TG_TRY(sums_impl(g, k, e0, e1, dsums, err.p, s));
+    unsigned herr = 0;
+    TG_TRY_CUDA(cudaMemcpyAsync(&herr, err.p, 4, cudaMemcpyDeviceToHost, s));
+    if (!dev_out) TG_TRY_CUDA(cudaMemcpyAsync(sums, d.p, len * 8, cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
-    return TG_OK;
+    return herr ? TG_EINTERNAL : TG_OK;
 }
 
 namespace {
@@ -1339,6 +1344,7 @@ extern "C" int tg_count_shard(const tg_graph *g, int32_t k, int32_t shard, int32
     if (!sums || nshards < 1 || shard < 0 || shard >= nshards) return TG_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t len = tg_global_len(g->L, k);
+    if (nshards == 1) return tg_count_range(g, k, 0, g->M, sums, stream);
     DevBuf<unsigned long long> d;
     unsigned long long *dsums = reinterpret_cast<unsigned long long *>(sums);
     const bool dev_out = tg_is_device_ptr(sums);
@@ -1346,9 +1352,7 @@ extern "C" int tg_count_shard(const tg_graph *g, int32_t k, int32_t shard, int32
         if (!d.alloc(len, s)) return TG_ENOMEM;
         dsums = d.p;
     }
-    if (nshards == 1) {
-        TG_TRY(sums_impl(g, k, 0, g->M, dsums, s));
-    } else {
+    {
         TG_TRY_CUDA(cudaMemsetAsync(dsums, 0, len * 8, s));
         tg_sched *sc = nullptr;
         TG_TRY(get_sched(g, s, &sc));

@@ -19,6 +19,7 @@
 #define TG_DERR_INPUT 1u      // node id or type out of range in the input
 #define TG_DERR_DIVISIBLE 2u  // a global sum not divisible by |E(H)|
 #define TG_DERR_BOUNDS 4u     // an internal bounds check failed
+#define TG_DERR_TOTALS 8u     // totals of one graph that contradict one another
 
 struct tg_sched;  // per-graph counting schedule (tg_count.cu)
 
@@ -211,10 +212,11 @@ int tg_cyc_edges(const tg_graph *g, int k, int level, const uint32_t *order, int
 
 // Undivided whole-graph sums from node-level and edge-level totals (tg_sums.cu):
 // tau of every edge and, for k = 4, Theta, the D sums over higher ids (see
-// k_node_aggr), the 4-cycle and the 4-clique totals by type multiset.
+// k_node_aggr), the up lists' typed offsets, the 4-cycle and the 4-clique totals by type
+// multiset.  Sets TG_DERR_TOTALS in err (may be NULL) where they contradict one another.
 int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t *theta,
-                  const uint32_t *dlow, const unsigned long long *c4w, const unsigned long long *k4,
-                  unsigned long long *hist, cudaStream_t s);
+                  const uint32_t *dlow, const int32_t *utoff, const unsigned long long *c4w,
+                  const unsigned long long *k4, unsigned long long *hist, unsigned *err, cudaStream_t s);
 
 // Counts through Alg. 1's typed triangle counts (tg_reuse.cu).  lists.order is
 // the grouped order of all M edges; order[0..count) the edges to count.  With
@@ -222,10 +224,12 @@ int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t 
 // With part.count > 1 (global sums only, k = 4), the call is one share of a
 // split count: order[0..count) is its slice of the edges, and the 4-cycle and
 // 4-clique totals (with their correction of the sums) are the part's own.
+// err: device error bits of the whole-graph sums (tg_sum_totals).
 int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
                    const uint32_t *order, int64_t count, uint64_t *rows, int64_t width,
                    unsigned long long *hist, const tg_tune &t, cudaStream_t s,
-                   const tg_part &part = tg_part(), uint64_t *const *rowmap = nullptr);
+                   const tg_part &part = tg_part(), uint64_t *const *rowmap = nullptr,
+                   unsigned *err = nullptr);
 
 // Per-edge rows of the whole graph into device memory `rows` (M x
 // tg_slots(L, k, level)), queued on s (tg_count.cu).

@@ -1191,7 +1191,7 @@ int tg_edge_units(const tg_graph *g, const uint32_t *ord, int64_t cnt, cudaStrea
 int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
                    const uint32_t *order, int64_t count, uint64_t *rows, int64_t width,
                    unsigned long long *hist, const tg_tune &t, cudaStream_t s,
-                   const tg_part &part, uint64_t *const *rowmap) {
+                   const tg_part &part, uint64_t *const *rowmap, unsigned *err) {
     if (count <= 0 && part.count <= 1) return TG_OK;  // a share of a split count still enumerates
     const int L = g->L, L2 = L * L;
     const int64_t M = g->M, n = g->n;
@@ -1304,7 +1304,7 @@ int tg_reuse_count(const tg_graph *g, int k, int level, const tg_lists &lists,
         if (k == 4) TG_TRY(tg_cyc_cliques(g, k4e.p, g4k.p, work, t, fast ? part : tg_part(), s));
         TG_TRY_CUDA(cudaEventRecord(g_last.ev[4], s));
         if (whole) {
-            TG_TRY(tg_sum_totals(g, k, tau.p, theta.p, dsum.p, g4c.p, g4k.p, hist, s));
+            TG_TRY(tg_sum_totals(g, k, tau.p, theta.p, dsum.p, lists.utoff, g4c.p, g4k.p, hist, err, s));
             TG_TRY_CUDA(cudaEventRecord(g_last.ev[5], s));
             g_last.edges = (uint64_t)count;
             g_last.ready = true;

@@ -23,6 +23,19 @@
 // Every N is summed as a count of copies (no division of a wrapped sum), so
 // the sums equal those of the per-edge pass (tg_edges.cu) mod 2^64.
 //
+// The factors |E(H)| are put in here, so their division afterwards tells nothing of the
+// totals (but for triangles).  What the totals say of one another is checked instead:
+//   per node       Theta_v[b][c] = Theta_v[c][b], and Theta_v[b][b] is even (both count
+//                  triangles at v, from the tau of different edges);
+//   per type pair  the triangles at the nodes by the types of the other two (Theta) are
+//                  those of the edges between the types (tau);
+//   per type       sum of D[.][a] = sum over w of u_w d_w^a, less the edges whose end of
+//                  smaller id has type a (u_w: neighbours of smaller id);
+//   per multiset   no induced count is negative (3-paths, 4-paths, 4-cycles, tailed
+//                  triangles, diamonds: below 2^60 while 2M < 2^31; stars may wrap).
+// A wrong tau, Theta or D, or 4-cycle and 4-clique totals that do not fit them, set
+// TG_DERR_TOTALS.
+//
 // The per-edge pass gathers three rows per triangle node and holds 3 L^2
 // 64-bit sums per edge; here an edge costs its tau row and a node its Theta
 // and D rows, read once.
@@ -56,7 +69,8 @@ __device__ __forceinline__ int64_t key3(int a, int b, int c) {
     return colex3(a, b, c);
 }
 
-// sums (zeroed): [edges: E2][P3: n3][H2: n3][P4: n4][S4: n4][TT: n4][D: n4]
+// sums (zeroed): [edges: E2][P3: n3][H2: n3][P4: n4][S4: n4][TT: n4][D: n4], then (k = 4)
+// the triangles of the nodes and of the edges by type pair [P] [P], the defects of D [L]
 struct SumParams {
     const int32_t *toff;
     const uint8_t *ntype;
@@ -64,14 +78,72 @@ struct SumParams {
     const uint32_t *tau;
     const uint32_t *theta;  // k = 4
     const uint32_t *dlow;   // k = 4: sum over w in Gamma_v^s, w > v, of d_w^a - [a = phi_v]
+    const int32_t *utoff;   // typed offsets of the up lists
+    unsigned *err;
     int64_t n, M;
     int32_t L, P, k;
     int64_t e2, n3, n4;
+    int64_t eblocks;  // CTAs of the edge totals; those after them make the checks
     unsigned long long *sums;
 };
 
 __device__ __forceinline__ void flush_nonzero(unsigned long long *dst, unsigned long long v) {
     if (v) atomicAdd(dst, v);
+}
+
+// ----------------------------------------------------------------- checks --
+// What Theta and D say of tau, of one another and of the degrees (see the head).  A
+// thread per entry of a row, the same entry of every row it takes, so its sums stay in
+// registers.  One more pass over the rows, by further CTAs of the edge totals' launch
+// (CTA `block` of `blocks`): counts of ER 100K/1M and of a power law of 8M edges take as
+// long as without it (1,518 us and 30.8 ms), 25 and 110 us longer with a launch of its
+// own, 45 and 500 us with the same sums inside k_sum_nodes, in its registers.
+// part: P + L words.
+constexpr int kCheckThreads = 256;
+constexpr int kCheckBatch = 4;  // rows in flight
+
+__device__ __forceinline__ void sum_checks(const SumParams &p, int64_t block, int64_t blocks,
+                                           unsigned long long *part) {
+    const int L = p.L, L2 = L * L, P = p.P, R = kCheckThreads / L2;
+    for (int x = threadIdx.x; x < P + L; x += kCheckThreads) part[x] = 0ull;
+    __syncthreads();
+    const int q = threadIdx.x % L2, s = q / L, a = q % L;
+    // triangles of (s, a); D of column a; thread q < L: the other side of D's column q
+    unsigned long long tri = 0, dsum = 0, defect = 0;
+    bool bad = false;
+    const int64_t step = blocks * R;
+    if (threadIdx.x < R * L2)
+        for (int64_t v0 = block * R + threadIdx.x / L2; v0 < p.n; v0 += step * kCheckBatch) {
+            uint32_t t[kCheckBatch], m[kCheckBatch], x[kCheckBatch];
+#pragma unroll
+            for (int y = 0; y < kCheckBatch; ++y) {
+                const int64_t v = v0 + y * step;
+                const bool in = v < p.n;
+                t[y] = in ? __ldg(p.theta + v * L2 + q) : 0u;
+                m[y] = in ? __ldg(p.theta + v * L2 + a * L + s) : 0u;
+                x[y] = in ? __ldg(p.dlow + v * L2 + q) : 0u;
+                if (q >= L || !in) continue;
+                const int32_t *to = p.toff + v * (L + 1);
+                const uint32_t up = (uint32_t)__ldg(p.utoff + v * (L + 1) + L);
+                defect += (unsigned long long)up * (uint32_t)(__ldg(to + q + 1) - __ldg(to + q));
+                if (q == p.ntype[v]) defect -= (uint32_t)__ldg(to + L) - up;
+            }
+#pragma unroll
+            for (int y = 0; y < kCheckBatch; ++y) {
+                bad |= t[y] != m[y] || (s == a && (t[y] & 1u));
+                tri += s == a ? t[y] >> 1 : t[y];
+                dsum += x[y];
+            }
+        }
+    if (threadIdx.x < R * L2) {
+        if (s <= a) flush_nonzero(part + pair_index(L, s, a), tri);
+        flush_nonzero(part + P + a, 0ull - dsum);
+        if (q < L) flush_nonzero(part + P + q, defect);
+    }
+    if (bad && p.err) atomicOr(p.err, TG_DERR_TOTALS);
+    __syncthreads();
+    unsigned long long *out = p.sums + p.e2 + 2 * p.n3 + 4 * p.n4;  // [P] triangles, [P] the edges', [L]
+    for (int x = threadIdx.x; x < P + L; x += kCheckThreads) flush_nonzero(out + (x < P ? x : x + P), part[x]);
 }
 
 // ------------------------------------------------------------ edge totals --
@@ -82,6 +154,7 @@ __device__ __forceinline__ void flush_nonzero(unsigned long long *dst, unsigned 
 // lane q holds the products of type pairs q, q + 32, ... in registers and adds
 // them to the CTA's table once per type pair present, on distinct addresses.
 constexpr int kSumWarps = 8;
+static_assert(kSumWarps * 32 == kCheckThreads, "the checks run in the same launch");
 
 template <int LP>
 __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
@@ -91,6 +164,10 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
     const bool four = p.k == 4;
     // [P][L] sums of tau, [P] edges, (k = 4) [P][P] products, then the rows
     unsigned long long *ts = reinterpret_cast<unsigned long long *>(smem);
+    if (blockIdx.x >= p.eblocks) {  // k = 4: P (L + 1 + P) words and more
+        sum_checks(p, blockIdx.x - p.eblocks, gridDim.x - p.eblocks, ts);
+        return;
+    }
     unsigned long long *ne = ts + P * L;
     unsigned long long *tab = ne + P;
     const int words = P * L + P + (four ? P * P : 0);
@@ -106,7 +183,7 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
         if (q < P) unpair(L, q, pa[z], pb[z]);
     }
     __syncthreads();
-    const int64_t nw = (int64_t)gridDim.x * kSumWarps;
+    const int64_t nw = p.eblocks * kSumWarps;
     for (int64_t c = (int64_t)blockIdx.x * kSumWarps + warp; c * 32 < p.M; c += nw) {
         const int64_t e0 = c * 32;
         const int cnt = (int)min((int64_t)32, p.M - e0);
@@ -181,6 +258,12 @@ __global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
             atomicAdd(s_d + key4(i, j, a, b), v);
         }
     }
+    if (!four) return;
+    for (int q = threadIdx.x; q < P; q += blockDim.x) {
+        unsigned long long v = 0;
+        for (int a = 0; a < L; ++a) v += ts[q * L + a];
+        flush_nonzero(s_d + p.n4 + P + q, v);
+    }
 }
 
 // ------------------------------------------------------------ node totals --
@@ -211,7 +294,7 @@ __device__ __forceinline__ unsigned long long c3(uint32_t x) {
 }
 
 template <int LP>
-__global__ void __launch_bounds__(kNodeThreads) k_sum_nodes(SumParams p) {
+__global__ void __launch_bounds__(kNodeThreads, LP <= 4 ? 4 : LP <= 8 ? 2 : 1) k_sum_nodes(SumParams p) {
     constexpr int kTeam = LP * LP < 32 ? 32 : LP * LP;
     constexpr int kTeams = kNodeThreads / kTeam;
     constexpr int kN4 = (LP + 2) * (LP + 1) * LP / 6;  // triples of types
@@ -331,31 +414,43 @@ __global__ void __launch_bounds__(kNodeThreads) k_sum_nodes(SumParams p) {
         flush_nonzero(z < p.n3 ? out3 + z : out4 + (z - p.n3), h3[z]);
 }
 
-// The undivided sums from the totals (and the 4-cycles W, 4-cliques K).
-__global__ void k_sum_combine(const unsigned long long *sums, int64_t e2, int64_t n3, int64_t n4,
+// The undivided sums from the totals (and the 4-cycles W, 4-cliques K), and the checks
+// of the totals.
+__global__ void k_sum_combine(const unsigned long long *sums, int64_t e2, int64_t n3, int64_t n4, int L,
                               int k, const unsigned long long *w, const unsigned long long *k4,
-                              unsigned long long *hist) {
+                              unsigned long long *hist, unsigned *err) {
     const int64_t off2 = e2 + n3, off4 = off2 + n3, len = off4 + (k == 4 ? n4 : 0);
+    const int P = L * (L + 1) / 2;
+    const unsigned long long *tri = sums + off4 + 4 * n4, *etri = tri + P, *defect = etri + P;
+    bool bad = false;
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < len;
          x += (int64_t)gridDim.x * blockDim.x) {
         if (x < e2) {
             hist[x] = sums[x];
         } else if (x < off2) {
-            hist[x] = 2 * sums[x] - 2 * sums[x + n3];
+            const unsigned long long p3 = sums[x] - sums[x + n3];
+            hist[x] = 2 * p3;
+            bad |= (long long)p3 < 0;
         } else if (x < off4) {
             hist[x] = sums[x];
         } else {
             const int64_t r = x - off4;
             const unsigned long long p4 = sums[x], s4 = sums[x + n4], tt = sums[x + 2 * n4],
                                      d = sums[x + 3 * n4], c = w[r], q = k4[r];
-            hist[off4 + r] = 3 * (p4 - 2 * tt + 6 * d - 4 * c - 12 * q);
+            const unsigned long long h3 = p4 - 2 * tt + 6 * d - 4 * c - 12 * q, h5 = c - d + 3 * q,
+                                     h6 = tt - 4 * d + 12 * q, h7 = d - 6 * q;
+            hist[off4 + r] = 3 * h3;
             hist[off4 + n4 + r] = 3 * (s4 - tt + 2 * d - 4 * q);
-            hist[off4 + 2 * n4 + r] = 4 * (c - d + 3 * q);
-            hist[off4 + 3 * n4 + r] = 4 * (tt - 4 * d + 12 * q);
-            hist[off4 + 4 * n4 + r] = 5 * (d - 6 * q);
+            hist[off4 + 2 * n4 + r] = 4 * h5;
+            hist[off4 + 3 * n4 + r] = 4 * h6;
+            hist[off4 + 4 * n4 + r] = 5 * h7;
             hist[off4 + 5 * n4 + r] = 6 * q;
+            bad |= (long long)(h3 | h5 | h6 | h7) < 0;
+            if (r < P) bad |= tri[r] != etri[r];  // L <= P <= C(L + 3, 4)
+            if (r < L) bad |= defect[r] != 0ull;
         }
     }
+    if (bad && err) atomicOr(err, TG_DERR_TOTALS);
 }
 
 size_t edges_smem(const SumParams &p, int LP) {
@@ -364,7 +459,7 @@ size_t edges_smem(const SumParams &p, int LP) {
 }
 
 template <int LP>
-int launch_sums(const SumParams &p, cudaStream_t s) {
+int launch_sums(SumParams p, cudaStream_t s) {
     TG_TRY(tg_allow_max_smem((const void *)k_sum_edges<LP>));
     TG_TRY(tg_allow_max_smem((const void *)k_sum_nodes<LP>));
     const size_t es = edges_smem(p, LP);
@@ -374,8 +469,13 @@ int launch_sums(const SumParams &p, cudaStream_t s) {
     TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nper, k_sum_nodes<LP>, kNodeThreads, ns));
     if (eper < 1 || nper < 1) return TG_EINVAL;
     const int64_t sms = tg_num_sms();
-    const int64_t eg = std::min<int64_t>(sms * eper, (p.M + kSumWarps * 32 - 1) / (kSumWarps * 32));
-    k_sum_edges<LP><<<(unsigned)std::max<int64_t>(1, eg), kSumWarps * 32, es, s>>>(p);
+    p.eblocks = std::max<int64_t>(1, std::min<int64_t>(sms * eper, (p.M + kSumWarps * 32 - 1) / (kSumWarps * 32)));
+    int64_t checks = 0;
+    if (p.k == 4) {
+        const int64_t rows = (int64_t)(kCheckThreads / (p.L * p.L)) * kCheckBatch;
+        checks = std::max<int64_t>(1, std::min<int64_t>(sms * eper, (p.n + rows - 1) / rows));
+    }
+    k_sum_edges<LP><<<(unsigned)(p.eblocks + checks), kSumWarps * 32, es, s>>>(p);
     tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     constexpr int kTeams = kNodeThreads / (LP * LP < 32 ? 32 : LP * LP);
@@ -389,8 +489,8 @@ int launch_sums(const SumParams &p, cudaStream_t s) {
 }  // namespace
 
 int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t *theta,
-                  const uint32_t *dlow, const unsigned long long *c4w, const unsigned long long *k4,
-                  unsigned long long *hist, cudaStream_t s) {
+                  const uint32_t *dlow, const int32_t *utoff, const unsigned long long *c4w,
+                  const unsigned long long *k4, unsigned long long *hist, unsigned *err, cudaStream_t s) {
     if (g->max_degree >= ((int64_t)1 << 27)) return TG_EOVERFLOW;  // as the per-edge pass
     SumParams p{};
     p.toff = g->toff;
@@ -399,6 +499,8 @@ int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t 
     p.tau = tau;
     p.theta = theta;
     p.dlow = dlow;
+    p.utoff = utoff;
+    p.err = err;
     p.n = g->n;
     p.M = g->M;
     p.L = g->L;
@@ -407,7 +509,7 @@ int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t 
     p.e2 = tg_binom(g->L + 1, 2);
     p.n3 = tg_binom(g->L + 2, 3);
     p.n4 = tg_binom(g->L + 3, 4);
-    const int64_t len = p.e2 + 2 * p.n3 + (k == 4 ? 4 * p.n4 : 0);
+    const int64_t len = p.e2 + 2 * p.n3 + (k == 4 ? 4 * p.n4 + 2 * p.P + p.L : 0);
     DevBuf<unsigned long long> sums;
     if (!sums.alloc(len, s)) return TG_ENOMEM;
     TG_TRY_CUDA(cudaMemsetAsync(sums.p, 0, len * 8, s));
@@ -418,7 +520,8 @@ int tg_sum_totals(const tg_graph *g, int k, const uint32_t *tau, const uint32_t 
         TG_TRY(launch_sums<8>(p, s));
     else
         TG_TRY(launch_sums<16>(p, s));
-    k_sum_combine<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(sums.p, p.e2, p.n3, p.n4, k, c4w, k4, hist);
+    k_sum_combine<<<(unsigned)((len + 255) / 256), 256, 0, s>>>(sums.p, p.e2, p.n3, p.n4, p.L, k, c4w, k4, hist,
+                                                                err);
     tg_note_launch();
     TG_TRY_CUDA(cudaGetLastError());
     return TG_OK;
