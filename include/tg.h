@@ -122,7 +122,10 @@ typedef struct {
     int64_t M;             /* undirected edges after simplification      */
     int64_t n_nonisolated; /* nodes with degree >= 1                     */
     int64_t max_degree;    /* Delta                                      */
-    int64_t device_bytes;  /* device memory held by the graph            */
+    int64_t device_bytes;  /* device memory held by the graph: the CSR and
+                              what counts have added so far and keep (the
+                              first one, oriented lists of 16 M + 4 n (L + 1)
+                              + 8 (n + 1) bytes; a shard, its order of 4 M) */
     int32_t L;             /* node types                                 */
     int32_t reserved;
 } tg_info;

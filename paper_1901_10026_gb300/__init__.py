@@ -246,7 +246,16 @@ class Graph:
         _check(lib().tg_graph_info(self._h, ctypes.byref(info)), "tg_graph_info")
         self.n, self.m_input, self.M = info.n, info.m_input, info.M
         self.n_nonisolated, self.max_degree = info.n_nonisolated, info.max_degree
-        self.device_bytes, self.L = info.device_bytes, info.L
+        self._device_bytes, self.L = info.device_bytes, info.L
+
+    @property
+    def device_bytes(self) -> int:
+        """Device memory the graph holds now (its counts add to it); once closed, what it held last asked."""
+        if self._h is not None:
+            info = _Info()
+            _check(lib().tg_graph_info(self._h, ctypes.byref(info)), "tg_graph_info")
+            self._device_bytes = info.device_bytes
+        return self._device_bytes
 
     @property
     def handle(self):

@@ -1055,6 +1055,14 @@ static int get_sched(const tg_graph *g, cudaStream_t s, tg_sched **out) {
     return TG_OK;
 }
 
+int64_t tg_sched_bytes(const tg_graph *g) {
+    std::lock_guard<std::mutex> lk(g->mu);
+    const tg_sched *sc = g->sched;
+    if (!sc) return 0;
+    return (g->n + 1) * 8 + g->n * (g->L + 1) * 4 + 4 * g->M * 4 + (sc->sorted ? g->M * 4 : 0) +
+           (sc->s ? g->n * 8 : 0);
+}
+
 int tg_graph_lists(const tg_graph *g, const tg_lists **out, cudaStream_t s) {
     tg_sched *sc = nullptr;
     TG_TRY(get_sched(g, s, &sc));

@@ -487,7 +487,7 @@ extern "C" int tg_graph_info(const tg_graph *g, tg_info *info) {
     info->M = g->M;
     info->n_nonisolated = g->n_nonisolated;
     info->max_degree = g->max_degree;
-    info->device_bytes = g->device_bytes;
+    info->device_bytes = g->device_bytes + tg_sched_bytes(g);
     info->L = g->L;
     info->reserved = 0;
     return TG_OK;

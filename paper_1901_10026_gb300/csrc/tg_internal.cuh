@@ -160,6 +160,8 @@ static inline int64_t tg_binom(int64_t a, int64_t b) {
     return r;
 }
 
+// Device bytes of the schedule that a graph's counts have built so far (tg_count.cu).
+int64_t tg_sched_bytes(const tg_graph *g);
 // Free the lazily built schedule of a graph (tg_count.cu).
 void tg_sched_free(tg_graph *g);
 // Stream-ordered frees for a graph used only on stream s (no device sync).
