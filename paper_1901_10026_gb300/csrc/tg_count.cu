@@ -924,10 +924,9 @@ extern "C" int tg_autotune(const tg_graph *g, int32_t k, tg_tune *best, void *st
     if (!out.alloc(tg_global_len(g->L, k), s)) return TG_ENOMEM;
     cudaEvent_t ev[2];
     TG_TRY_CUDA(cudaEventCreate(&ev[0]));
-    if (cudaEventCreate(&ev[1]) != cudaSuccess) {
-        cudaEventDestroy(ev[0]);
-        return TG_ECUDA;
-    }
+    const cudaError_t made = cudaEventCreate(&ev[1]);
+    if (made != cudaSuccess) cudaEventDestroy(ev[0]);
+    TG_TRY_CUDA(made);
     // one count under candidate c, in milliseconds
     auto timed = [&](const tg_tune &c, float &ms) -> int {
         TG_TRY(tg_set_tune(&c));
@@ -1042,9 +1041,13 @@ static int get_sched(const tg_graph *g, cudaStream_t s, tg_sched **out) {
     }
     tg_sched *sc = new (std::nothrow) tg_sched();
     if (!sc) return TG_ENOMEM;
-    int r = tg_build_lists(g, sc->lists, s);
-    // other threads may read the lists on their own streams from here on
-    if (r == TG_OK && cudaStreamSynchronize(s) != cudaSuccess) r = TG_ECUDA;
+    auto make = [&]() -> int {
+        TG_TRY(tg_build_lists(g, sc->lists, s));
+        // other threads may read the lists on their own streams from here on
+        TG_TRY_CUDA(cudaStreamSynchronize(s));
+        return TG_OK;
+    };
+    const int r = make();
     if (r != TG_OK) {
         sched_dfree(sc, s);
         delete sc;
