@@ -122,12 +122,16 @@ int tg_attach_arcs(tg_graph *g, const int32_t *src, const int32_t *dst, int64_t 
 int tg_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, cudaStream_t s);
 int tg_scan_i64(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s);
 // LSD radix sort of uint64 keys on their low `bits` bits (stable).  `keys` and
-// `tmp` hold n entries each; *result points at whichever holds the output.
+// `tmp` hold n entries each; *result points at whichever holds the output.  looks:
+// idle looks at a late tile before its keys are counted by the tile that needs them
+// (-1: no look at all; tests).
+constexpr int TG_SORT_LOOKS = 1 << 18;
 int tg_radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int bits, cudaStream_t s,
-                      uint64_t **result);
+                      uint64_t **result, int looks = TG_SORT_LOOKS);
 // Same, carrying a uint32 value per key (vals/vtmp); *vresult gets the output.
 int tg_radix_sort_kv(uint64_t *keys, uint64_t *tmp, uint32_t *vals, uint32_t *vtmp, int64_t n,
-                     int bits, cudaStream_t s, uint64_t **result, uint32_t **vresult);
+                     int bits, cudaStream_t s, uint64_t **result, uint32_t **vresult,
+                     int looks = TG_SORT_LOOKS);
 
 int tg_bitlen(uint64_t x);  // number of bits needed to represent x (0 -> 0)
 

@@ -292,7 +292,7 @@ int tg_scan_i64(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s) {
 // A tile's counts per digit are published in two steps, its own count and the
 // sum over all tiles up to it, each a word with its state in the top bits.  A tile
 // waits only for tiles of smaller tickets, which are running or done, and for at
-// most kSortSpin looks at their words: then it counts the keys before it itself.
+// most TG_SORT_LOOKS idle looks at their words: then it counts the keys before it itself.
 // Up to kSmallKeys keys one CTA makes all passes in shared memory.
 //
 // Measured (CSR build, before -> now): R-MAT-21 (33.6M draws) 14.6 -> 8.8 ms, ER
@@ -305,7 +305,6 @@ constexpr int kSortThreads = 512;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
-constexpr int kSortSpin = 1 << 18;
 constexpr unsigned long long kSortOwn = 1ull << 62, kSortSum = 2ull << 62, kSortMask = kSortOwn - 1ull;
 constexpr int kSmallThreads = 1024, kSmallItems = 12, kSmallKeys = kSmallThreads * kSmallItems;
 
@@ -405,7 +404,8 @@ template <bool kVals>
 __global__ void __launch_bounds__(kSortThreads) k_sort_digit(const uint64_t *in, uint64_t *out,
                                                              const uint32_t *vin, uint32_t *vout,
                                                              int64_t n, int shift, const uint32_t *counts,
-                                                             unsigned long long *state, uint32_t *ticket) {
+                                                             unsigned long long *state, uint32_t *ticket,
+                                                             int looks) {
     extern __shared__ __align__(16) unsigned char smem[];
     SortSmem<kVals> &sm = *reinterpret_cast<SortSmem<kVals> *>(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_digit(const uint64_t *in,
         int spin = 0;
         for (int64_t t = (int64_t)tile - 1; t >= 0;) {
             const unsigned long long w = *(volatile unsigned long long *)(state + (size_t)t * 256 + tid);
-            if (!(w & ~kSortMask)) {
-                if (++spin > kSortSpin) {
+            if (!(w & ~kSortMask) || looks < 0) {
+                if (++spin > looks) {
                     sm.late = 1u;
                     break;
                 }
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_sort_small(uint64_t *keys, ui
 
 template <bool kVals>
 int sort_impl(uint64_t *keys, uint64_t *tmp, uint32_t *vals, uint32_t *vtmp, int64_t n, int bits,
-              cudaStream_t s, uint64_t **result, uint32_t **vresult) {
+              cudaStream_t s, uint64_t **result, uint32_t **vresult, int looks) {
     *result = keys;
     if (vresult) *vresult = vals;
     if (n <= 1 || bits <= 0) return TG_OK;
@@ -573,7 +573,7 @@ int sort_impl(uint64_t *keys, uint64_t *tmp, uint32_t *vals, uint32_t *vtmp, int
     uint32_t *va = vals, *vb = vtmp;
     for (int p = 0; p < passes; ++p) {
         k_sort_digit<kVals><<<(unsigned)tiles, kSortThreads, sizeof(SortSmem<kVals>), s>>>(
-            a, b, va, vb, n, 8 * p, counts + p * 256, buf.p + (size_t)p * tiles * 256, tickets + p);
+            a, b, va, vb, n, 8 * p, counts + p * 256, buf.p + (size_t)p * tiles * 256, tickets + p, looks);
         tg_note_launch();
         TG_TRY_CUDA(cudaGetLastError());
         std::swap(a, b);
@@ -587,11 +587,11 @@ int sort_impl(uint64_t *keys, uint64_t *tmp, uint32_t *vals, uint32_t *vtmp, int
 }  // namespace
 
 int tg_radix_sort_kv(uint64_t *keys, uint64_t *tmp, uint32_t *vals, uint32_t *vtmp, int64_t n,
-                     int bits, cudaStream_t s, uint64_t **result, uint32_t **vresult) {
-    return sort_impl<true>(keys, tmp, vals, vtmp, n, bits, s, result, vresult);
+                     int bits, cudaStream_t s, uint64_t **result, uint32_t **vresult, int looks) {
+    return sort_impl<true>(keys, tmp, vals, vtmp, n, bits, s, result, vresult, looks);
 }
 
 int tg_radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int bits, cudaStream_t s,
-                      uint64_t **result) {
-    return sort_impl<false>(keys, tmp, nullptr, nullptr, n, bits, s, result, nullptr);
+                      uint64_t **result, int looks) {
+    return sort_impl<false>(keys, tmp, nullptr, nullptr, n, bits, s, result, nullptr, looks);
 }

@@ -115,3 +115,20 @@ extern "C" int tgi_sum_totals(const tg_graph *g, int k, int mistake, int64_t at,
     *err = down(derr.p, 1)[0];
     return TG_OK;
 }
+
+// The radix sort on host keys (and values, unless NULL), in place.
+extern "C" int tgi_sort(int64_t n, int bits, int looks, uint64_t *keys, uint32_t *vals) {
+    const std::vector<uint64_t> k(keys, keys + n);
+    const std::vector<uint32_t> v(vals ? vals : (const uint32_t *)keys, vals ? vals + n : (const uint32_t *)keys + n);
+    const Up<uint64_t> k1(k), k2(k);
+    const Up<uint32_t> v1(v), v2(v);
+    uint64_t *kr = nullptr;
+    uint32_t *vr = nullptr;
+    const int r = vals ? tg_radix_sort_kv(k1.p, k2.p, v1.p, v2.p, n, bits, nullptr, &kr, &vr, looks)
+                       : tg_radix_sort_u64(k1.p, k2.p, n, bits, nullptr, &kr, looks);
+    if (r != TG_OK) return r;
+    if (cudaDeviceSynchronize() != cudaSuccess) return TG_ECUDA;
+    cudaMemcpy(keys, kr, n * 8, cudaMemcpyDeviceToHost);
+    if (vals) cudaMemcpy(vals, vr, n * 4, cudaMemcpyDeviceToHost);
+    return TG_OK;
+}
