@@ -361,25 +361,6 @@ __device__ __forceinline__ int classify(const EdgeCtx &c, uint32_t w) {
     return contains(c.adj, c.bj, c.toj, w) ? CLS_SJ : CLS_I;
 }
 
-__device__ __forceinline__ void record_marked(int *cnt, int P, int ocls, int okid, int pr,
-                                              int rcls, int rid) {
-    atomicAdd(&cnt[(ocls == CLS_T ? C_G8 : C_G3) * P + pr], -1);
-    if (ocls == CLS_SI) {
-        if (rcls == CLS_SI && rid < okid) atomicAdd(&cnt[C_G7 * P + pr], 1);
-    } else if (ocls == CLS_SJ) {
-        if (rcls == CLS_SJ && rid < okid)
-            atomicAdd(&cnt[C_G7 * P + pr], 1);
-        else if (rcls == CLS_SI)
-            atomicAdd(&cnt[C_G6 * P + pr], 1);
-    } else {
-        if (rcls == CLS_T) {
-            if (rid < okid) atomicAdd(&cnt[C_G12 * P + pr], 1);
-        } else {
-            atomicAdd(&cnt[C_G10 * P + pr], 1);
-        }
-    }
-}
-
 // Orbit row incremented by a marked pair (w_k of class ocls, w_r of class
 // rcls, lower = w_r < w_k), or -1: Alg. 2 (g7 inside one S-set with the
 // symmetry break, g6 from the S_j pass) and Alg. 3 (g12 inside T with the

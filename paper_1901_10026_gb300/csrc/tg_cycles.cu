@@ -95,7 +95,6 @@ struct C4Params {
     const struct C4Unit *wunits;  // walk kernel: position ranges of the split anchors
     int64_t n_units;
     int32_t phase;             // split kernel: the pass of this launch
-    int32_t mark;              // pass 0 marks far ends in the slot's bitmap
     unsigned long long *work;  // [4]: wedges
     // dense waves (global mode): the costly anchors heavy[q], their walk
     // positions (member costs d_u, exclusive prefix per anchor at pbase[q]),
@@ -148,16 +147,14 @@ __device__ __forceinline__ C4Smem c4_smem(unsigned char *smem, int TM, int acc_l
 // One pass over one tile of anchor a's list (list positions [tile, tile_end),
 // at most p.tile of them): the members u (neighbours ranked below a) of the
 // tile and, for each, the entries b of u's list ranked below a.  The members'
-// lists are walked as one sequence of positions, of which only [pos_lo, pos_hi)
-// is taken.  Pass 0 counts the middles per (b, type), and lists each b the
-// first time it is met (in `list`, count in *nb) or marks it in the slot's
-// bitmap (p.mark); pass 1 (per-edge mode only) adds the cycles each wedge
-// closes to its two edges.  Returns the length of the tile's sequence.  Called
-// by every thread of the CTA (it holds barriers).
-__device__ int64_t c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int ta, int64_t ba,
-                           int tile, int tile_end, int64_t pos_lo, int64_t pos_hi, int phase,
-                           uint32_t *cnt, uint32_t *list, unsigned int *nb,
-                           unsigned long long &wk) {
+// lists are walked as one sequence of positions.  Pass 0 counts the middles per
+// (b, type), and lists each b the first time it is met (in `list`, count in *nb)
+// or, without a list, marks it in the slot's bitmap; pass 1 (per-edge mode only)
+// adds the cycles each wedge closes to its two edges.  Called by every thread of
+// the CTA (it holds barriers).
+__device__ void c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int ta, int64_t ba,
+                        int tile, int tile_end, int phase, uint32_t *cnt, uint32_t *list,
+                        unsigned int *nb, unsigned long long &wk) {
     const int tid = threadIdx.x;
     const int L = p.L, L2 = L * L, TM = p.tile;
     const int x = tile + tid;
@@ -189,10 +186,7 @@ __device__ int64_t c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int 
     if (phase == 1)
         for (int q = tid; q < nmem * L2; q += blockDim.x) sm.acc[q] = 0ull;
     __syncthreads();
-    const int64_t lim = total < pos_hi ? total : pos_hi;
-    for (int64_t base = pos_lo > 0 ? pos_lo : 0; base < lim; base += blockDim.x) {
-        const int64_t pos = base + tid;
-        if (pos >= lim) continue;
+    for (int64_t pos = tid; pos < total; pos += blockDim.x) {
         int lo = 0, hi = nmem - 1;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
@@ -215,7 +209,7 @@ __device__ int64_t c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int 
             if (list) {
                 // the first wedge to reach b lists it
                 if (!(atomicOr(bw, bit) & bit)) list[atomicAdd(nb, 1u)] = b;
-            } else if (p.mark) {
+            } else {
                 atomicOr(bw, bit);  // marks b for the scan of k_c4_pairs
             }
             ++wk;
@@ -255,7 +249,6 @@ __device__ int64_t c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int 
         }
         __syncthreads();
     }
-    return total;
 }
 
 // Far end b of anchor a (counters cb, per type): global mode adds the cycles
@@ -385,12 +378,10 @@ __global__ void __launch_bounds__(kC4Threads) k_c4(C4Params p, const uint32_t *a
         if (tid == 0) *sm.s_nb = 0u;
         __syncthreads();
         for (int tile = 0; tile < da; tile += p.tile)
-            c4_tile(p, sm, a, ta, ba, tile, min(da, tile + p.tile), 0, INT64_MAX, 0, cnt, list,
-                    sm.s_nb, wk);
+            c4_tile(p, sm, a, ta, ba, tile, min(da, tile + p.tile), 0, cnt, list, sm.s_nb, wk);
         if (!p.g4)
             for (int tile = 0; tile < da; tile += p.tile)
-                c4_tile(p, sm, a, ta, ba, tile, min(da, tile + p.tile), 0, INT64_MAX, 1, cnt, list,
-                        sm.s_nb, wk);
+                c4_tile(p, sm, a, ta, ba, tile, min(da, tile + p.tile), 1, cnt, list, sm.s_nb, wk);
         __syncthreads();
         c4_pairs(p, sm, ta, cnt, list, *sm.s_nb, tid, blockDim.x);
     }
@@ -417,8 +408,7 @@ __global__ void __launch_bounds__(kC4Threads) k_c4_split(C4Params p) {
         const uint32_t a = (uint32_t)un.y;
         const int64_t ba = p.rowptr[a];
         uint32_t *cnt = p.scratch + (int64_t)un.x * p.slot_words;
-        c4_tile(p, sm, a, p.ntype[a], ba, un.z, un.w, 0, INT64_MAX, p.phase, cnt, nullptr, nullptr,
-                wk);
+        c4_tile(p, sm, a, p.ntype[a], ba, un.z, un.w, p.phase, cnt, nullptr, nullptr, wk);
     }
     c4_finish(p, sm, wk);
 }
@@ -1473,10 +1463,7 @@ struct K4Params {
     int32_t L, P;
     int32_t cap;               // W entries per warp in shared memory
     unsigned long long *queue;
-    unsigned long long *k4e;   // per-edge mode: M * P, 4-cliques by the types of the two
-                               // other nodes
-    unsigned long long *g4;    // global mode: C(L+3,4) 4-clique counts by type multiset
-    int64_t n4;
+    unsigned long long *k4e;   // M * P, 4-cliques by the types of the two other nodes
     unsigned long long *work;  // [5]: candidate tests, [6]: 4-cliques
     int64_t min_d0;            // only x0 with up lists longer than this
 };
@@ -1488,6 +1475,7 @@ __device__ __forceinline__ void k4_add(unsigned long long *k4e, int64_t e, int P
     atomicAdd(k4e + e * P + pair_index(L, a, b), v);
 }
 
+// 4-cliques per edge, one warp per lowest node x0.
 __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1496,13 +1484,6 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
     int32_t *w_p0 = reinterpret_cast<int32_t *>(w_ent + cap);  // position in x0's list
     int32_t *w_pv = w_p0 + cap;                                  // position in v's list
     uint32_t *xacc = reinterpret_cast<uint32_t *>(w_pv + cap);  // cap * L
-    unsigned long long *h4 = reinterpret_cast<unsigned long long *>(
-        smem + (size_t)kK4Warps * cap * (3 + L) * 4);  // global mode: n4 entries
-    const bool global = p.g4 != nullptr;
-    if (global) {
-        for (int64_t q = threadIdx.x; q < p.n4; q += blockDim.x) h4[q] = 0ull;
-        __syncthreads();
-    }
     const uint32_t below = (1u << lane) - 1u;
     unsigned long long wk_cand = 0, wk_k4 = 0;
 
@@ -1562,7 +1543,7 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
                     continue;
                 }
                 const bool staged = nw <= cap;
-                if (staged && !global)
+                if (staged)
                     for (int q = lane; q < nw * L; q += 32) xacc[q] = 0u;
                 __syncwarp();
                 // every w of W (staged: from shared memory; else re-derived)
@@ -1609,7 +1590,7 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
                                 const uint32_t xe = __ldg(p.uadj + bw + r);
                                 {
                                     ++wk_cand;
-                                    int64_t e0x = -1, evx = -1;
+                                    int64_t e0x = -1;
                                     if (staged) {
                                         int lo = 0, hi = nw;
                                         while (lo < hi) {
@@ -1621,7 +1602,7 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
                                         }
                                         if (lo < nw && w_ent[lo] == xe) {
                                             // (x0,x) and (v,x) are summed per x below
-                                            if (!global) atomicAdd(xacc + lo * L + tw, 1u);
+                                            atomicAdd(xacc + lo * L + tw, 1u);
                                             e0x = 0;
                                         }
                                     } else {
@@ -1630,20 +1611,14 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
                                             const int pxv = find_pos(p.uadj, bv, tov, xe);
                                             if (pxv >= 0) {
                                                 e0x = 0;
-                                                if (!global) {
-                                                    evx = __ldg(p.ueid + bv + pxv);
-                                                    k4_add(p.k4e, __ldg(p.ueid + b0 + px0), P, L,
-                                                           tv, tw, 1ull);
-                                                    k4_add(p.k4e, evx, P, L, t0, tw, 1ull);
-                                                }
+                                                k4_add(p.k4e, __ldg(p.ueid + b0 + px0), P, L, tv, tw, 1ull);
+                                                k4_add(p.k4e, __ldg(p.ueid + bv + pxv), P, L, t0, tw, 1ull);
                                             }
                                         }
                                     }
                                     if (e0x >= 0) {
                                         key = (int)(xe >> TG_TSHIFT);
-                                        if (!global)
-                                            k4_add(p.k4e, __ldg(p.ueid + bw + r), P, L, t0, tv,
-                                                   1ull);
+                                        k4_add(p.k4e, __ldg(p.ueid + bw + r), P, L, t0, tv, 1ull);
                                         ++wk_k4;
                                     }
                                 }
@@ -1652,26 +1627,16 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
                             const unsigned mm = __match_any_sync(kFull, key);
                             if (key >= 0 && lane == __ffs(mm) - 1) {
                                 const unsigned long long c = (unsigned long long)__popc(mm);
-                                if (global) {
-                                    int q0 = t0, q1 = tv, q2 = tw, q3 = key;
-                                    sort2(q0, q1);
-                                    sort2(q2, q3);
-                                    sort2(q0, q2);
-                                    sort2(q1, q3);
-                                    sort2(q1, q2);
-                                    atomicAdd(h4 + colex4(q0, q1, q2, q3), c);
-                                } else {
-                                    k4_add(p.k4e, e0v, P, L, tw, key, c);
-                                    k4_add(p.k4e, e0w, P, L, tv, key, c);
-                                    k4_add(p.k4e, evw, P, L, t0, key, c);
-                                }
+                                k4_add(p.k4e, e0v, P, L, tw, key, c);
+                                k4_add(p.k4e, e0w, P, L, tv, key, c);
+                                k4_add(p.k4e, evw, P, L, t0, key, c);
                             }
                         }
                         if (staged) ++k;
                     }
                     if (!staged) c1 += 32;
                 }
-                if (staged && !global) {
+                if (staged) {
                     __syncwarp();
                     for (int q = lane; q < nw * L; q += 32) {
                         const uint32_t c = xacc[q];
@@ -1685,11 +1650,6 @@ __global__ void __launch_bounds__(kK4Warps * 32) k_k4(K4Params p) {
                 __syncwarp();
             }
         }
-    }
-    if (global) {
-        __syncthreads();
-        for (int64_t q = threadIdx.x; q < p.n4; q += blockDim.x)
-            if (h4[q]) atomicAdd(p.g4 + q, h4[q]);
     }
     if (p.work) {
         if (wk_cand) atomicAdd(p.work + 5, wk_cand);
@@ -2337,7 +2297,6 @@ int tg_cyc_cycles(const tg_graph *g, unsigned long long *c4e, unsigned long long
     p.g4 = g4;
     p.n4 = n4;
     p.work = work;
-    p.mark = 1;
     p.half = 0;
     p.bits_off = n * (L + 1);
 
@@ -2458,23 +2417,7 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     const int L = g->L;
     const bool global = g4 != nullptr;
     const int64_t n4 = tg_binom(L + 3, 4);
-    const size_t hbytes = global ? (size_t)n4 * 8 : 0;
-    const size_t avail = (size_t)tg_smem_optin() - 1024 - hbytes;
-    const size_t per_entry = (size_t)(3 + L) * 4;
-    // W entries staged per warp; hash_slots caps it (a small cap sends large W
-    // sets down the path that tests membership in the global lists instead)
-    int cap = (int)std::min<size_t>(std::min(512, t.hash_slots), avail / kK4Warps / per_entry);
-    cap &= ~31;
-    if (cap < 32) return TG_EINVAL;
-    const size_t smem = (size_t)kK4Warps * cap * per_entry + hbytes;
-    TG_TRY(tg_allow_max_smem((const void *)k_k4));
-    int per_sm = 0;
-    TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_k4, kK4Warps * 32, smem));
-    if (per_sm < 1) per_sm = 1;
-    int64_t grid = (int64_t)tg_num_sms() * per_sm;
-    const int64_t need = (g->n + kK4Warps - 1) / kK4Warps;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
+    const size_t avail = (size_t)tg_smem_optin() - 1024;
     const int64_t n = g->n;
     const tg_lists *up = nullptr;
     TG_TRY(tg_graph_lists(g, &up, s));
@@ -2519,7 +2462,7 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
         int hlg = 5;
         while ((1 << hlg) < 2 * gcap) ++hlg;
         size_t gsmem = h4b + (size_t)kK4GWarps * (gcap + 2 * (1 << hlg)) * 4;
-        while (gsmem > avail + hbytes && gcap > 32) {
+        while (gsmem > avail && gcap > 32) {
             gcap -= 32;
             hlg = 5;
             while ((1 << hlg) < 2 * gcap) ++hlg;
@@ -2541,6 +2484,21 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
         TG_TRY_CUDA(cudaGetLastError());
         return TG_OK;
     }
+    const size_t per_entry = (size_t)(3 + L) * 4;
+    // W entries staged per warp; hash_slots caps it (a small cap sends large W
+    // sets down the path that tests membership in the global lists instead)
+    int cap = (int)std::min<size_t>(std::min(512, t.hash_slots), avail / kK4Warps / per_entry);
+    cap &= ~31;
+    if (cap < 32) return TG_EINVAL;
+    const size_t smem = (size_t)kK4Warps * cap * per_entry;
+    TG_TRY(tg_allow_max_smem((const void *)k_k4));
+    int per_sm = 0;
+    TG_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_k4, kK4Warps * 32, smem));
+    if (per_sm < 1) per_sm = 1;
+    int64_t grid = (int64_t)tg_num_sms() * per_sm;
+    const int64_t need = (g->n + kK4Warps - 1) / kK4Warps;
+    if (grid > need) grid = need;
+    if (grid < 1) grid = 1;
     K4Params p{};
     p.uoff = up->uoff;
     p.uadj = up->uadj;
@@ -2553,8 +2511,6 @@ int tg_cyc_cliques(const tg_graph *g, unsigned long long *k4e, unsigned long lon
     p.cap = cap;
     p.queue = queue.p;
     p.k4e = k4e;
-    p.g4 = g4;
-    p.n4 = n4;
     p.work = work;
     p.min_d0 = bits_max;
     k_k4<<<(unsigned)grid, kK4Warps * 32, smem, s>>>(p); tg_note_launch();
