@@ -404,16 +404,17 @@ typedef struct {
     int32_t hash_slots;  /* slots of the per-edge Gamma_i hash (power of 2);
                             CYCLES kernel: cap on the 4-clique candidates
                             staged per warp and on the per-warp far-end
-                            table of the lightest 4-cycle anchors (global
-                            counts); below 64 the costly 4-cycle anchors are
-                            walked in member tiles instead of warp units    */
+                            table of the lightest 4-cycle anchors; below 64
+                            the costly 4-cycle anchors are walked in member
+                            tiles instead of warp units                     */
     int64_t bitmap_bits; /* cap on the node ids covered by the bitmap       */
     int32_t grid_limit;  /* cap on the CTAs of one counting launch          */
     int32_t edge_pass;   /* CYCLES kernel, k = 4: TG_EDGE_PASS_AUTO keeps the
                             per-edge T sums in memory between two kernels
                             when they fit in a quarter of free memory, else
                             runs the fused kernel; TG_EDGE_PASS_FUSED always
-                            runs the fused kernel                           */
+                            runs the fused kernel, also for whole-graph global
+                            counts, which need no per-edge pass under AUTO  */
     int32_t edge_batch;  /* CYCLES kernel, k = 4: most edges whose T sums are
                             held in memory at once (the per-edge pass runs in
                             batches of work units); 0: as many as fit in a

@@ -9,9 +9,10 @@
 //      so high-degree nodes get small ids and, for an edge, the endpoint with
 //      the larger new id never has the larger degree (the d_i <= d_j
 //      orientation of Thm. "3-node time complexity");
-//   4. one radix sort of the 2M directed entries keyed (src, type, dst) gives
-//      every adjacency list sorted by (type, id); entries are stored packed
-//      as (type << 28) | id;
+//   4. every adjacency list sorted by (type, id), entries packed as
+//      (type << 28) | id: by one radix sort of the 2M directed entries keyed
+//      (src, type, dst), or, where no node has more than kListMax neighbours,
+//      by scattering the entries to their lists and sorting each list apart;
 //   5. per-node type offsets toff[v][t] (start of Gamma_v^t inside row v).
 #include <algorithm>
 #include <stdlib.h>
@@ -165,6 +166,12 @@ __global__ void k_fill_adj(const uint64_t *key, const uint32_t *val, int64_t tot
 // Bound by the scattered 8-byte writes and their adds, then by instructions.  Against
 // keys, radix passes and a fill: ER 1M/5M 0.93 -> 0.27 ms (the k = 3 count 2.54 -> 1.89),
 // ER 100K/1M 0.22 -> 0.05 (1.70 -> 1.52), ER 1000 532 -> 486 us in all.
+//
+// The line at 64: whole builds by radix passes and by lists took 0.46 and 0.34 ms at a
+// mean degree of 10 (100,000 nodes), 0.71 and 0.49 at 30 (longest list 59).  With eight
+// entries a lane, for lists up to 128, they took 0.51 at 30 and 1.23 ms where four
+// entries take 1.10 (1M nodes, mean degree 10), but 0.71 against 1.03 by radix passes at
+// a mean degree of 60 (longest list 97): a second instance would pay there.
 constexpr int kListMax = 64;
 constexpr int kListLanes = 16;  // lanes of a list, up to 4 entries each
 

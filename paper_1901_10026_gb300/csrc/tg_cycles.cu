@@ -251,9 +251,6 @@ __device__ void c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int ta,
     }
 }
 
-// Far end b of anchor a (counters cb, per type): global mode adds the cycles
-// per type pair of middles (C(c_t, 2) for t = t', c_t c_t' for t < t') under
-// the multiset {a, b, t, t'}; both modes then clear b's counters.
 // The cycles of one far end b (type tb) of an anchor of type ta, from its
 // middle counts c[t] (t < L): C(c_t, 2) for t = t' and c_t c_t' for t < t',
 // each under the multiset {ta, tb, t, t'}, into the shared histogram h4.  Only
@@ -286,6 +283,8 @@ __device__ __forceinline__ void c4_add(unsigned long long *h4, int L, int ta, in
     }
 }
 
+// Far end b of anchor a (counters cb, per type): global mode adds its cycles; both
+// modes then clear b's counters.
 __device__ __forceinline__ void c4_one(const C4Params &p, unsigned long long *h4, int ta,
                                        uint32_t *cb, uint32_t b) {
     const int L = p.L;
@@ -1121,7 +1120,12 @@ __global__ void __launch_bounds__(kC4WalkWarps * 32) k_c4_bin_walk(C4Bin p) {
 }
 
 // Counts of a far-end row of k_c4_bin_gram (a power of two from L on; L <= 8), 0
-// for more types (k_c4_bin_pairs).
+// for more types (k_c4_bin_pairs).  Counts of a power law of 100K nodes and 1M edges
+// (hub 36K) take 4.8, 4.1, 3.9 ms with 2, 3, 4 types, 3.4 to 3.8 with 5 to 8 and 9.0
+// with 9.  Rows of eight counts for 2 to 4 types, on the tensor cores, would take 3.8,
+// 3.5, 3.4 ms.  A row of 9 to 16 counts spans two matrices of eight: its products are not
+// written, and k_c4_bin_pairs is what there was (18.4 ms in all before the windows had
+// one type).
 __host__ __device__ constexpr int bin_lanes(int L) { return L <= 2 ? 2 : L <= 4 ? 4 : L <= 8 ? 8 : 0; }
 
 // Type of window w.

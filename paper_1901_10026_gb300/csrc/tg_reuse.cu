@@ -458,7 +458,7 @@ __global__ void k_tau_first(const int64_t *rowptr, const int64_t *uoff, int64_t 
 constexpr int kAggrSmall = 64;  // degree bound of the lane groups
 constexpr int kAggrChunk = 2048;
 
-// chunks of node v's typed ranges (0 for a node left to the one-thread kernel)
+// chunks of node v's typed ranges (0 for a node left to k_node_aggr_small)
 __global__ void k_aggr_chunks(const int64_t *rowptr, const int32_t *toff, int64_t n, int32_t L,
                               int dsmall, uint32_t *nch) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
