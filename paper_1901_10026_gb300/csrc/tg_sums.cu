@@ -156,8 +156,10 @@ __device__ __forceinline__ void sum_checks(const SumParams &p, int64_t block, in
 constexpr int kSumWarps = 8;
 static_assert(kSumWarps * 32 == kCheckThreads, "the checks run in the same launch");
 
+// Five CTAs per SM: with the registers that the checks would take there are four, and
+// the k = 3 count of an ER graph of 5M edges takes 1,862 and not 1,847 us.
 template <int LP>
-__global__ void __launch_bounds__(kSumWarps * 32) k_sum_edges(SumParams p) {
+__global__ void __launch_bounds__(kSumWarps * 32, LP <= 8 ? 5 : 1) k_sum_edges(SumParams p) {
     constexpr int kPairs = LP * (LP + 1) / 2, kSlots = (kPairs + 31) / 32;
     extern __shared__ __align__(16) unsigned char smem[];
     const int L = p.L, P = p.P, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
