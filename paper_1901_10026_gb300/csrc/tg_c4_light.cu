@@ -136,13 +136,20 @@ __global__ void __launch_bounds__(kCostThreads) k_c4_classify(
     }
 }
 
+// Up to so many split anchors are sorted on the host, more on the device.  1,024 take 33
+// us there and the two launches and the sort 20 here; but the 300,000 of a cycle
+// (unroll 4) took 6 ms there, while a hub's few hundred, sorted here, made counts of
+// power laws 20 us longer (4.46 ms) and seven unions of a batch 180 (12.6 ms).
+constexpr int64_t kHostSort = 1024;
+
 __global__ void k_c4_heavy_keys(const uint32_t *list, int64_t count, uint64_t *keys) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < count;
          q += (int64_t)gridDim.x * blockDim.x)
         keys[q] = list[q];
 }
 
-__global__ void k_c4_heavy_info(const uint64_t *list, int64_t count, const int64_t *rowptr,
+template <class Id>
+__global__ void k_c4_heavy_info(const Id *list, int64_t count, const int64_t *rowptr,
                                 const uint8_t *ntype, const unsigned long long *cost,
                                 C4HeavyInfo *out) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < count;
@@ -567,20 +574,26 @@ int tg_c4_classify(const tg_graph *g, const tg_tune &t, const tg_part &part, boo
 int tg_c4_heavy(const tg_graph *g, const C4Lists &cls, C4HeavyInfo *host, cudaStream_t s) {
     const int64_t count = cls.size[kC4Split];
     if (count == 0) return TG_OK;
-    // sorted here and not on the host, where the 300,000 anchors of a cycle (unroll 4)
-    // took 6 of the 51 ms of its count
+    const uint32_t *list = cls.list.p + (int64_t)kC4Split * cls.n;
+    const unsigned grid = (unsigned)std::min<int64_t>((count + 255) / 256, 4096);
     DevBuf<C4HeavyInfo> info;
     DevBuf<uint64_t> k1, k2;
-    if (!info.alloc(count, s) || !k1.alloc(count, s) || !k2.alloc(count, s)) return TG_ENOMEM;
-    const unsigned grid = (unsigned)std::min<int64_t>((count + 255) / 256, 4096);
-    k_c4_heavy_keys<<<grid, 256, 0, s>>>(cls.list.p + (int64_t)kC4Split * cls.n, count, k1.p); tg_note_launch();
-    TG_TRY_CUDA(cudaGetLastError());
-    uint64_t *sorted = nullptr;
-    TG_TRY(tg_radix_sort_u64(k1.p, k2.p, count, tg_bitlen((uint64_t)(g->n - 1)), s, &sorted));
-    k_c4_heavy_info<<<grid, 256, 0, s>>>(sorted, count, g->rowptr, g->ntype, cls.cost.p, info.p); tg_note_launch();
+    if (!info.alloc(count, s)) return TG_ENOMEM;
+    if (count <= kHostSort) {
+        k_c4_heavy_info<<<grid, 256, 0, s>>>(list, count, g->rowptr, g->ntype, cls.cost.p, info.p); tg_note_launch();
+    } else {
+        if (!k1.alloc(count, s) || !k2.alloc(count, s)) return TG_ENOMEM;
+        k_c4_heavy_keys<<<grid, 256, 0, s>>>(list, count, k1.p); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+        uint64_t *sorted = nullptr;
+        TG_TRY(tg_radix_sort_u64(k1.p, k2.p, count, tg_bitlen((uint64_t)(g->n - 1)), s, &sorted));
+        k_c4_heavy_info<<<grid, 256, 0, s>>>(sorted, count, g->rowptr, g->ntype, cls.cost.p, info.p); tg_note_launch();
+    }
     TG_TRY_CUDA(cudaGetLastError());
     TG_TRY_CUDA(cudaMemcpyAsync(host, info.p, count * sizeof(C4HeavyInfo), cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
+    if (count <= kHostSort)
+        std::sort(host, host + count, [](const C4HeavyInfo &x, const C4HeavyInfo &y) { return x.a < y.a; });
     return TG_OK;
 }
 
