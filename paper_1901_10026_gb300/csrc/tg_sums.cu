@@ -107,12 +107,11 @@ __device__ __forceinline__ void sum_checks(const SumParams &p, int64_t block, in
     const int L = p.L, L2 = L * L, P = p.P, R = kCheckThreads / L2;
     for (int x = threadIdx.x; x < P + L; x += kCheckThreads) part[x] = 0ull;
     __syncthreads();
-    const int q = threadIdx.x % L2, s = q / L, a = q % L;
-    // triangles of (s, a); D of column a; thread q < L: the other side of D's column q
-    unsigned long long tri = 0, dsum = 0, defect = 0;
-    bool bad = false;
-    const int64_t step = blocks * R;
-    if (threadIdx.x < R * L2)
+    if (threadIdx.x < R * L2) {
+        const int q = threadIdx.x % L2, s = q / L, a = q % L;
+        unsigned long long tri = 0, dsum = 0;  // triangles of (s, a), D of column a
+        bool bad = false;
+        const int64_t step = blocks * R;
         for (int64_t v0 = block * R + threadIdx.x / L2; v0 < p.n; v0 += step * kCheckBatch) {
             uint32_t t[kCheckBatch], m[kCheckBatch], x[kCheckBatch];
 #pragma unroll
@@ -122,11 +121,6 @@ __device__ __forceinline__ void sum_checks(const SumParams &p, int64_t block, in
                 t[y] = in ? __ldg(p.theta + v * L2 + q) : 0u;
                 m[y] = in ? __ldg(p.theta + v * L2 + a * L + s) : 0u;
                 x[y] = in ? __ldg(p.dlow + v * L2 + q) : 0u;
-                if (q >= L || !in) continue;
-                const int32_t *to = p.toff + v * (L + 1);
-                const uint32_t up = (uint32_t)__ldg(p.utoff + v * (L + 1) + L);
-                defect += (unsigned long long)up * (uint32_t)(__ldg(to + q + 1) - __ldg(to + q));
-                if (q == p.ntype[v]) defect -= (uint32_t)__ldg(to + L) - up;
             }
 #pragma unroll
             for (int y = 0; y < kCheckBatch; ++y) {
@@ -135,12 +129,36 @@ __device__ __forceinline__ void sum_checks(const SumParams &p, int64_t block, in
                 dsum += x[y];
             }
         }
-    if (threadIdx.x < R * L2) {
         if (s <= a) flush_nonzero(part + pair_index(L, s, a), tri);
         flush_nonzero(part + P + a, 0ull - dsum);
-        if (q < L) flush_nonzero(part + P + q, defect);
+        if (bad && p.err) atomicOr(p.err, TG_DERR_TOTALS);
     }
-    if (bad && p.err) atomicOr(p.err, TG_DERR_TOTALS);
+    // the other side of D: a thread per type of a node
+    const int R2 = kCheckThreads / L, b = threadIdx.x % L;
+    if (threadIdx.x < R2 * L) {
+        unsigned long long sum = 0;
+        const int64_t step = blocks * R2;
+        for (int64_t v0 = block * R2 + threadIdx.x / L; v0 < p.n; v0 += step * 2) {
+            uint32_t up[2], d[2], all[2];
+            int tv[2];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const int64_t v = v0 + y * step;
+                const bool in = v < p.n;
+                const int32_t *to = p.toff + v * (L + 1);
+                up[y] = in ? (uint32_t)__ldg(p.utoff + v * (L + 1) + L) : 0u;
+                d[y] = in ? (uint32_t)(__ldg(to + b + 1) - __ldg(to + b)) : 0u;
+                all[y] = in ? (uint32_t)__ldg(to + L) : 0u;
+                tv[y] = in ? (int)p.ntype[v] : -1;
+            }
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                sum += (unsigned long long)up[y] * d[y];
+                if (b == tv[y]) sum -= all[y] - up[y];
+            }
+        }
+        flush_nonzero(part + P + b, sum);
+    }
     __syncthreads();
     unsigned long long *out = p.sums + p.e2 + 2 * p.n3 + 4 * p.n4;  // [P] triangles, [P] the edges', [L]
     for (int x = threadIdx.x; x < P + L; x += kCheckThreads) flush_nonzero(out + (x < P ? x : x + P), part[x]);
