@@ -1279,13 +1279,13 @@ extern "C" int tg_count_range(const tg_graph *g, int32_t k, int64_t e0, int64_t 
     DevBuf<unsigned long long> d;
     DevBuf<unsigned> err;
     unsigned long long *dsums = reinterpret_cast<unsigned long long *>(sums);
-    const bool dev_out = tg_is_device_ptr(sums);
-    if (!err.alloc(1, s) || (!dev_out && !d.alloc(len, s))) return TG_ENOMEM;
+    const bool dev_out = tg_is_device_ptr(sums), whole = e0 == 0 && e1 == g->M;  // see sums_impl
+    if ((whole && !err.alloc(1, s)) || (!dev_out && !d.alloc(len, s))) return TG_ENOMEM;
     if (!dev_out) dsums = d.p;
-    TG_TRY_CUDA(cudaMemsetAsync(err.p, 0, 4, s));
+    if (whole) TG_TRY_CUDA(cudaMemsetAsync(err.p, 0, 4, s));
     TG_TRY(sums_impl(g, k, e0, e1, dsums, err.p, s));
     unsigned herr = 0;
-    TG_TRY_CUDA(cudaMemcpyAsync(&herr, err.p, 4, cudaMemcpyDeviceToHost, s));
+    if (whole) TG_TRY_CUDA(cudaMemcpyAsync(&herr, err.p, 4, cudaMemcpyDeviceToHost, s));
     if (!dev_out) TG_TRY_CUDA(cudaMemcpyAsync(sums, d.p, len * 8, cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));
     return herr ? TG_EINTERNAL : TG_OK;
