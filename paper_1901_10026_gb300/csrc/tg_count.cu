@@ -1344,41 +1344,39 @@ extern "C" int tg_count_shard(const tg_graph *g, int32_t k, int32_t shard, int32
         if (!d.alloc(len, s)) return TG_ENOMEM;
         dsums = d.p;
     }
-    {
-        TG_TRY_CUDA(cudaMemsetAsync(dsums, 0, len * 8, s));
-        tg_sched *sc = nullptr;
-        TG_TRY(get_sched(g, s, &sc));
-        TG_TRY(sched_sorted(g, sc, s));
-        const int64_t M = g->M;
-        int64_t q[2] = {0, 0};
-        if (M > 0) {
-            DevBuf<int64_t> cost, pre, qs;
-            if (!cost.alloc(M + 1, s) || !pre.alloc(M + 1, s) || !qs.alloc(2, s)) return TG_ENOMEM;
-            k_order_cost<<<grid_for(M + 1), 256, 0, s>>>(sc->sorted, g->edges, g->rowptr, M, cost.p); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-            TG_TRY(tg_scan_i64(cost.p, pre.p, M + 1, s));
-            k_split_points<<<1, 32, 0, s>>>(pre.p, M, shard, nshards, qs.p); tg_note_launch();
-            TG_TRY_CUDA(cudaGetLastError());
-            TG_TRY_CUDA(cudaMemcpyAsync(q, qs.p, 16, cudaMemcpyDeviceToHost, s));
-            TG_TRY_CUDA(cudaStreamSynchronize(s));
-        }
-        const tg_tune t = tune_now();
-        if (t.kernel == TG_KERNEL_AUTO || t.kernel == TG_KERNEL_CYCLES) {
-            // a slice of the edges, and a share of the whole-graph enumerations
-            tg_part part;
-            part.index = shard;
-            part.count = nshards;
-            if (k == 4)
-                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], q[1] - q[0],
-                                      nullptr, 0, dsums, t, s, part));
-            else if (q[1] > q[0])
-                TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], q[1] - q[0],
-                                      nullptr, 0, dsums, t, s));
-        } else if (q[1] > q[0]) {
-            // the per-edge kernels need nothing beyond the slice's edges
-            TG_TRY(launch_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], 0, q[1] - q[0],
-                                nullptr, 0, dsums, s));
-        }
+    TG_TRY_CUDA(cudaMemsetAsync(dsums, 0, len * 8, s));
+    tg_sched *sc = nullptr;
+    TG_TRY(get_sched(g, s, &sc));
+    TG_TRY(sched_sorted(g, sc, s));
+    const int64_t M = g->M;
+    int64_t q[2] = {0, 0};
+    if (M > 0) {
+        DevBuf<int64_t> cost, pre, qs;
+        if (!cost.alloc(M + 1, s) || !pre.alloc(M + 1, s) || !qs.alloc(2, s)) return TG_ENOMEM;
+        k_order_cost<<<grid_for(M + 1), 256, 0, s>>>(sc->sorted, g->edges, g->rowptr, M, cost.p); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+        TG_TRY(tg_scan_i64(cost.p, pre.p, M + 1, s));
+        k_split_points<<<1, 32, 0, s>>>(pre.p, M, shard, nshards, qs.p); tg_note_launch();
+        TG_TRY_CUDA(cudaGetLastError());
+        TG_TRY_CUDA(cudaMemcpyAsync(q, qs.p, 16, cudaMemcpyDeviceToHost, s));
+        TG_TRY_CUDA(cudaStreamSynchronize(s));
+    }
+    const tg_tune t = tune_now();
+    if (t.kernel == TG_KERNEL_AUTO || t.kernel == TG_KERNEL_CYCLES) {
+        // a slice of the edges, and a share of the whole-graph enumerations
+        tg_part part;
+        part.index = shard;
+        part.count = nshards;
+        if (k == 4)
+            TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], q[1] - q[0],
+                                  nullptr, 0, dsums, t, s, part));
+        else if (q[1] > q[0])
+            TG_TRY(tg_reuse_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], q[1] - q[0],
+                                  nullptr, 0, dsums, t, s));
+    } else if (q[1] > q[0]) {
+        // the per-edge kernels need nothing beyond the slice's edges
+        TG_TRY(launch_count(g, k, TG_GRAPHLET, sc->lists, sc->sorted + q[0], 0, q[1] - q[0],
+                            nullptr, 0, dsums, s));
     }
     if (!dev_out) TG_TRY_CUDA(cudaMemcpyAsync(sums, dsums, len * 8, cudaMemcpyDeviceToHost, s));
     TG_TRY_CUDA(cudaStreamSynchronize(s));

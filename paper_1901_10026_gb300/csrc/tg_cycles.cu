@@ -186,7 +186,11 @@ __device__ void c4_tile(const C4Params &p, const C4Smem &sm, uint32_t a, int ta,
     if (phase == 1)
         for (int q = tid; q < nmem * L2; q += blockDim.x) sm.acc[q] = 0ull;
     __syncthreads();
-    for (int64_t pos = tid; pos < total; pos += blockDim.x) {
+    // the CTA's threads make the same number of steps: a loop over each thread's own
+    // positions took 3.01 and not 2.78 ms for K_{64,20000}
+    for (int64_t base = 0; base < total; base += blockDim.x) {
+        const int64_t pos = base + tid;
+        if (pos >= total) continue;
         int lo = 0, hi = nmem - 1;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
